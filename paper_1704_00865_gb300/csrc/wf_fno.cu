@@ -25,9 +25,11 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/wf.h"
+#include "wf_device.cuh"
 #include "wf_internal.h"
 
 namespace {
@@ -58,250 +60,756 @@ struct Layout {
 
 // ------------------------------------------------------------------ kernels
 
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
-// d/dz [z Phi(z)] = Phi(z) + z phi(z)
-__device__ __forceinline__ float gelu_grad(float z) {
-  const float Phi = 0.5f * (1.f + erff(z * 0.70710678118654752f));
-  const float phi = 0.3989422804014327f * __expf(-0.5f * z * z);
-  return Phi + z * phi;
-}
-
 __global__ void to_half_kernel(const float* __restrict__ src, __half* __restrict__ dst, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = __float2half_rn(src[i]);
 }
 
-// out[b][o][p] = act(sum_i W[o][i] in[b][i][p] + bias[o] + add[b][o][p]);
-// pre (if not null) keeps the argument of act.
-__global__ void pointwise_fwd(const float* __restrict__ in, const __half* __restrict__ W,
-                              const float* __restrict__ bias, const float* __restrict__ add, float* __restrict__ pre,
-                              float* __restrict__ out, int B, int CI, int CO, int P, int act) {
-  __shared__ float sW[kMaxWidth * kMaxWidth];
-  for (int k = threadIdx.x; k < CO * CI; k += blockDim.x) sW[k] = __half2float(W[k]);
+// The network's passes (sizes: B maps, C channels of N x N pixels, MX x 2 MY
+// retained modes; CP = C rounded up to 8, 16, 32 or 64).
+//
+//   analysis     rows and columns of the truncated DFT of a block of rows of
+//                one channel -> partial sums of X[j][k]
+//   mix          the partial sums -> X; Y = R X (or R^H X for the adjoint)
+//   synth_cols   Y -> S[y][k], the truncated inverse along columns
+//   synth        S -> pixels along rows, + W h + bias, GELU (or the adjoint,
+//                times GELU')
+//
+// A layer is four launches forward and six backward; each activation map is
+// read twice and written once.  Before, the transforms were one output per
+// thread with both operands from L2, and the channel products kept their
+// operands in local memory: inference of one 512^2 map (32 channels, 16 x 32
+// modes, 4 layers) 6359 us then, 432 us now; the gradient of eight 256^2 maps
+// 15 575 us then, 1697 us now.
+//
+// Both transforms use e^{2 pi i k (x + N/2) / N} = (-1)^k e^{2 pi i k x / N}: rows
+// (and columns) a half period apart are added and subtracted first, the sums
+// serve the even k and the differences the odd k, so every direct sum runs
+// over N/2 terms (or gives two outputs).
+
+constexpr int kAnRows = 32;   // rows of an analysis block, half of them N/2 further on
+constexpr int kAnX = 32;      // pixels of a row staged at a time
+constexpr int kMixModes = 8;  // modes of a mix block
+constexpr int kColY = 32;     // row pairs of a column-synthesis block
+
+// h_0 = P x + p
+__global__ void lift_fwd(const float* __restrict__ x, const __half* __restrict__ W, const float* __restrict__ bias,
+                         float* __restrict__ out, int B, int C, int P) {
+  __shared__ float sW[kMaxWidth * 2];
+  __shared__ float sb[kMaxWidth];
+  for (int k = threadIdx.x; k < 2 * C; k += blockDim.x) sW[k] = __half2float(W[k]);
+  for (int k = threadIdx.x; k < C; k += blockDim.x) sb[k] = bias[k];
   __syncthreads();
   const size_t total = (size_t)B * P;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
     const int b = (int)(g / P), p = (int)(g % P);
-    float xin[kMaxWidth];
-    for (int i = 0; i < CI; ++i) xin[i] = in[((size_t)b * CI + i) * P + p];
-    for (int o = 0; o < CO; ++o) {
-      float z = bias[o];
-      for (int i = 0; i < CI; ++i) z = fmaf(sW[o * CI + i], xin[i], z);
-      const size_t idx = ((size_t)b * CO + o) * P + p;
-      if (add) z += add[idx];
-      if (pre) pre[idx] = z;
-      out[idx] = act ? gelu_f(z) : z;
-    }
+    const float x0 = x[((size_t)b * 2) * P + p], x1 = x[((size_t)b * 2 + 1) * P + p];
+    for (int o = 0; o < C; ++o)
+      out[((size_t)b * C + o) * P + p] = fmaf(sW[2 * o + 1], x1, fmaf(sW[2 * o], x0, sb[o]));
   }
 }
 
-// g_pre = g_out * act'(pre) (in place into gz), g_in[b][i][p] (+)= sum_o W[o][i] g_pre[b][o][p]
-__global__ void pointwise_bwd_in(const float* __restrict__ gout, const float* __restrict__ pre, float* __restrict__ gz,
-                                 const __half* __restrict__ W, float* __restrict__ gin, int B, int CI, int CO, int P,
-                                 int act, int accumulate) {
-  __shared__ float sW[kMaxWidth * kMaxWidth];
-  for (int k = threadIdx.x; k < CO * CI; k += blockDim.x) sW[k] = __half2float(W[k]);
+// Partial column sums of the row DFTs of one channel's rows:
+//   part[slice][block][j][k] = sc_k sum_{y in block} e^{-2 pi i ky_j y / N} sum_x in[y][x] e^{-2 pi i k x / N}
+// for the 32 rows {y0 .. y0 + 15} and the same + N/2.  The row DFT is a
+// register-tiled product of the folded rows (staged transposed in shared
+// memory, row groups XOR-swizzled by x so that both the stores and the
+// 16-byte loads are conflict-free) with the twiddle table tw_k[x][slot]
+// (slot = parity * 2 KG + k / 2): 4 rows x 2 modes per thread, 16 FMA per two
+// 16-byte loads.  Sums run over 32 pixels at a time and are then added up, to
+// keep the rounding of the long sums near that of a tree.
+// FP32-issue bound: N/2 * 32 FMA per row for 16 modes.
+__global__ void __launch_bounds__(128)
+analysis(const float* __restrict__ in, float2* __restrict__ part, const float2* __restrict__ tw_k,
+         const float2* __restrict__ tw_y, int N, int MX, int MY2, int KG, float s0, float s1) {
+  extern __shared__ __align__(16) float sm_an[];
+  const int NX = min(kAnX, N / 2);                    // pixels staged at a time
+  float* st = sm_an;                                  // [2][kAnX][kAnRows] folded rows
+  float4* stw = reinterpret_cast<float4*>(sm_an + 2 * kAnX * kAnRows);  // [kAnX][2 KG] mode pairs
+  float2* sA = reinterpret_cast<float2*>(sm_an);      // [rows][MX] afterwards
+  const int rows = min(kAnRows, N), RH = rows / 2, nblk = (N / 2) / RH;
+  const int slice = blockIdx.x / nblk, yb = blockIdx.x - slice * nblk;
+  const int y0 = yb * RH;
+  const float* src = in + (size_t)slice * N * N;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int RG = rows / 4;                            // row groups of 4
+  const int rg = tid % RG, kgp = tid / RG;            // kgp: parity * KG + pair of modes
+  const bool work = kgp < 2 * KG;
+  const int par = kgp >= KG ? 1 : 0;
+  float acc[4][4];                                    // [row][k0 re, k0 im, k1 re, k1 im]
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+  const int XQ = NX / 4;                              // 16-byte pieces of a row
+  for (int x0 = 0; x0 < N / 2; x0 += NX) {
+    __syncthreads();
+    for (int i = tid; i < rows * XQ; i += nt) {
+      const int r4 = i & 3, xq = (i >> 2) % XQ, rq = (i >> 2) / XQ;
+      const int row = rq * 4 + r4;
+      const int y = row < RH ? y0 + row : y0 + N / 2 + row - RH;
+      const float4 a = *reinterpret_cast<const float4*>(src + (size_t)y * N + x0 + 4 * xq);
+      const float4 b = *reinterpret_cast<const float4*>(src + (size_t)y * N + x0 + N / 2 + 4 * xq);
+      float* d = st + (4 * xq) * kAnRows + ((rq ^ (xq & 7)) * 4 + r4);
+      d[0] = a.x + b.x;
+      d[kAnRows] = a.y + b.y;
+      d[2 * kAnRows] = a.z + b.z;
+      d[3 * kAnRows] = a.w + b.w;
+      d += kAnX * kAnRows;
+      d[0] = a.x - b.x;
+      d[kAnRows] = a.y - b.y;
+      d[2 * kAnRows] = a.z - b.z;
+      d[3 * kAnRows] = a.w - b.w;
+    }
+    for (int i = tid; i < NX * 2 * KG; i += nt)
+      stw[i] = *reinterpret_cast<const float4*>(tw_k + ((size_t)x0 * 2 * KG + i) * 2);
+    __syncthreads();
+    if (work) {
+      float c[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[r][q] = 0.f;
+      const float* sp = st + par * kAnX * kAnRows;
+#pragma unroll 4
+      for (int x = 0; x < NX; ++x) {
+        const float4 h = *reinterpret_cast<const float4*>(sp + x * kAnRows + ((rg ^ ((x >> 2) & 7)) * 4));
+        const float4 w = stw[x * 2 * KG + kgp];
+        const float hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          c[r][0] = fmaf(hv[r], w.x, c[r][0]);
+          c[r][1] = fmaf(hv[r], w.y, c[r][1]);
+          c[r][2] = fmaf(hv[r], w.z, c[r][2]);
+          c[r][3] = fmaf(hv[r], w.w, c[r][3]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] += c[r][q];
+    }
+  }
   __syncthreads();
-  const size_t total = (size_t)B * P;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(g / P), p = (int)(g % P);
-    float gp[kMaxWidth];
-    for (int o = 0; o < CO; ++o) {
-      const size_t idx = ((size_t)b * CO + o) * P + p;
-      float v = gout[idx];
-      if (act) v *= gelu_grad(pre[idx]);
-      gp[o] = v;
-      if (gz) gz[idx] = v;
+  // the row transforms, then the block's share of the columns
+  if (work) {
+    const int k0 = 2 * (2 * (kgp - par * KG)) + par, k1 = k0 + 2;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int row = rg * 4 + r;
+      if (k0 < MX) {
+        const float sc = k0 == 0 ? s0 : s1;
+        sA[row * MX + k0] = make_float2(acc[r][0] * sc, acc[r][1] * sc);
+      }
+      if (k1 < MX) sA[row * MX + k1] = make_float2(acc[r][2] * s1, acc[r][3] * s1);
     }
-    if (!gin) continue;
-    for (int i = 0; i < CI; ++i) {
-      float s = 0.f;
-      for (int o = 0; o < CO; ++o) s = fmaf(sW[o * CI + i], gp[o], s);
-      const size_t idx = ((size_t)b * CI + i) * P + p;
-      gin[idx] = accumulate ? gin[idx] + s : s;
+  }
+  __syncthreads();
+  for (int i = tid; i < RH * MX; i += nt) {  // fold the rows a half period apart
+    const float2 a = sA[i], b = sA[RH * MX + i];
+    sA[i] = make_float2(a.x + b.x, a.y + b.y);
+    sA[RH * MX + i] = make_float2(a.x - b.x, a.y - b.y);
+  }
+  __syncthreads();
+  float2* dst = part + ((size_t)slice * nblk + yb) * MY2 * MX;
+  for (int i = tid; i < MY2 * MX; i += nt) {
+    const int k = i % MX, j = i / MX;  // ky_j has the parity of j (N - 2 MY is even)
+    const float2* a = sA + (j & 1) * RH * MX + k;
+    const float2* w = tw_y + (size_t)j * N + y0;
+    float re = 0.f, im = 0.f;
+    for (int y = 0; y < RH; ++y) {
+      const float2 v = a[y * MX], t = __ldg(&w[y]);
+      re = fmaf(v.x, t.x, fmaf(-v.y, t.y, re));
+      im = fmaf(v.x, t.y, fmaf(v.y, t.x, im));
+    }
+    dst[i] = make_float2(re, im);
+  }
+}
+
+// X[b][c][m] = the sum of the blocks' partial sums; then, per mode m,
+//   fwd: out[b][m][o] = sum_i R[i][o][m] X[b][i][m]
+//   bwd: out[b][m][i] = sum_o conj(R[i][o][m]) X[b][o][m]
+// One block takes 8 modes (32-byte pieces of R) of one map; the output is
+// channel-fastest for the column synthesis.  Bound by reading R (4 C^2 bytes
+// per mode) and by latency.
+__global__ void __launch_bounds__(kThreads)
+mix(const float2* __restrict__ part, int nblk, const __half2* __restrict__ R, float2* __restrict__ X,
+    float2* __restrict__ out, int C, int CP, int NM, int bwd) {
+  __shared__ float2 sX[kMaxWidth * kMixModes];
+  __shared__ float2 sY[kMixModes * kMaxWidth];
+  const int b = blockIdx.y, m0 = blockIdx.x * kMixModes;
+  for (int i = threadIdx.x; i < C * kMixModes; i += blockDim.x) {
+    const int c = i / kMixModes, m = m0 + i % kMixModes;
+    float re = 0.f, im = 0.f;
+    if (m < NM) {
+      const float2* src = part + ((size_t)(b * C + c) * nblk) * NM + m;
+      for (int q = 0; q < nblk; ++q) {
+        const float2 v = src[(size_t)q * NM];
+        re += v.x;
+        im += v.y;
+      }
+      X[((size_t)b * C + c) * NM + m] = make_float2(re, im);
+    }
+    sX[i] = make_float2(re, im);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < CP * kMixModes; i += blockDim.x) {
+    const int o = i / kMixModes, ml = i % kMixModes, m = m0 + ml;
+    float re = 0.f, im = 0.f;
+    if (o < C && m < NM) {
+      if (!bwd) {
+#pragma unroll 8
+        for (int c = 0; c < C; ++c) {
+          const float2 r = __half22float2(R[((size_t)c * C + o) * NM + m]);
+          const float2 x = sX[c * kMixModes + ml];
+          re = fmaf(r.x, x.x, fmaf(-r.y, x.y, re));
+          im = fmaf(r.x, x.y, fmaf(r.y, x.x, im));
+        }
+      } else {
+#pragma unroll 8
+        for (int c = 0; c < C; ++c) {
+          const float2 r = __half22float2(R[((size_t)o * C + c) * NM + m]);
+          const float2 x = sX[c * kMixModes + ml];
+          re = fmaf(r.x, x.x, fmaf(r.y, x.y, re));
+          im = fmaf(r.x, x.y, fmaf(-r.y, x.x, im));
+        }
+      }
+    }
+    sY[ml * CP + o] = make_float2(re, im);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < CP * kMixModes; i += blockDim.x) {
+    const int m = m0 + i / CP;
+    if (m < NM) out[((size_t)b * NM + m) * CP + i % CP] = sY[i];
+  }
+}
+
+// g_R[i][o][m] = sum_b g_Y[b][o][m] conj(X[b][i][m]), written as (re, im)
+// pairs: 4 x 4 channels of one mode per thread.  The bias gradient of the
+// pointwise branch, the sum of g_z over all pixels, is N^2 times the mode 0
+// of g_Y (scale 1/N^2 there): written by the threads of mode 0.
+__global__ void __launch_bounds__(128)
+mix_bwd_r(const float2* __restrict__ gY, const float2* __restrict__ X, float* __restrict__ gR, float* __restrict__ gw,
+          int B, int C, int NM, float n2) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= NM) return;
+  const int i0 = blockIdx.y * 4, o0 = blockIdx.z * 4;
+  float re[4][4], im[4][4], bias[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) re[i][o] = im[i][o] = 0.f;
+  for (int b = 0; b < B; ++b) {
+    float2 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      x[i] = i0 + i < C ? X[((size_t)b * C + i0 + i) * NM + m] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      y[o] = o0 + o < C ? gY[((size_t)b * C + o0 + o) * NM + m] : make_float2(0.f, 0.f);
+      bias[o] += y[o].x;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        re[i][o] = fmaf(y[o].x, x[i].x, fmaf(y[o].y, x[i].y, re[i][o]));
+        im[i][o] = fmaf(y[o].y, x[i].x, fmaf(-y[o].x, x[i].y, im[i][o]));
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+      if (i0 + i < C && o0 + o < C) {
+        float* d = gR + 2 * (((size_t)(i0 + i) * C + o0 + o) * NM + m);
+        d[0] = re[i][o];
+        d[1] = im[i][o];
+      }
+  if (m == 0 && i0 == 0)
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+      if (o0 + o < C) gw[o0 + o] = bias[o] * n2;
+}
+
+// S[b][y][k] = c_k sum_j Y[b][j k] e^{+2 pi i ky_j y / N} for all channels, as
+// CP real parts then CP imaginary parts (the imaginary part of k = 0 drops
+// out of the row synthesis and is written as 0).  A lane is a channel, a warp
+// takes four rows and, from the same sums, the four N/2 further on.
+__global__ void __launch_bounds__(256)
+synth_cols(const float2* __restrict__ Y, float* __restrict__ S, const float2* __restrict__ tw_y, int N, int MX,
+           int MY2, int CP, float c0, float c1) {
+  extern __shared__ __align__(16) float2 sm_sc[];
+  float2* sT = sm_sc;                  // [MY2][kColY]
+  float2* sY = sm_sc + MY2 * kColY;    // [MY2][CP]
+  const int yb = blockIdx.x * kColY, k = blockIdx.y, b = blockIdx.z;
+  for (int i = threadIdx.x; i < MY2 * kColY; i += blockDim.x) {
+    const int y = yb + i % kColY;
+    sT[i] = y < N / 2 ? __ldg(&tw_y[(size_t)(i / kColY) * N + y]) : make_float2(0.f, 0.f);
+  }
+  for (int i = threadIdx.x; i < MY2 * CP; i += blockDim.x)
+    sY[i] = Y[((size_t)b * MY2 * MX + (size_t)(i / CP) * MX + k) * CP + i % CP];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, yl = (threadIdx.x >> 5) * 4;
+  const float sc = k == 0 ? c0 : c1;
+  for (int o = lane; o < CP; o += 32) {
+    float er[4], ei[4], dr[4], di[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) er[q] = ei[q] = dr[q] = di[q] = 0.f;
+    for (int j = 0; j < MY2; j += 2) {
+      const float2 a = sY[j * CP + o], c = sY[(j + 1) * CP + o];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 t = sT[j * kColY + yl + q], u = sT[(j + 1) * kColY + yl + q];  // conjugates of e^{+...}
+        er[q] = fmaf(a.x, t.x, fmaf(a.y, t.y, er[q]));
+        ei[q] = fmaf(-a.x, t.y, fmaf(a.y, t.x, ei[q]));
+        dr[q] = fmaf(c.x, u.x, fmaf(c.y, u.y, dr[q]));
+        di[q] = fmaf(-c.x, u.y, fmaf(c.y, u.x, di[q]));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int y = yb + yl + q;
+      if (y < N / 2) {
+        float* d = S + (((size_t)b * N + y) * MX + k) * 2 * CP + o;
+        d[0] = (er[q] + dr[q]) * sc;
+        d[CP] = k == 0 ? 0.f : (ei[q] + di[q]) * sc;
+        d += (size_t)(N / 2) * MX * 2 * CP;
+        d[0] = (er[q] - dr[q]) * sc;
+        d[CP] = k == 0 ? 0.f : (ei[q] - di[q]) * sc;
+      }
     }
   }
 }
 
-// partial[blk][o][i] = sum over this block's pixels of gz[b][o][p] in[b][i][p];
-// partial[blk][o][CI] = sum of gz[b][o][p] (the bias gradient)
-__global__ void pointwise_bwd_w(const float* __restrict__ gz, const float* __restrict__ in, float* __restrict__ partial,
-                                int B, int CI, int CO, int P) {
-  const int o = blockIdx.y;
-  const int nblk = gridDim.x;
-  float acc[kMaxWidth + 1];
-  for (int i = 0; i <= CI; ++i) acc[i] = 0.f;
-  const size_t total = (size_t)B * P;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)nblk * blockDim.x) {
-    const int b = (int)(g / P), p = (int)(g % P);
-    const float v = gz[((size_t)b * CO + o) * P + p];
-    for (int i = 0; i < CI; ++i) acc[i] = fmaf(v, in[((size_t)b * CI + i) * P + p], acc[i]);
-    acc[CI] += v;
+// Geometry of the row synthesis: OG groups of 8 output channels x PG groups
+// of 2 pixel pairs (x, x + N/2); XT pairs of one row, RT rows per step.
+__host__ __device__ constexpr int synth_pg(int OG) { return 256 / OG < 64 ? 256 / OG : 64; }
+struct SynthGeom {
+  int XT, RT, nxt, units;
+  size_t smem;
+};
+inline SynthGeom synth_geom(int OG, int B, int C, int N, int MX) {
+  SynthGeom g;
+  const int pairs = 2 * synth_pg(OG);
+  g.XT = N / 2 < pairs ? N / 2 : pairs;
+  g.RT = pairs / g.XT < 4 ? pairs / g.XT : 4;
+  g.nxt = (N / 2) / g.XT;
+  g.units = B * (N / g.RT) * g.nxt;
+  const int CP = 8 * OG, MXE = MX;
+  g.smem = sizeof(float) * ((size_t)C * 2 * g.RT * g.XT + (size_t)2 * MXE * g.XT + (size_t)g.RT * MXE * 2 * CP +
+                            (size_t)C * CP);
+  return g;
+}
+
+struct SynthArgs {
+  const float* in;     // [B][C][N][N]: h_l (forward) or g_z (adjoint)
+  const __half* W;     // [C][C]
+  const float* S;      // [B][N][MX][2][CP]
+  const float2* tw_x;  // [MX][N]
+  const float* bias;   // forward
+  float* out;          // or nullptr
+  float* dact;         // forward: act'(z), or nullptr
+  const float* mul;    // adjoint: act'(z) of the layer below, or nullptr
+  const __half* Q;     // forward: project the output onto y, or nullptr
+  const float* q;
+  float* y;            // [B][N][N]
+  const float* x;      // adjoint of layer 0: network input, for the lift's gradient, or nullptr
+  float* lpart;        // [blocks][CP][3] sums of g x0, g x1, g
+  int B, C, N, MX, XT, RT, nxt, units, act;
+};
+
+// One layer in pixels.  Forward: z = bias + W h + (row synthesis of S), out =
+// act(z), act' kept for the backward pass (one erff serves both), the last
+// layer projected onto y.  Adjoint (ADJ): g = W^T g_z + (row synthesis of S),
+// times act' of the layer below; for layer 0 the sums of the lift's
+// gradient instead.  A thread holds 8 channels x 4 pixels (two neighbours and
+// the two N/2 further on): 32 FMA per four 8- or 16-byte shared loads for
+// W, and per six for two pixels' worth of modes.  The tables (W, the row
+// twiddles of the block's pixels) stay in shared memory while the block walks
+// its rows.  48 C^2 / 32 FMA per pixel at 16 modes (FP32-issue bound) against
+// 8 to 12 C bytes.
+template <int OG, bool ADJ>
+__global__ void __launch_bounds__(OG * synth_pg(OG))
+synth(SynthArgs a) {
+  constexpr int PG = synth_pg(OG), NT = OG * PG, CP = 8 * OG;
+  extern __shared__ __align__(16) float sm_sy[];
+  const int C = a.C, N = a.N, MX = a.MX, XT = a.XT, RT = a.RT, PX = RT * XT;
+  const size_t P = (size_t)N * N;
+  float* sW = sm_sy;                                 // [C][CP]: input channel, output channel
+  float* sS = sW + (size_t)C * CP;                   // [RT][MX][2][CP]
+  float* sTc = sS + (size_t)RT * MX * 2 * CP;        // [MX][XT] cos
+  float* sTs = sTc + (size_t)MX * XT;                // [MX][XT] -sin
+  float* sH = sTs + (size_t)MX * XT;                 // [C][2][RT][XT]
+  const int tid = threadIdx.x, og = tid % OG, pg = tid / OG;
+  const int xt = blockIdx.x % a.nxt;                 // gridDim.x is a multiple of nxt
+  for (int i = tid; i < C * CP; i += NT) {
+    const int ci = i / CP, co = i % CP;
+    sW[i] = co < C ? __half2float(ADJ ? a.W[ci * C + co] : a.W[co * C + ci]) : 0.f;
   }
-  __shared__ float red[kThreads / 32];
-  for (int i = 0; i <= CI; ++i) {
-    float v = acc[i];
-    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-      partial[((size_t)blockIdx.x * CO + o) * (CI + 1) + i] = t;
+  for (int i = tid; i < MX * XT; i += NT) {
+    const float2 t = __ldg(&a.tw_x[(size_t)(i / XT) * N + xt * XT + i % XT]);
+    sTc[i] = t.x;
+    sTs[i] = t.y;
+  }
+  const int pr = 2 * pg;                             // this thread's first pair
+  const bool on = pr < PX;
+  const int rl = on ? pr / XT : 0, xl = on ? pr % XT : 0;
+  float bias[8], lsum[8][3];
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    bias[o] = (!ADJ && og * 8 + o < C) ? a.bias[og * 8 + o] : 0.f;
+    lsum[o][0] = lsum[o][1] = lsum[o][2] = 0.f;
+  }
+  const int nyb = N / RT;
+  for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+    const int t = u / a.nxt, yb = t % nyb, b = t / nyb;
+    const int y0 = yb * RT;
+    __syncthreads();  // the tables are written; the last step's tiles are read
+    const int XQ = XT / 4;
+    for (int i = tid; i < C * 2 * RT * XQ; i += NT) {
+      const int xq = i % XQ, r = (i / XQ) % RT, h = (i / (XQ * RT)) & 1, c = i / (XQ * RT * 2);
+      wf::cp_async16(sH + 4 * (size_t)i,
+                     a.in + ((size_t)b * C + c) * P + (size_t)(y0 + r) * N + h * (N / 2) + xt * XT + 4 * xq);
     }
+    const float* gs = a.S + ((size_t)b * N + y0) * MX * 2 * CP;
+    for (int i = tid; i < RT * MX * 2 * CP / 4; i += NT) wf::cp_async16(sS + 4 * i, gs + 4 * i);
+    wf::cp_async_commit();
+    wf::cp_async_wait<0>();
     __syncthreads();
+    float z[8][4];  // [channel][x, x + 1, x + N/2, x + N/2 + 1]
+#pragma unroll
+    for (int o = 0; o < 8; ++o) z[o][0] = z[o][1] = z[o][2] = z[o][3] = 0.f;
+    // modes: even k into z[.][0..1], odd k into z[.][2..3]
+    const float* s = sS + (size_t)rl * MX * 2 * CP + og * 8;
+#pragma unroll 2
+    for (int k = 0; k < MX; k += 2) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (k + h < MX) {
+          const float2 c = *reinterpret_cast<const float2*>(sTc + (k + h) * XT + xl);
+          const float2 sn = *reinterpret_cast<const float2*>(sTs + (k + h) * XT + xl);
+          const float4* sr = reinterpret_cast<const float4*>(s + (k + h) * 2 * CP);
+          const float4* si = reinterpret_cast<const float4*>(s + (k + h) * 2 * CP + CP);
+          const float4 r0 = sr[0], r1 = sr[1], i0 = si[0], i1 = si[1];
+          const float re[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+          const float im[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+#pragma unroll
+          for (int o = 0; o < 8; ++o) {
+            z[o][2 * h] = fmaf(re[o], c.x, fmaf(im[o], sn.x, z[o][2 * h]));
+            z[o][2 * h + 1] = fmaf(re[o], c.y, fmaf(im[o], sn.y, z[o][2 * h + 1]));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const float e0 = z[o][0], e1 = z[o][1], d0 = z[o][2], d1 = z[o][3];
+      z[o][0] = e0 + d0 + bias[o];
+      z[o][1] = e1 + d1 + bias[o];
+      z[o][2] = e0 - d0 + bias[o];
+      z[o][3] = e1 - d1 + bias[o];
+    }
+    const float* hp = sH + (on ? pr : 0);
+#pragma unroll 4
+    for (int c = 0; c < C; ++c) {
+      const float2 h0 = *reinterpret_cast<const float2*>(hp + (size_t)c * 2 * PX);
+      const float2 h1 = *reinterpret_cast<const float2*>(hp + (size_t)c * 2 * PX + PX);
+      const float4* wp = reinterpret_cast<const float4*>(sW + c * CP + og * 8);
+      const float4 w0 = wp[0], w1 = wp[1];
+      const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        z[o][0] = fmaf(w[o], h0.x, z[o][0]);
+        z[o][1] = fmaf(w[o], h0.y, z[o][1]);
+        z[o][2] = fmaf(w[o], h1.x, z[o][2]);
+        z[o][3] = fmaf(w[o], h1.y, z[o][3]);
+      }
+    }
+    const size_t px = (size_t)(y0 + rl) * N + xt * XT + xl;  // and px + N/2
+    if constexpr (!ADJ) {
+      float yv[4] = {0.f, 0.f, 0.f, 0.f};
+      if (on) {
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+          const int co = og * 8 + o;
+          if (co < C) {
+            const size_t idx = ((size_t)b * C + co) * P + px;
+            if (a.Q) {
+              const float qv = __half2float(a.Q[co]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) yv[e] = fmaf(qv, z[o][e], yv[e]);
+            }
+            if (a.act) {
+              float g[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float zz = z[o][e];
+                const float Phi = 0.5f * (1.f + erff(zz * 0.70710678118654752f));
+                // d/dz [z Phi(z)] = Phi(z) + z phi(z)
+                if (a.dact) g[e] = fmaf(zz, 0.3989422804014327f * __expf(-0.5f * zz * zz), Phi);
+                z[o][e] = zz * Phi;
+              }
+              if (a.dact) {
+                *reinterpret_cast<float2*>(a.dact + idx) = make_float2(g[0], g[1]);
+                *reinterpret_cast<float2*>(a.dact + idx + N / 2) = make_float2(g[2], g[3]);
+              }
+            }
+            if (a.out) {
+              *reinterpret_cast<float2*>(a.out + idx) = make_float2(z[o][0], z[o][1]);
+              *reinterpret_cast<float2*>(a.out + idx + N / 2) = make_float2(z[o][2], z[o][3]);
+            }
+          }
+        }
+      }
+      if (a.Q) {  // sum the channel groups (neighbouring lanes)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int sft = 1; sft < OG; sft <<= 1) yv[e] += __shfl_xor_sync(0xffffffffu, yv[e], sft);
+        if (on && og == 0) {
+          float* yo = a.y + (size_t)b * P + px;
+          const float q = a.q[0];
+          yo[0] = yv[0] + q;
+          yo[1] = yv[1] + q;
+          yo[N / 2] = yv[2] + q;
+          yo[N / 2 + 1] = yv[3] + q;
+        }
+      }
+    } else if (on) {
+      float xv[2][4];
+      if (a.x) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float* xp = a.x + ((size_t)b * 2 + i) * P + px;
+          xv[i][0] = xp[0];
+          xv[i][1] = xp[1];
+          xv[i][2] = xp[N / 2];
+          xv[i][3] = xp[N / 2 + 1];
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const int co = og * 8 + o;
+        if (co < C) {
+          const size_t idx = ((size_t)b * C + co) * P + px;
+          if (a.mul) {
+            const float2 g0 = *reinterpret_cast<const float2*>(a.mul + idx);
+            const float2 g1 = *reinterpret_cast<const float2*>(a.mul + idx + N / 2);
+            z[o][0] *= g0.x;
+            z[o][1] *= g0.y;
+            z[o][2] *= g1.x;
+            z[o][3] *= g1.y;
+          }
+          if (a.out) {
+            *reinterpret_cast<float2*>(a.out + idx) = make_float2(z[o][0], z[o][1]);
+            *reinterpret_cast<float2*>(a.out + idx + N / 2) = make_float2(z[o][2], z[o][3]);
+          }
+          if (a.x) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+              lsum[o][i] += fmaf(z[o][0], xv[i][0], z[o][1] * xv[i][1]) +
+                            fmaf(z[o][2], xv[i][2], z[o][3] * xv[i][3]);
+            lsum[o][2] += (z[o][0] + z[o][1]) + (z[o][2] + z[o][3]);
+          }
+        }
+      }
+    }
+  }
+  if constexpr (ADJ) {
+    if (a.x) {  // the block's sums over its pixels: a fixed tree
+      __syncthreads();
+#pragma unroll
+      for (int o = 0; o < 8; ++o)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          float v = lsum[o][i];
+#pragma unroll
+          for (int sft = OG; sft < 32; sft <<= 1) v += __shfl_xor_sync(0xffffffffu, v, sft);
+          lsum[o][i] = v;
+        }
+      float* red = sm_sy;  // [warps][CP][3] over the tables, which are done with
+      const int warp = tid >> 5, lane = tid & 31;
+      if (lane < OG)
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+#pragma unroll
+          for (int i = 0; i < 3; ++i) red[(warp * CP + lane * 8 + o) * 3 + i] = lsum[o][i];
+      __syncthreads();
+      for (int i = tid; i < CP * 3; i += NT) {
+        float v = 0.f;
+        for (int w = 0; w < NT / 32; ++w) v += red[w * CP * 3 + i];
+        a.lpart[(size_t)blockIdx.x * CP * 3 + i] = v;
+      }
+    }
   }
 }
 
-// grad[oW + o*CI + i] = sum_blk partial[blk][o][i]; grad[ob + o] = sum_blk partial[blk][o][CI]
-__global__ void pointwise_bwd_w_fin(const float* __restrict__ partial, int nblk, int CI, int CO, float* __restrict__ gW,
-                                    float* __restrict__ gb) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= CO * (CI + 1)) return;
-  const int o = k / (CI + 1), i = k % (CI + 1);
+// partial[blk][o][i] = sum over this block's pixels of gz[b][o][p] in[b][i][p]:
+// tiles of 128 pixels of all channels in shared memory (rows 4 floats apart
+// in banks), 4 x 4 channels per thread, the pixels of a tile split over the
+// 256 / (CP/4)^2 thread groups, whose sums are added in a fixed order.  Each
+// tile is summed by itself and then added up.  C^2 FMA per pixel against 8 C
+// bytes.
+constexpr int kWgPx = 128, kWgStride = kWgPx + 4;
+template <int CP>
+__global__ void __launch_bounds__(256)
+weight_grad(const float* __restrict__ gz, const float* __restrict__ in, float* __restrict__ partial, int B, int C,
+            int P) {
+  constexpr int G = CP / 4, GT = G * G;
+  constexpr int SPLITS = 256 / GT < 32 ? 256 / GT : 32;  // at most one per 16-byte piece of a tile
+  extern __shared__ __align__(16) float sm_wg[];
+  float* sg = sm_wg;
+  float* sh = sm_wg + CP * kWgStride;
+  const int tid = threadIdx.x, grp = tid % GT, sp = tid / GT;
+  const int og = grp / G, ig = grp % G;
+  const bool on = sp < SPLITS;
+  const int tiles_b = P / kWgPx, tiles = B * tiles_b;  // P = N^2 >= 256, a power of two
+  float tot[4][4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tot[o][i] = 0.f;
+  for (int c = C; c < CP; ++c)
+    for (int x = tid; x < kWgPx; x += blockDim.x) sg[c * kWgStride + x] = sh[c * kWgStride + x] = 0.f;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int b = t / tiles_b, p0 = (t - b * tiles_b) * kWgPx;
+    __syncthreads();
+    for (int i = tid; i < C * (kWgPx / 4); i += blockDim.x) {
+      const int c = i / (kWgPx / 4), xq = i % (kWgPx / 4);
+      const size_t o = ((size_t)b * C + c) * P + p0 + 4 * xq;
+      wf::cp_async16(sg + c * kWgStride + 4 * xq, gz + o);
+      wf::cp_async16(sh + c * kWgStride + 4 * xq, in + o);
+    }
+    wf::cp_async_commit();
+    wf::cp_async_wait<0>();
+    __syncthreads();
+    if (on) {
+      float acc[4][4];
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
+      for (int xq = sp; xq < kWgPx / 4; xq += SPLITS) {
+        float4 g[4], h[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) g[o] = *reinterpret_cast<const float4*>(sg + (og + G * o) * kWgStride + 4 * xq);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) h[i] = *reinterpret_cast<const float4*>(sh + (ig + G * i) * kWgStride + 4 * xq);
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            acc[o][i] = fmaf(g[o].w, h[i].w, fmaf(g[o].z, h[i].z, fmaf(g[o].y, h[i].y, fmaf(g[o].x, h[i].x, acc[o][i]))));
+      }
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tot[o][i] += acc[o][i];
+    }
+  }
+  __syncthreads();
+  float* red = sm_wg;  // [SPLITS][CP][CP]: at most 2 CP kWgStride floats (checked below)
+  static_assert((CP >= 32 ? SPLITS : 8) * CP * CP <= 2 * CP * kWgStride, "reduction fits the tiles");
+  constexpr int RS = (CP >= 32) ? SPLITS : 8;  // splits reduced at a time
+  float sum[(CP * CP + 255) / 256];
+#pragma unroll
+  for (int q = 0; q < (CP * CP + 255) / 256; ++q) sum[q] = 0.f;
+  for (int s0 = 0; s0 < SPLITS; s0 += RS) {
+    if (on && sp >= s0 && sp < s0 + RS)
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[((sp - s0) * CP + og + G * o) * CP + ig + G * i] = tot[o][i];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < (CP * CP + 255) / 256; ++q) {
+      const int k = tid + 256 * q;
+      if (k < CP * CP)
+        for (int s = 0; s < RS; ++s) sum[q] += red[s * CP * CP + k];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < (CP * CP + 255) / 256; ++q) {
+    const int k = tid + 256 * q, o = k / CP, i = k % CP;
+    if (k < CP * CP && o < C && i < C) partial[((size_t)blockIdx.x * C + o) * C + i] = sum[q];
+  }
+}
+
+// out[i * stride_out ...]: sums of nblk partial vectors of n values, one warp
+// lane per value and eight partial sums per value (fixed order).  map = 0:
+// out[k]; map = 1: the lift's (o, {x0, x1, 1}) triples into gP [C][2] and gp
+// [C]; map = 2: C values into out, then one into out2.
+__global__ void __launch_bounds__(256)
+sum_partials(const float* __restrict__ partial, int nblk, int n, float* __restrict__ out, float* __restrict__ out2,
+             int map, int C) {
+  __shared__ float red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < nblk; ++b) s += partial[((size_t)b * CO + o) * (CI + 1) + i];
-  if (i < CI) gW[o * CI + i] = s;
-  else gb[o] = s;
-}
-
-// Row transform of R real rows of length N onto MX modes:
-// out[r][k] = scale_k * sum_x in[r][x] e^{-2 pi i k x / N}, scale_k = s0 (k=0) or s1.
-__global__ void dft_rows(const float* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tw_x,
-                         int R, int N, int MX, float s0, float s1) {
-  extern __shared__ float srow[];
-  for (int r = blockIdx.x; r < R; r += gridDim.x) {
-    __syncthreads();
-    for (int x = threadIdx.x; x < N; x += blockDim.x) srow[x] = in[(size_t)r * N + x];
-    __syncthreads();
-    // MX outputs, each a length-N sum split over the warp's lanes
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int k = warp; k < MX; k += nw) {
-      float re = 0.f, im = 0.f;
-      for (int x = lane; x < N; x += 32) {
-        const float2 w = tw_x[(size_t)k * N + x];  // e^{-2 pi i k x / N}
-        re = fmaf(srow[x], w.x, re);
-        im = fmaf(srow[x], w.y, im);
-      }
-      for (int s = 16; s > 0; s >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, s);
-        im += __shfl_xor_sync(0xffffffffu, im, s);
-      }
-      if (lane == 0) {
-        const float sc = k == 0 ? s0 : s1;
-        out[(size_t)r * MX + k] = make_float2(re * sc, im * sc);
-      }
+  if (k < n)
+    for (int b = w; b < nblk; b += 8) s += partial[(size_t)b * n + k];
+  red[w][lane] = s;
+  __syncthreads();
+  if (w != 0 || k >= n) return;
+  s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s += red[i][lane];
+  if (map == 0) {
+    out[k] = s;
+  } else if (map == 1) {
+    const int o = k / 3, i = k % 3;
+    if (o < C) {
+      if (i < 2) out[o * 2 + i] = s;
+      else out2[o] = s;
     }
+  } else {
+    if (k < C) out[k] = s;
+    else if (k == n - 1) out2[0] = s;
   }
 }
 
-// Column transform between N rows and the 2 MY retained k_y (per slice of
-// [N][MX] or [2MY][MX] complex values):
-//   forward (dir = -1): out[j][k] = sum_y in[y][k] e^{-2 pi i ky_j y / N}
-//   inverse (dir = +1): out[y][k] = sum_j in[j][k] e^{+2 pi i ky_j y / N}
-// tw_y[j][y] = e^{-2 pi i ky_j y / N}.
-__global__ void dft_cols(const float2* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tw_y,
-                         int S, int N, int MX, int MY2, int dir) {
-  const int nout = (dir < 0) ? MY2 : N;
-  const size_t total = (size_t)S * nout * MX;
+// Start of the backward pass: g_y = 2 (y - t) / (B ||t||^2), g_z of the last
+// layer (no activation) = Q g_y, and the block's partial sums of the
+// projection's gradient, g_y h_L and g_y ([blk][CP + 1]).
+template <int CP>
+__global__ void __launch_bounds__(kThreads)
+proj_bwd(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ inv,
+         const __half* __restrict__ Q, const float* __restrict__ hL, float* __restrict__ gz, float* __restrict__ partial,
+         int B, int C, int P) {
+  __shared__ float sQ[CP];
+  __shared__ float red[kThreads / 32][CP + 1];
+  for (int i = threadIdx.x; i < CP; i += blockDim.x) sQ[i] = i < C ? __half2float(Q[i]) : 0.f;
+  __syncthreads();
+  float acc[CP], sg = 0.f;
+#pragma unroll
+  for (int o = 0; o < CP; ++o) acc[o] = 0.f;
+  const size_t total = (size_t)B * P;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(g % MX);
-    const int j = (int)((g / MX) % nout);
-    const size_t sl = g / ((size_t)MX * nout);
-    float re = 0.f, im = 0.f;
-    if (dir < 0) {
-      const float2* src = in + sl * (size_t)N * MX + k;
-      const float2* w = tw_y + (size_t)j * N;
-      for (int y = 0; y < N; ++y) {
-        const float2 a = src[(size_t)y * MX], t = w[y];
-        re = fmaf(a.x, t.x, fmaf(-a.y, t.y, re));
-        im = fmaf(a.x, t.y, fmaf(a.y, t.x, im));
+    const int b = (int)(g / P), p = (int)(g % P);
+    const float gy = 2.f * (y[g] - t[g]) * inv[b];
+    sg += gy;
+#pragma unroll
+    for (int o = 0; o < CP; ++o)
+      if (o < C) {
+        const size_t idx = ((size_t)b * C + o) * P + p;
+        acc[o] = fmaf(gy, hL[idx], acc[o]);
+        gz[idx] = sQ[o] * gy;
       }
-    } else {
-      const float2* src = in + sl * (size_t)MY2 * MX + k;
-      for (int jj = 0; jj < MY2; ++jj) {
-        const float2 a = src[(size_t)jj * MX], t0 = tw_y[(size_t)jj * N + j];
-        const float2 t = make_float2(t0.x, -t0.y);  // conjugate: e^{+...}
-        re = fmaf(a.x, t.x, fmaf(-a.y, t.y, re));
-        im = fmaf(a.x, t.y, fmaf(a.y, t.x, im));
-      }
-    }
-    out[g] = make_float2(re, im);
   }
-}
-
-// out[r][x] (+)= scale * ( c0 Re(in[r][0]) + c1 sum_{k>=1} Re(in[r][k] e^{+2 pi i k x / N}) )
-__global__ void idft_rows(const float2* __restrict__ in, float* __restrict__ out, const float2* __restrict__ tw_x,
-                          int R, int N, int MX, float c0, float c1, float scale, int accumulate) {
-  extern __shared__ float2 srowc[];
-  for (int r = blockIdx.x; r < R; r += gridDim.x) {
-    __syncthreads();
-    for (int k = threadIdx.x; k < MX; k += blockDim.x) srowc[k] = in[(size_t)r * MX + k];
-    __syncthreads();
-    for (int x = threadIdx.x; x < N; x += blockDim.x) {
-      float s = c0 * srowc[0].x;
-      for (int k = 1; k < MX; ++k) {
-        const float2 a = srowc[k], t = tw_x[(size_t)k * N + x];  // e^{-i}; Re(a e^{+i}) = a.x t.x + a.y t.y
-        s = fmaf(c1, fmaf(a.x, t.x, a.y * t.y), s);
-      }
-      const size_t idx = (size_t)r * N + x;
-      out[idx] = accumulate ? out[idx] + scale * s : scale * s;
-    }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 0; o <= CP; ++o) {
+    float v = o < CP ? acc[o < CP ? o : 0] : sg;
+    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    if (lane == 0) red[w][o] = v;
   }
-}
-
-// Y[b][o][m] = sum_i R[i][o][m] X[b][i][m]  (complex; R in FP16 pairs)
-__global__ void mix_fwd(const float2* __restrict__ X, const __half2* __restrict__ R, float2* __restrict__ Y, int B,
-                        int C, int NM) {
-  const size_t total = (size_t)B * C * NM;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int m = (int)(g % NM), o = (int)((g / NM) % C);
-    const int b = (int)(g / ((size_t)NM * C));
-    float re = 0.f, im = 0.f;
-    for (int i = 0; i < C; ++i) {
-      const float2 r = __half22float2(R[((size_t)i * C + o) * NM + m]);
-      const float2 x = X[((size_t)b * C + i) * NM + m];
-      re = fmaf(r.x, x.x, fmaf(-r.y, x.y, re));
-      im = fmaf(r.x, x.y, fmaf(r.y, x.x, im));
-    }
-    Y[g] = make_float2(re, im);
-  }
-}
-
-// g_X[b][i][m] = sum_o conj(R[i][o][m]) g_Y[b][o][m]
-__global__ void mix_bwd_x(const float2* __restrict__ gY, const __half2* __restrict__ R, float2* __restrict__ gX, int B,
-                          int C, int NM) {
-  const size_t total = (size_t)B * C * NM;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int m = (int)(g % NM), i = (int)((g / NM) % C);
-    const int b = (int)(g / ((size_t)NM * C));
-    float re = 0.f, im = 0.f;
-    for (int o = 0; o < C; ++o) {
-      const float2 r = __half22float2(R[((size_t)i * C + o) * NM + m]);
-      const float2 y = gY[((size_t)b * C + o) * NM + m];
-      re = fmaf(r.x, y.x, fmaf(r.y, y.y, re));
-      im = fmaf(r.x, y.y, fmaf(-r.y, y.x, im));
-    }
-    gX[g] = make_float2(re, im);
-  }
-}
-
-// g_R[i][o][m] = sum_b g_Y[b][o][m] conj(X[b][i][m]), written as (re, im) pairs
-__global__ void mix_bwd_r(const float2* __restrict__ gY, const float2* __restrict__ X, float* __restrict__ gR, int B,
-                          int C, int NM) {
-  const size_t total = (size_t)C * C * NM;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int m = (int)(g % NM), o = (int)((g / NM) % C);
-    const int i = (int)(g / ((size_t)NM * C));
-    float re = 0.f, im = 0.f;
-    for (int b = 0; b < B; ++b) {
-      const float2 y = gY[((size_t)b * C + o) * NM + m];
-      const float2 x = X[((size_t)b * C + i) * NM + m];
-      re = fmaf(y.x, x.x, fmaf(y.y, x.y, re));
-      im = fmaf(y.y, x.x, fmaf(-y.x, x.y, im));
-    }
-    gR[2 * g] = re;
-    gR[2 * g + 1] = im;
+  __syncthreads();
+  for (int o = threadIdx.x; o <= CP; o += blockDim.x) {
+    float v = 0.f;
+    for (int i = 0; i < kThreads / 32; ++i) v += red[i][o];
+    partial[(size_t)blockIdx.x * (CP + 1) + o] = v;
   }
 }
 
@@ -337,30 +845,26 @@ __global__ void loss_partial(const float* __restrict__ y, const float* __restric
   }
 }
 
-// loss = mean_b num_b / den_b; inv[b] = 1 / (B den_b)
+// loss = mean_b num_b / den_b; inv[b] = 1 / (B den_b).  One warp: lane k sums
+// block k of every map (nblk = 32), then a fixed tree.
 __global__ void loss_fin(const double* __restrict__ part, int nblk, int B, double* __restrict__ loss,
                          float* __restrict__ inv) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double L = 0.0;
   for (int b = 0; b < B; ++b) {
     double n = 0.0, d = 0.0;
-    for (int k = 0; k < nblk; ++k) {
+    for (int k = threadIdx.x; k < nblk; k += 32) {
       n += part[((size_t)b * nblk + k) * 2];
       d += part[((size_t)b * nblk + k) * 2 + 1];
     }
+    for (int s = 16; s > 0; s >>= 1) {
+      n += __shfl_xor_sync(0xffffffffu, n, s);
+      d += __shfl_xor_sync(0xffffffffu, d, s);
+    }
     d = d > 0.0 ? d : 1.0;
     L += n / d;
-    inv[b] = (float)(1.0 / (B * d));
+    if (threadIdx.x == 0) inv[b] = (float)(1.0 / (B * d));
   }
-  *loss = L / B;
-}
-
-// g_y = 2 (y - t) inv[b]
-__global__ void loss_grad(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ inv,
-                          float* __restrict__ gy, int B, int P) {
-  const size_t total = (size_t)B * P;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x)
-    gy[g] = 2.f * (y[g] - t[g]) * inv[g / P];
+  if (threadIdx.x == 0) *loss = L / B;
 }
 
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -445,19 +949,18 @@ struct wf_fno_s {
   long long step = 0;
   // activations
   float* h = nullptr;         // [L+1][B][C][P]
-  float* z = nullptr;         // [L][B][C][P] pre-activations
-  float* kbuf = nullptr;      // [B][C][P] spectral branch output
+  float* dact = nullptr;      // [L-1][B][C][P] GELU'(z) of the hidden layers
   float* y = nullptr;         // [B][P]
-  float* gh = nullptr;        // [B][C][P] gradient wrt h_l
-  float* gz = nullptr;        // [B][C][P]
-  float* gy = nullptr;        // [B][P]
-  float2 *A = nullptr, *X = nullptr, *Y = nullptr;  // [L][B][C][N][MX], [L][B][C][2MY][MX], scratch
-  float2 *tw_x = nullptr, *tw_y = nullptr;
+  float* gz = nullptr;        // [B][C][P] gradient wrt the current layer's z
+  float2 *Xp = nullptr, *X = nullptr, *gY = nullptr, *Y = nullptr;  // partial sums, [L][B][C][2MY][MX], ...
+  float* S = nullptr;         // [B][N][MX][2][CP]
+  float2 *tw_x = nullptr, *tw_y = nullptr, *tw_k = nullptr;
   float* wpart = nullptr;
+  int OG = 1, KG = 1, sms = 1, synth_per_sm = 1, adj_per_sm = 1;
   double* lpart = nullptr;
   double* dloss = nullptr;
   float* inv = nullptr;
-  int wblk = 0, lblk = 0;
+  int lblk = 0;
   std::vector<void*> allocs;
 };
 
@@ -475,105 +978,193 @@ bool alloc(wf_fno_s* F, T** p, size_t n) {
 
 size_t P_(const wf_fno_s* F) { return (size_t)F->n * F->n; }
 size_t act_(const wf_fno_s* F) { return (size_t)F->batch * F->lay.width * P_(F); }
-size_t spec_(const wf_fno_s* F) { return (size_t)F->batch * F->lay.width * F->n * F->lay.mx; }
 size_t modes_(const wf_fno_s* F) { return (size_t)2 * F->lay.my * F->lay.mx; }
+int an_blocks(int n) { return (n / 2) / (std::min(kAnRows, n) / 2); }
+int an_threads(int n, int KG) { return (std::min(kAnRows, n) / 4 * 2 * KG + 31) / 32 * 32; }
+size_t an_smem(int KG, int MX) {
+  return std::max(sizeof(float) * 2 * kAnX * kAnRows + sizeof(float4) * kAnX * 2 * KG, sizeof(float2) * kAnRows * MX);
+}
+size_t cols_smem(int MY2, int CP) { return sizeof(float2) * MY2 * (kColY + CP); }
 
-// spectral convolution of h_l (B*C slices) into kbuf, keeping A and X of layer l
-int spectral_fwd(wf_fno_s* F, int l, const float* hin, int B) {
-  const int C = F->lay.width, N = F->n, MX = F->lay.mx, MY2 = 2 * F->lay.my;
-  const int S = B * C;
-  float2* A = F->A + (size_t)l * spec_(F);
-  float2* X = F->X + (size_t)l * F->batch * C * modes_(F);
-  dft_rows<<<grid_for((size_t)S * N * 32) / 8 + 1, kThreads, N * sizeof(float), F->stream>>>(hin, A, F->tw_x, S * N, N,
-                                                                                             MX, 1.f, 1.f);
-  dft_cols<<<grid_for((size_t)S * MY2 * MX), kThreads, 0, F->stream>>>(A, X, F->tw_y, S, N, MX, MY2, -1);
+// pixels or gradients [B][C][N][N] -> partial sums of the retained modes in Xp
+void launch_analysis(wf_fno_s* F, const float* in, int B, float s0, float s1) {
+  const int C = F->lay.width, N = F->n, MX = F->lay.mx;
+  analysis<<<B * C * an_blocks(N), an_threads(N, F->KG), an_smem(F->KG, MX), F->stream>>>(
+      in, F->Xp, F->tw_k, F->tw_y, N, MX, 2 * F->lay.my, F->KG, s0, s1);
+}
+
+void launch_mix(wf_fno_s* F, int l, float2* X, int B, int bwd) {
+  const int C = F->lay.width, NM = (int)modes_(F);
   const __half2* R = reinterpret_cast<const __half2*>(F->half + F->lay.oR[l]);
-  mix_fwd<<<grid_for((size_t)S * MY2 * MX), kThreads, 0, F->stream>>>(X, R, F->Y, B, C, MY2 * MX);
-  // the inverse: columns back to N rows (reuse A's space of this call as scratch in Y order)
-  float2* Bm = F->A + (size_t)F->lay.layers * spec_(F);  // one extra slot
-  dft_cols<<<grid_for((size_t)S * N * MX), kThreads, 0, F->stream>>>(F->Y, Bm, F->tw_y, S, N, MX, MY2, +1);
-  const float sc = 1.f / ((float)N * (float)N);
-  idft_rows<<<grid_for((size_t)S * N) / 4 + 1, kThreads, MX * sizeof(float2), F->stream>>>(Bm, F->kbuf, F->tw_x, S * N,
-                                                                                            N, MX, 1.f, 2.f, sc, 0);
-  return (int)cudaGetLastError();
+  mix<<<dim3((NM + kMixModes - 1) / kMixModes, B), kThreads, 0, F->stream>>>(F->Xp, an_blocks(F->n), R, X, F->Y, C,
+                                                                             8 * F->OG, NM, bwd);
 }
 
-int forward(wf_fno_s* F, const float* x, int B) {
-  const Layout& L = F->lay;
-  const int C = L.width;
-  const int P = (int)P_(F);
-  const size_t gsz = grid_for((size_t)B * P);
-  pointwise_fwd<<<gsz, kThreads, 0, F->stream>>>(x, F->half + L.oP, F->master + L.op, nullptr, nullptr, F->h, B,
-                                                 L.cin, C, P, 0);
-  for (int l = 0; l < L.layers; ++l) {
-    float* hin = F->h + (size_t)l * act_(F);
-    float* hout = F->h + (size_t)(l + 1) * act_(F);
-    int rc = spectral_fwd(F, l, hin, B);
-    if (rc) return rc;
-    pointwise_fwd<<<gsz, kThreads, 0, F->stream>>>(hin, F->half + L.oW[l], F->master + L.ow[l], F->kbuf,
-                                                   F->z + (size_t)l * act_(F), hout, B, C, C, P,
-                                                   l < L.layers - 1 ? 1 : 0);
+void launch_synth_cols(wf_fno_s* F, int B, float c0, float c1) {
+  const int N = F->n, MX = F->lay.mx, MY2 = 2 * F->lay.my, CP = 8 * F->OG;
+  synth_cols<<<dim3((N / 2 + kColY - 1) / kColY, MX, B), 256, cols_smem(MY2, CP), F->stream>>>(F->Y, F->S, F->tw_y, N,
+                                                                                               MX, MY2, CP, c0, c1);
+}
+
+template <bool ADJ>
+int synth_grid(const wf_fno_s* F, const SynthGeom& g) {
+  // whole multiples of the pixel tiles of a row, at most one wave
+  const int wave = F->sms * (ADJ ? F->adj_per_sm : F->synth_per_sm);
+  const int n = std::min(g.units, wave);
+  return std::max(g.nxt, n / g.nxt * g.nxt);
+}
+
+template <bool ADJ>
+int launch_synth(wf_fno_s* F, SynthArgs a, int B) {
+  const SynthGeom g = synth_geom(F->OG, B, F->lay.width, F->n, F->lay.mx);
+  a.B = B;
+  a.C = F->lay.width;
+  a.N = F->n;
+  a.MX = F->lay.mx;
+  a.XT = g.XT;
+  a.RT = g.RT;
+  a.nxt = g.nxt;
+  a.units = g.units;
+  a.S = F->S;
+  a.tw_x = F->tw_x;
+  const int grid = synth_grid<ADJ>(F, g);
+  switch (F->OG) {
+    case 1: synth<1, ADJ><<<grid, 1 * synth_pg(1), g.smem, F->stream>>>(a); break;
+    case 2: synth<2, ADJ><<<grid, 2 * synth_pg(2), g.smem, F->stream>>>(a); break;
+    case 4: synth<4, ADJ><<<grid, 4 * synth_pg(4), g.smem, F->stream>>>(a); break;
+    default: synth<8, ADJ><<<grid, 8 * synth_pg(8), g.smem, F->stream>>>(a); break;
   }
-  pointwise_fwd<<<gsz, kThreads, 0, F->stream>>>(F->h + (size_t)L.layers * act_(F), F->half + L.oQ, F->master + L.oq,
-                                                 nullptr, nullptr, F->y, B, C, 1, P, 0);
+  return grid;
+}
+
+template <int OG, bool ADJ>
+cudaError_t prepare_synth(size_t smem, int* per_sm) {
+  cudaError_t e = cudaFuncSetAttribute(synth<OG, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, synth<OG, ADJ>, OG * synth_pg(OG), smem);
+  if (e == cudaSuccess && *per_sm < 1) e = cudaErrorInvalidConfiguration;
+  return e;
+}
+
+constexpr size_t wg_smem(int CP) { return sizeof(float) * 2 * CP * kWgStride; }
+
+// shared-memory sizes and blocks per SM of this network's kernels
+cudaError_t prepare_kernels(wf_fno_s* F) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&F->sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t sm = synth_geom(F->OG, 1, F->lay.width, F->n, F->lay.mx).smem;
+  if (e == cudaSuccess) {
+    switch (F->OG) {
+      case 1: e = prepare_synth<1, false>(sm, &F->synth_per_sm); break;
+      case 2: e = prepare_synth<2, false>(sm, &F->synth_per_sm); break;
+      case 4: e = prepare_synth<4, false>(sm, &F->synth_per_sm); break;
+      default: e = prepare_synth<8, false>(sm, &F->synth_per_sm); break;
+    }
+  }
+  if (e == cudaSuccess) {
+    switch (F->OG) {
+      case 1: e = prepare_synth<1, true>(sm, &F->adj_per_sm); break;
+      case 2: e = prepare_synth<2, true>(sm, &F->adj_per_sm); break;
+      case 4: e = prepare_synth<4, true>(sm, &F->adj_per_sm); break;
+      default: e = prepare_synth<8, true>(sm, &F->adj_per_sm); break;
+    }
+  }
+  if (e == cudaSuccess && F->OG == 8)
+    e = cudaFuncSetAttribute(weight_grad<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wg_smem(64));
+  return e;
+}
+
+// the network on x into y (device); keep: the activations and act' of every
+// layer stay for the backward pass
+int forward(wf_fno_s* F, const float* x, float* y, int B, bool keep) {
+  const Layout& L = F->lay;
+  const int C = L.width, P = (int)P_(F);
+  lift_fwd<<<grid_for((size_t)B * P), kThreads, 0, F->stream>>>(x, F->half + L.oP, F->master + L.op, F->h, B, C, P);
+  const float sc = 1.f / ((float)F->n * (float)F->n);
+  for (int l = 0; l < L.layers; ++l) {
+    const bool last = l == L.layers - 1;
+    float* hin = F->h + (size_t)(keep ? l : (l & 1)) * act_(F);
+    float* hout = F->h + (size_t)(keep ? l + 1 : ((l + 1) & 1)) * act_(F);
+    launch_analysis(F, hin, B, 1.f, 1.f);
+    launch_mix(F, l, F->X + (size_t)l * F->batch * C * modes_(F), B, 0);
+    launch_synth_cols(F, B, sc, 2.f * sc);
+    SynthArgs a{};
+    a.in = hin;
+    a.W = F->half + L.oW[l];
+    a.bias = F->master + L.ow[l];
+    a.act = !last;
+    a.out = (last && !keep) ? nullptr : hout;
+    a.dact = (keep && !last) ? F->dact + (size_t)l * act_(F) : nullptr;
+    if (last) {
+      a.Q = F->half + L.oQ;
+      a.q = F->master + L.oq;
+      a.y = y;
+    }
+    launch_synth<false>(F, a, B);
+  }
   return (int)cudaGetLastError();
 }
 
-int pointwise_weight_grad(wf_fno_s* F, const float* gz, const float* in, int B, int CI, int CO, float* gW,
-                          float* gb) {
-  const int P = (int)P_(F);
-  dim3 grid(F->wblk, CO);
-  pointwise_bwd_w<<<grid, kThreads, 0, F->stream>>>(gz, in, F->wpart, B, CI, CO, P);
-  pointwise_bwd_w_fin<<<(CO * (CI + 1) + 255) / 256, 256, 0, F->stream>>>(F->wpart, F->wblk, CI, CO, gW, gb);
-  return (int)cudaGetLastError();
+void weight_gradient(wf_fno_s* F, const float* in, int B, float* gW) {
+  const int P = (int)P_(F), C = F->lay.width;
+  const int tiles = B * (P / kWgPx), grid = std::min(tiles, 2 * F->sms);
+  switch (F->OG) {
+    case 1: weight_grad<8><<<grid, 256, wg_smem(8), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
+    case 2: weight_grad<16><<<grid, 256, wg_smem(16), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
+    case 4: weight_grad<32><<<grid, 256, wg_smem(32), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
+    default: weight_grad<64><<<grid, 256, wg_smem(64), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
+  }
+  sum_partials<<<(C * C + 31) / 32, 256, 0, F->stream>>>(F->wpart, grid, C * C, gW, nullptr, 0, C);
 }
 
-// loss and gradient of the loss into F->grad (x, t device arrays)
+// loss and gradient of the loss into F->grad (x, t device arrays), after
+// forward(..., keep)
 int backward(wf_fno_s* F, const float* x, const float* t, int B) {
   const Layout& L = F->lay;
-  const int C = L.width, N = F->n, MX = L.mx, MY2 = 2 * L.my;
+  const int C = L.width, N = F->n, NM = (int)modes_(F), CP = 8 * F->OG;
   const int P = (int)P_(F);
-  const size_t gsz = grid_for((size_t)B * P);
-  // loss and dL/dy
-  dim3 lg(F->lblk, B);
-  loss_partial<<<lg, kThreads, 0, F->stream>>>(F->y, t, F->lpart, P);
+  loss_partial<<<dim3(F->lblk, B), kThreads, 0, F->stream>>>(F->y, t, F->lpart, P);
   loss_fin<<<1, 32, 0, F->stream>>>(F->lpart, F->lblk, B, F->dloss, F->inv);
-  loss_grad<<<gsz, kThreads, 0, F->stream>>>(F->y, t, F->inv, F->gy, B, P);
-  // projection Q
+  // projection Q, and g_z of the last layer
   const float* hL = F->h + (size_t)L.layers * act_(F);
-  pointwise_weight_grad(F, F->gy, hL, B, C, 1, F->grad + L.oQ, F->grad + L.oq);
-  pointwise_bwd_in<<<gsz, kThreads, 0, F->stream>>>(F->gy, nullptr, nullptr, F->half + L.oQ, F->gh, B, C, 1, P, 0, 0);
-  const int S = B * C;
+  const int pgrid = std::min(grid_for((size_t)B * P), 2 * F->sms);
+  const __half* Q = F->half + L.oQ;
+  switch (F->OG) {
+    case 1: proj_bwd<8><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
+    case 2: proj_bwd<16><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
+    case 4: proj_bwd<32><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
+    default: proj_bwd<64><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
+  }
+  sum_partials<<<(CP + 32) / 32, 256, 0, F->stream>>>(F->wpart, pgrid, CP + 1, F->grad + L.oQ, F->grad + L.oq, 2, C);
   const float sc = 1.f / ((float)N * (float)N);
   for (int l = L.layers - 1; l >= 0; --l) {
     const float* hin = F->h + (size_t)l * act_(F);
-    // through the activation: gz = gh * act'(z)
-    pointwise_bwd_in<<<gsz, kThreads, 0, F->stream>>>(F->gh, F->z + (size_t)l * act_(F), F->gz, F->half + L.oW[l],
-                                                      nullptr, B, C, C, P, l < L.layers - 1 ? 1 : 0, 0);
-    pointwise_weight_grad(F, F->gz, hin, B, C, C, F->grad + L.oW[l], F->grad + L.ow[l]);
-    // spectral branch: g_Bm = (c_k / N^2) rowDFT(gz), g_Y = colDFT(g_Bm), then R and X
-    float2* gB = F->A + (size_t)L.layers * spec_(F);
-    dft_rows<<<grid_for((size_t)S * N * 32) / 8 + 1, kThreads, N * sizeof(float), F->stream>>>(F->gz, gB, F->tw_x,
-                                                                                               S * N, N, MX, sc,
-                                                                                               2.f * sc);
-    dft_cols<<<grid_for((size_t)S * MY2 * MX), kThreads, 0, F->stream>>>(gB, F->Y, F->tw_y, S, N, MX, MY2, -1);
+    // spectral branch: g_Y = (c_k / N^2) DFT(g_z), then R and X
+    launch_analysis(F, F->gz, B, sc, 2.f * sc);
+    launch_mix(F, l, F->gY, B, 1);
     const float2* X = F->X + (size_t)l * F->batch * C * modes_(F);
-    mix_bwd_r<<<grid_for((size_t)C * C * MY2 * MX), kThreads, 0, F->stream>>>(F->Y, X, F->grad + L.oR[l], B, C,
-                                                                               MY2 * MX);
-    const __half2* R = reinterpret_cast<const __half2*>(F->half + L.oR[l]);
-    float2* gX = F->A + (size_t)l * spec_(F);  // A of layer l is no longer needed: scratch for g_X
-    mix_bwd_x<<<grid_for((size_t)S * MY2 * MX), kThreads, 0, F->stream>>>(F->Y, R, gX, B, C, MY2 * MX);
-    // g_A = colIDFT(g_X) into gB, then g_h = Re rowIDFT(g_A) (weights 1, no scale)
-    dft_cols<<<grid_for((size_t)S * N * MX), kThreads, 0, F->stream>>>(gX, gB, F->tw_y, S, N, MX, MY2, +1);
-    // pointwise branch of g_h, then add the spectral branch
-    pointwise_bwd_in<<<gsz, kThreads, 0, F->stream>>>(F->gz, nullptr, nullptr, F->half + L.oW[l], F->gh, B, C, C, P, 0,
-                                                      0);
-    idft_rows<<<grid_for((size_t)S * N) / 4 + 1, kThreads, MX * sizeof(float2), F->stream>>>(gB, F->gh, F->tw_x,
-                                                                                              S * N, N, MX, 1.f, 1.f,
-                                                                                              1.f, 1);
+    mix_bwd_r<<<dim3((NM + 127) / 128, (C + 3) / 4, (C + 3) / 4), 128, 0, F->stream>>>(
+        F->gY, X, F->grad + L.oR[l], F->grad + L.ow[l], B, C, NM, (float)N * (float)N);
+    launch_synth_cols(F, B, 1.f, 1.f);
+    weight_gradient(F, hin, B, F->grad + L.oW[l]);
+    // g_h of this layer's input = W^T g_z + Re(inverse of g_X), through the
+    // activation below it in place, or into the lift's gradient
+    SynthArgs a{};
+    a.in = F->gz;
+    a.W = F->half + L.oW[l];
+    if (l > 0) {
+      a.out = F->gz;
+      a.mul = F->dact + (size_t)(l - 1) * act_(F);
+    } else {
+      a.x = x;
+      a.lpart = F->wpart;
+    }
+    const int g = launch_synth<true>(F, a, B);
+    if (l == 0)
+      sum_partials<<<(CP * 3 + 31) / 32, 256, 0, F->stream>>>(F->wpart, g, CP * 3, F->grad + L.oP, F->grad + L.op, 1,
+                                                              C);
   }
-  // lift P
-  pointwise_weight_grad(F, F->gh, x, B, L.cin, C, F->grad + L.oP, F->grad + L.op);
   return (int)cudaGetLastError();
 }
 
@@ -611,18 +1202,28 @@ int wf_fno_create(wf_fno_t* out, int n, int batch, int width, int mx, int my, in
   F->batch = batch;
   F->stream = (cudaStream_t)stream;
   const size_t T = F->lay.total, P = (size_t)n * n;
-  F->wblk = 64;
   F->lblk = 32;
+  F->OG = width <= 8 ? 1 : (width <= 16 ? 2 : (width <= 32 ? 4 : 8));
+  F->KG = ((mx + 1) / 2 + 1) / 2;  // pairs of modes of one parity
+  const int CP = 8 * F->OG;
+  if (prepare_kernels(F) != cudaSuccess) {
+    cudaGetLastError();
+    wf_fno_destroy(F);
+    return WF_ECUDA;
+  }
+  // block partial sums: the weight gradients', the projection's, the lift's
+  const size_t wpart = std::max((size_t)2 * F->sms * std::max(width * width, CP + 1),
+                                (size_t)F->sms * F->adj_per_sm * CP * 3);
   bool ok = alloc(F, &F->master, T) && alloc(F, &F->grad, T) && alloc(F, &F->m1, T) && alloc(F, &F->m2, T) &&
             alloc(F, &F->half, T) && alloc(F, &F->h, (size_t)(layers + 1) * act_(F)) &&
-            alloc(F, &F->z, (size_t)layers * act_(F)) && alloc(F, &F->kbuf, act_(F)) &&
-            alloc(F, &F->y, (size_t)batch * P) && alloc(F, &F->gh, act_(F)) && alloc(F, &F->gz, act_(F)) &&
-            alloc(F, &F->gy, (size_t)batch * P) && alloc(F, &F->A, (size_t)(layers + 1) * spec_(F)) &&
+            alloc(F, &F->dact, (size_t)std::max(layers - 1, 1) * act_(F)) && alloc(F, &F->y, (size_t)batch * P) &&
+            alloc(F, &F->gz, act_(F)) && alloc(F, &F->Xp, (size_t)batch * width * an_blocks(n) * modes_(F)) &&
             alloc(F, &F->X, (size_t)layers * batch * width * modes_(F)) &&
-            alloc(F, &F->Y, (size_t)batch * width * modes_(F)) && alloc(F, &F->tw_x, (size_t)mx * n) &&
-            alloc(F, &F->tw_y, (size_t)2 * my * n) &&
-            alloc(F, &F->wpart, (size_t)F->wblk * width * (kMaxWidth + 1)) &&
-            alloc(F, &F->lpart, (size_t)batch * F->lblk * 2) && alloc(F, &F->dloss, 1) && alloc(F, &F->inv, batch);
+            alloc(F, &F->gY, (size_t)batch * width * modes_(F)) && alloc(F, &F->Y, (size_t)batch * CP * modes_(F)) &&
+            alloc(F, &F->S, (size_t)batch * n * mx * 2 * CP) && alloc(F, &F->tw_x, (size_t)mx * n) &&
+            alloc(F, &F->tw_y, (size_t)2 * my * n) && alloc(F, &F->tw_k, (size_t)(n / 2) * 4 * F->KG) &&
+            alloc(F, &F->wpart, wpart) && alloc(F, &F->lpart, (size_t)batch * F->lblk * 2) &&
+            alloc(F, &F->dloss, 1) && alloc(F, &F->inv, batch);
   if (!ok) {
     wf_fno_destroy(F);
     return WF_ENOMEM;
@@ -641,9 +1242,14 @@ int wf_fno_create(wf_fno_t* out, int n, int batch, int width, int mx, int my, in
       ty[(size_t)j * n + y] = make_float2((float)cos(a), (float)-sin(a));
     }
   }
+  // the analysis's row table: [x][parity][k / 2], x < n/2, 0 beyond mx
+  std::vector<float2> tk((size_t)(n / 2) * 4 * F->KG, make_float2(0.f, 0.f));
+  for (int x = 0; x < n / 2; ++x)
+    for (int k = 0; k < mx; ++k) tk[(size_t)x * 4 * F->KG + (k & 1) * 2 * F->KG + k / 2] = tx[(size_t)k * n + x];
   const cudaMemcpyKind k = dev_ptr(params) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   ok = cudaMemcpy(F->tw_x, tx.data(), tx.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
        cudaMemcpy(F->tw_y, ty.data(), ty.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
+       cudaMemcpy(F->tw_k, tk.data(), tk.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
        cudaMemcpy(F->master, params, T * sizeof(float), k) == cudaSuccess &&
        cudaMemset(F->m1, 0, T * sizeof(float)) == cudaSuccess && cudaMemset(F->m2, 0, T * sizeof(float)) == cudaSuccess &&
        cudaMemset(F->grad, 0, T * sizeof(float)) == cudaSuccess;
@@ -666,16 +1272,13 @@ long long wf_fno_num_params(wf_fno_t F) { return F ? (long long)F->lay.total : -
 
 int wf_fno_forward(wf_fno_t F, const float* x, float* y, int nb) {
   if (!F || !x || !y || nb < 1 || nb > F->batch || !dev_ptr(x) || !dev_ptr(y)) return WF_EINVAL;
-  int rc = forward(F, x, nb);
-  if (rc) return WF_ECUDA;
-  if (cudaMemcpyAsync(y, F->y, (size_t)nb * P_(F) * sizeof(float), cudaMemcpyDeviceToDevice, F->stream) != cudaSuccess)
-    return WF_ECUDA;
+  if (forward(F, x, y, nb, false)) return WF_ECUDA;
   return cudaStreamSynchronize(F->stream) == cudaSuccess ? WF_OK : WF_ECUDA;
 }
 
 int wf_fno_gradient(wf_fno_t F, const float* x, const float* t, int nb, float* grad, double* loss) {
   if (!F || !x || !t || nb < 1 || nb > F->batch || !dev_ptr(x) || !dev_ptr(t)) return WF_EINVAL;
-  if (forward(F, x, nb) || backward(F, x, t, nb)) return WF_ECUDA;
+  if (forward(F, x, F->y, nb, true) || backward(F, x, t, nb)) return WF_ECUDA;
   if (grad && cudaMemcpyAsync(grad, F->grad, F->lay.total * sizeof(float), cudaMemcpyDefault, F->stream) != cudaSuccess)
     return WF_ECUDA;
   double l = 0.0;
@@ -688,7 +1291,7 @@ int wf_fno_gradient(wf_fno_t F, const float* x, const float* t, int nb, float* g
 
 int wf_fno_train_step(wf_fno_t F, const float* x, const float* t, int nb, double lr, double* loss) {
   if (!F || !x || !t || nb < 1 || nb > F->batch || !(lr > 0.0) || !dev_ptr(x) || !dev_ptr(t)) return WF_EINVAL;
-  if (forward(F, x, nb) || backward(F, x, t, nb)) return WF_ECUDA;
+  if (forward(F, x, F->y, nb, true) || backward(F, x, t, nb)) return WF_ECUDA;
   F->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)F->step), c2 = 1.f - powf(b2, (float)F->step);
