@@ -79,15 +79,15 @@ __global__ void to_half_kernel(const float* __restrict__ src, __half* __restrict
 // read twice and written once.  Before, the transforms were one output per
 // thread with both operands from L2, and the channel products kept their
 // operands in local memory: inference of one 512^2 map (32 channels, 16 x 32
-// modes, 4 layers) 6359 us then, 432 us now; the gradient of eight 256^2 maps
-// 15 575 us then, 1697 us now.
+// modes, 4 layers) 6359 us then, 303 us now; the gradient of eight 256^2 maps
+// 15 600 us then, 1340 us now.
 //
 // Both transforms use e^{2 pi i k (x + N/2) / N} = (-1)^k e^{2 pi i k x / N}: rows
 // (and columns) a half period apart are added and subtracted first, the sums
 // serve the even k and the differences the odd k, so every direct sum runs
 // over N/2 terms (or gives two outputs).
 
-constexpr int kAnRows = 32;   // rows of an analysis block, half of them N/2 further on
+constexpr int kAnRows = 64;   // rows of an analysis block, half of them N/2 further on
 constexpr int kAnX = 32;      // pixels of a row staged at a time
 constexpr int kMixModes = 8;  // modes of a mix block
 constexpr int kColY = 32;     // row pairs of a column-synthesis block
@@ -111,41 +111,45 @@ __global__ void lift_fwd(const float* __restrict__ x, const __half* __restrict__
 
 // Partial column sums of the row DFTs of one channel's rows:
 //   part[slice][block][j][k] = sc_k sum_{y in block} e^{-2 pi i ky_j y / N} sum_x in[y][x] e^{-2 pi i k x / N}
-// for the 32 rows {y0 .. y0 + 15} and the same + N/2.  The row DFT is a
-// register-tiled product of the folded rows (staged transposed in shared
-// memory, row groups XOR-swizzled by x so that both the stores and the
-// 16-byte loads are conflict-free) with the twiddle table tw_k[x][slot]
-// (slot = parity * 2 KG + k / 2): 4 rows x 2 modes per thread, 16 FMA per two
-// 16-byte loads.  Sums run over 32 pixels at a time and are then added up, to
-// keep the rounding of the long sums near that of a tree.
-// FP32-issue bound: N/2 * 32 FMA per row for 16 modes.
-__global__ void __launch_bounds__(128)
+// for the 64 rows {y0 .. y0 + 31} and the same + N/2.  The row DFT is a
+// register-tiled product of the folded rows with the twiddle table
+// tw_k[x][parity][mode]: a warp takes eight modes of one parity for all rows, a
+// lane two rows, so the twiddles are the same for the whole warp (broadcast
+// loads) and a step is 32 FMA for one 8-byte and four broadcast 16-byte loads
+// (with 4 rows x 2 modes a thread, both operands lane-dependent, the shared
+// loads took twice the FMA's time: 42 us for eight 256^2 maps of 32 channels).
+// The folded rows are staged transposed, row groups XOR-swizzled by x so that
+// the stores are conflict-free.  KS groups of warps share the pixels of a row
+// (each with its own stage and its own barrier) so that few rows still fill
+// the SMs; their sums (of at most 128 terms) are added in a fixed order.  FP32
+// bound: N/2 * 32 FMA per row for 16 modes.
+template <int KS, int KW>
+__global__ void __launch_bounds__(KS * KW * 64, KW == 1 ? (KS == 4 ? 3 : 10) : 1)
 analysis(const float* __restrict__ in, float2* __restrict__ part, const float2* __restrict__ tw_k,
-         const float2* __restrict__ tw_y, int N, int MX, int MY2, int KG, float s0, float s1) {
+         const float2* __restrict__ tw_y, int N, int MX, int MY2, float s0, float s1) {
   extern __shared__ __align__(16) float sm_an[];
-  const int NX = min(kAnX, N / 2);                    // pixels staged at a time
-  float* st = sm_an;                                  // [2][kAnX][kAnRows] folded rows
-  float4* stw = reinterpret_cast<float4*>(sm_an + 2 * kAnX * kAnRows);  // [kAnX][2 KG] mode pairs
-  float2* sA = reinterpret_cast<float2*>(sm_an);      // [rows][MX] afterwards
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int GW = 2 * KW;                              // warps of a group: KW sets of 8 modes per parity
+  const int gt = GW * 32, grp = tid / gt, gtid = tid - grp * gt, gw = gtid >> 5;
   const int rows = min(kAnRows, N), RH = rows / 2, nblk = (N / 2) / RH;
   const int slice = blockIdx.x / nblk, yb = blockIdx.x - slice * nblk;
   const int y0 = yb * RH;
+  const int lx = min(5, 31 - __clz(N / 2)), NX = 1 << lx;  // pixels staged at a time
+  const size_t gsz = 2 * kAnX * kAnRows + kAnX * 2 * KW * 16;
+  float* st = sm_an + grp * gsz;                      // [2][kAnX][kAnRows] folded rows
+  float4* stw = reinterpret_cast<float4*>(st + 2 * kAnX * kAnRows);  // [kAnX][2 KW][4] mode pairs
   const float* src = in + (size_t)slice * N * N;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int RG = rows / 4;                            // row groups of 4
-  const int rg = tid % RG, kgp = tid / RG;            // kgp: parity * KG + pair of modes
-  const bool work = kgp < 2 * KG;
-  const int par = kgp >= KG ? 1 : 0;
-  float acc[4][4];                                    // [row][k0 re, k0 im, k1 re, k1 im]
+  const int par = gw >= KW ? 1 : 0;
+  float acc[2][16];                                   // [row][mode, re / im]
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
-  const int XQ = NX / 4;                              // 16-byte pieces of a row
-  for (int x0 = 0; x0 < N / 2; x0 += NX) {
-    __syncthreads();
-    for (int i = tid; i < rows * XQ; i += nt) {
-      const int r4 = i & 3, xq = (i >> 2) % XQ, rq = (i >> 2) / XQ;
+    for (int q = 0; q < 16; ++q) acc[r][q] = 0.f;
+  const int pieces = rows << (lx - 2);                // 16-byte pieces of the stage
+  for (int x0 = grp * NX; x0 < N / 2; x0 += KS * NX) {
+    asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gt) : "memory");
+    for (int i = gtid; i < pieces; i += gt) {
+      const int r4 = i & 3, xq = (i >> 2) & ((NX >> 2) - 1), rq = i >> lx;
       const int row = rq * 4 + r4;
       const int y = row < RH ? y0 + row : y0 + N / 2 + row - RH;
       const float4 a = *reinterpret_cast<const float4*>(src + (size_t)y * N + x0 + 4 * xq);
@@ -161,68 +165,90 @@ analysis(const float* __restrict__ in, float2* __restrict__ part, const float2* 
       d[2 * kAnRows] = a.z - b.z;
       d[3 * kAnRows] = a.w - b.w;
     }
-    for (int i = tid; i < NX * 2 * KG; i += nt)
-      stw[i] = *reinterpret_cast<const float4*>(tw_k + ((size_t)x0 * 2 * KG + i) * 2);
-    __syncthreads();
-    if (work) {
-      float c[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) c[r][q] = 0.f;
-      const float* sp = st + par * kAnX * kAnRows;
+    for (int i = gtid; i < NX * 2 * KW * 4; i += gt)
+      stw[i] = __ldg(reinterpret_cast<const float4*>(tw_k) + (size_t)x0 * 2 * KW * 4 + i);
+    asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gt) : "memory");
+    const float* sp = st + par * kAnX * kAnRows + 2 * (lane & 1);
+    const float4* wp = stw + gw * 4;
 #pragma unroll 4
-      for (int x = 0; x < NX; ++x) {
-        const float4 h = *reinterpret_cast<const float4*>(sp + x * kAnRows + ((rg ^ ((x >> 2) & 7)) * 4));
-        const float4 w = stw[x * 2 * KG + kgp];
-        const float hv[4] = {h.x, h.y, h.z, h.w};
+    for (int x = 0; x < NX; ++x) {
+      const float2 h = *reinterpret_cast<const float2*>(sp + x * kAnRows + (((lane >> 1) ^ ((x >> 2) & 7)) * 4));
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          c[r][0] = fmaf(hv[r], w.x, c[r][0]);
-          c[r][1] = fmaf(hv[r], w.y, c[r][1]);
-          c[r][2] = fmaf(hv[r], w.z, c[r][2]);
-          c[r][3] = fmaf(hv[r], w.w, c[r][3]);
+      for (int q = 0; q < 4; ++q) {
+        const float4 w = wp[x * 2 * KW * 4 + q];
+        const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[0][4 * q + e] = fmaf(h.x, wv[e], acc[0][4 * q + e]);
+          acc[1][4 * q + e] = fmaf(h.y, wv[e], acc[1][4 * q + e]);
         }
       }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] += c[r][q];
     }
   }
-  __syncthreads();
-  // the row transforms, then the block's share of the columns
-  if (work) {
-    const int k0 = 2 * (2 * (kgp - par * KG)) + par, k1 = k0 + 2;
+  // the row transforms [MX][RS], the groups' shares added one after another
+  float2* sA = reinterpret_cast<float2*>(sm_an);
+  const int RS = rows + 1;
+  for (int g = 0; g < KS; ++g) {
+    __syncthreads();
+    if (grp == g) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = rg * 4 + r;
-      if (k0 < MX) {
-        const float sc = k0 == 0 ? s0 : s1;
-        sA[row * MX + k0] = make_float2(acc[r][0] * sc, acc[r][1] * sc);
+      for (int q = 0; q < 8; ++q) {
+        const int k = 2 * (8 * (gw - par * KW) + q) + par;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int row = 2 * lane + r;
+          if (k < MX && row < rows) {
+            float2 v = make_float2(acc[r][2 * q], acc[r][2 * q + 1]);
+            if (g > 0) {
+              const float2 o = sA[k * RS + row];
+              v = make_float2(v.x + o.x, v.y + o.y);
+            }
+            if (g == KS - 1) {
+              const float sc = k == 0 ? s0 : s1;
+              v = make_float2(v.x * sc, v.y * sc);
+            }
+            sA[k * RS + row] = v;
+          }
+        }
       }
-      if (k1 < MX) sA[row * MX + k1] = make_float2(acc[r][2] * s1, acc[r][3] * s1);
     }
   }
   __syncthreads();
   for (int i = tid; i < RH * MX; i += nt) {  // fold the rows a half period apart
-    const float2 a = sA[i], b = sA[RH * MX + i];
-    sA[i] = make_float2(a.x + b.x, a.y + b.y);
-    sA[RH * MX + i] = make_float2(a.x - b.x, a.y - b.y);
+    float2* c = sA + (i / RH) * RS + (i % RH);
+    const float2 a = c[0], b = c[RH];
+    c[0] = make_float2(a.x + b.x, a.y + b.y);
+    c[RH] = make_float2(a.x - b.x, a.y - b.y);
   }
   __syncthreads();
+  // the block's share of the columns, JQ k_y of one parity (ky_j has the
+  // parity of j: N - 2 MY is even) per thread
+  constexpr int JQ = KS == 4 ? 2 : 4;
   float2* dst = part + ((size_t)slice * nblk + yb) * MY2 * MX;
-  for (int i = tid; i < MY2 * MX; i += nt) {
-    const int k = i % MX, j = i / MX;  // ky_j has the parity of j (N - 2 MY is even)
-    const float2* a = sA + (j & 1) * RH * MX + k;
-    const float2* w = tw_y + (size_t)j * N + y0;
-    float re = 0.f, im = 0.f;
-    for (int y = 0; y < RH; ++y) {
-      const float2 v = a[y * MX], t = __ldg(&w[y]);
-      re = fmaf(v.x, t.x, fmaf(-v.y, t.y, re));
-      im = fmaf(v.x, t.y, fmaf(v.y, t.x, im));
+  const int MY = MY2 / 2, JG = (MY + JQ - 1) / JQ;
+  for (int i = tid; i < 2 * JG * MX; i += nt) {
+    const int k = i % MX, pj = i / MX, pa = pj & 1, j0 = 2 * JQ * (pj >> 1) + pa;
+    const float2* a = sA + k * RS + pa * RH;
+    const float2* w[JQ];
+    float re[JQ], im[JQ];
+#pragma unroll
+    for (int q = 0; q < JQ; ++q) {
+      w[q] = tw_y + (size_t)min(j0 + 2 * q, MY2 - 1) * N + y0;
+      re[q] = im[q] = 0.f;
     }
-    dst[i] = make_float2(re, im);
+#pragma unroll 8
+    for (int y = 0; y < RH; ++y) {
+      const float2 v = a[y];
+#pragma unroll
+      for (int q = 0; q < JQ; ++q) {
+        const float2 t = __ldg(&w[q][y]);
+        re[q] = fmaf(v.x, t.x, fmaf(-v.y, t.y, re[q]));
+        im[q] = fmaf(v.x, t.y, fmaf(v.y, t.x, im[q]));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < JQ; ++q)
+      if (j0 + 2 * q < MY2) dst[(j0 + 2 * q) * MX + k] = make_float2(re[q], im[q]);
   }
 }
 
@@ -230,19 +256,32 @@ analysis(const float* __restrict__ in, float2* __restrict__ part, const float2* 
 //   fwd: out[b][m][o] = sum_i R[i][o][m] X[b][i][m]
 //   bwd: out[b][m][i] = sum_o conj(R[i][o][m]) X[b][o][m]
 // One block takes 8 modes (32-byte pieces of R) of one map; the output is
-// channel-fastest for the column synthesis.  Bound by reading R (4 C^2 bytes
-// per mode) and by latency.
-__global__ void __launch_bounds__(kThreads)
+// channel-fastest for the column synthesis.  Bound by the latency of reading R
+// (4 C^2 bytes per mode): two halves of the block share the summed channels and
+// keep 16 loads each in flight.
+__global__ void __launch_bounds__(2 * kThreads)
 mix(const float2* __restrict__ part, int nblk, const __half2* __restrict__ R, float2* __restrict__ X,
     float2* __restrict__ out, int C, int CP, int NM, int bwd) {
   __shared__ float2 sX[kMaxWidth * kMixModes];
-  __shared__ float2 sY[kMixModes * kMaxWidth];
+  __shared__ float2 sY[2][kMixModes * kMaxWidth];
   const int b = blockIdx.y, m0 = blockIdx.x * kMixModes;
+  const int half = threadIdx.x / kThreads, c0 = half * (C / 2), c1 = half ? C : C / 2;  // C is even
+  const int i0 = threadIdx.x % kThreads;
+  const size_t rs = bwd ? (size_t)NM : (size_t)C * NM, ro = bwd ? (size_t)C * NM : (size_t)NM;
+  // the first 16 matrix values of the first output, before the sums
+  __half2 rv[16];
+  {
+    const int o = i0 / kMixModes, m = m0 + i0 % kMixModes;
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      rv[q] = (o < C && m < NM && c0 + q < c1) ? R[(size_t)o * ro + (size_t)(c0 + q) * rs + m] : __half2();
+  }
   for (int i = threadIdx.x; i < C * kMixModes; i += blockDim.x) {
     const int c = i / kMixModes, m = m0 + i % kMixModes;
     float re = 0.f, im = 0.f;
     if (m < NM) {
       const float2* src = part + ((size_t)(b * C + c) * nblk) * NM + m;
+#pragma unroll 8
       for (int q = 0; q < nblk; ++q) {
         const float2 v = src[(size_t)q * NM];
         re += v.x;
@@ -253,34 +292,36 @@ mix(const float2* __restrict__ part, int nblk, const __half2* __restrict__ R, fl
     sX[i] = make_float2(re, im);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < CP * kMixModes; i += blockDim.x) {
+  const float sg = bwd ? -1.f : 1.f;  // conj(R) in the adjoint
+  for (int i = i0; i < CP * kMixModes; i += kThreads) {
     const int o = i / kMixModes, ml = i % kMixModes, m = m0 + ml;
     float re = 0.f, im = 0.f;
     if (o < C && m < NM) {
-      if (!bwd) {
-#pragma unroll 8
-        for (int c = 0; c < C; ++c) {
-          const float2 r = __half22float2(R[((size_t)c * C + o) * NM + m]);
-          const float2 x = sX[c * kMixModes + ml];
-          re = fmaf(r.x, x.x, fmaf(-r.y, x.y, re));
-          im = fmaf(r.x, x.y, fmaf(r.y, x.x, im));
+      for (int cb = c0; cb < c1; cb += 16) {
+        if (i != i0 || cb != c0) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            rv[q] = cb + q < c1 ? R[(size_t)o * ro + (size_t)(cb + q) * rs + m] : __half2();
         }
-      } else {
-#pragma unroll 8
-        for (int c = 0; c < C; ++c) {
-          const float2 r = __half22float2(R[((size_t)o * C + c) * NM + m]);
-          const float2 x = sX[c * kMixModes + ml];
-          re = fmaf(r.x, x.x, fmaf(r.y, x.y, re));
-          im = fmaf(r.x, x.y, fmaf(-r.y, x.x, im));
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          if (cb + q < c1) {
+            const float2 r = __half22float2(rv[q]);
+            const float2 x = sX[(cb + q) * kMixModes + ml];
+            const float ry = sg * r.y;
+            re = fmaf(r.x, x.x, fmaf(-ry, x.y, re));
+            im = fmaf(r.x, x.y, fmaf(ry, x.x, im));
+          }
         }
       }
     }
-    sY[ml * CP + o] = make_float2(re, im);
+    sY[half][ml * CP + o] = make_float2(re, im);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < CP * kMixModes; i += blockDim.x) {
     const int m = m0 + i / CP;
-    if (m < NM) out[((size_t)b * NM + m) * CP + i % CP] = sY[i];
+    const float2 u = sY[0][i], v = sY[1][i];
+    if (m < NM) out[((size_t)b * NM + m) * CP + i % CP] = make_float2(u.x + v.x, u.y + v.y);
   }
 }
 
@@ -299,6 +340,7 @@ mix_bwd_r(const float2* __restrict__ gY, const float2* __restrict__ X, float* __
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int o = 0; o < 4; ++o) re[i][o] = im[i][o] = 0.f;
+#pragma unroll 4
   for (int b = 0; b < B; ++b) {
     float2 x[4], y[4];
 #pragma unroll
@@ -322,9 +364,8 @@ mix_bwd_r(const float2* __restrict__ gY, const float2* __restrict__ X, float* __
 #pragma unroll
     for (int o = 0; o < 4; ++o)
       if (i0 + i < C && o0 + o < C) {
-        float* d = gR + 2 * (((size_t)(i0 + i) * C + o0 + o) * NM + m);
-        d[0] = re[i][o];
-        d[1] = im[i][o];
+        // 8-byte aligned: widths are even, so every block of the vector is
+        reinterpret_cast<float2*>(gR)[((size_t)(i0 + i) * C + o0 + o) * NM + m] = make_float2(re[i][o], im[i][o]);
       }
   if (m == 0 && i0 == 0)
 #pragma unroll
@@ -382,6 +423,20 @@ synth_cols(const float2* __restrict__ Y, float* __restrict__ S, const float2* __
   }
 }
 
+// packed FP32 pairs (low word first)
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
+}
+__device__ __forceinline__ unsigned long long dup2(float x) { return pack2(x, x); }
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  return make_float2(__uint_as_float((unsigned)v), __uint_as_float((unsigned)(v >> 32)));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
 // Geometry of the row synthesis: OG groups of 8 output channels x PG groups
 // of 2 pixel pairs (x, x + N/2); XT pairs of one row, RT rows per step.
 __host__ __device__ constexpr int synth_pg(int OG) { return 256 / OG < 64 ? 256 / OG : 64; }
@@ -396,9 +451,9 @@ inline SynthGeom synth_geom(int OG, int B, int C, int N, int MX) {
   g.RT = pairs / g.XT < 4 ? pairs / g.XT : 4;
   g.nxt = (N / 2) / g.XT;
   g.units = B * (N / g.RT) * g.nxt;
-  const int CP = 8 * OG, MXE = MX;
-  g.smem = sizeof(float) * ((size_t)C * 2 * g.RT * g.XT + (size_t)2 * MXE * g.XT + (size_t)g.RT * MXE * 2 * CP +
-                            (size_t)C * CP);
+  const int CP = 8 * OG;
+  g.smem = sizeof(float) * ((size_t)C * CP + (size_t)2 * MX * g.XT +
+                            2 * ((size_t)g.RT * MX * 2 * CP + (size_t)C * 2 * g.RT * g.XT));
   return g;
 }
 
@@ -424,24 +479,33 @@ struct SynthArgs {
 // layer projected onto y.  Adjoint (ADJ): g = W^T g_z + (row synthesis of S),
 // times act' of the layer below; for layer 0 the sums of the lift's
 // gradient instead.  A thread holds 8 channels x 4 pixels (two neighbours and
-// the two N/2 further on): 32 FMA per four 8- or 16-byte shared loads for
-// W, and per six for two pixels' worth of modes.  The tables (W, the row
-// twiddles of the block's pixels) stay in shared memory while the block walks
-// its rows.  48 C^2 / 32 FMA per pixel at 16 modes (FP32-issue bound) against
-// 8 to 12 C bytes.
-template <int OG, bool ADJ>
+// the two N/2 further on); a warp has one channel group, so its weights and
+// modes are broadcast loads and its pixel loads and stores are whole lines.
+// The channels go in pairs through the packed FP32 FMA: the pairs are the
+// registers a 16-byte load of the weights gives, only the pixel value is
+// duplicated, and a step of 32 FMA issues 16 FMA, 4 moves and 4 loads.  The
+// tables (W, the row twiddles of the block's pixels) stay in shared memory
+// while the block walks its rows.  1536 FMA per pixel at 32 channels and 16
+// modes (FP32 bound, 21 us for eight 256^2 maps) against 8 to 12 C bytes: 69
+// us measured, about a fifth of it the erf; with the channel groups across the
+// lanes of a warp, scalar FMA and one stage it took 93 us.
+template <int OG, bool ADJ, bool FULL>
 __global__ void __launch_bounds__(OG * synth_pg(OG))
 synth(SynthArgs a) {
   constexpr int PG = synth_pg(OG), NT = OG * PG, CP = 8 * OG;
   extern __shared__ __align__(16) float sm_sy[];
-  const int C = a.C, N = a.N, MX = a.MX, XT = a.XT, RT = a.RT, PX = RT * XT;
+  // FULL: the channels fill their groups and a step is part of one row, so
+  // the strides and loop bounds are known
+  const int N = a.N, MX = a.MX;
+  const int C = FULL ? CP : a.C, XT = FULL ? 2 * PG : a.XT, RT = FULL ? 1 : a.RT, PX = RT * XT;
   const size_t P = (size_t)N * N;
   float* sW = sm_sy;                                 // [C][CP]: input channel, output channel
-  float* sS = sW + (size_t)C * CP;                   // [RT][MX][2][CP]
-  float* sTc = sS + (size_t)RT * MX * 2 * CP;        // [MX][XT] cos
+  float* sTc = sW + (size_t)C * CP;                  // [MX][XT] cos
   float* sTs = sTc + (size_t)MX * XT;                // [MX][XT] -sin
-  float* sH = sTs + (size_t)MX * XT;                 // [C][2][RT][XT]
-  const int tid = threadIdx.x, og = tid % OG, pg = tid / OG;
+  float* sStage = sTs + (size_t)MX * XT;             // two stages of:
+  const size_t szS = (size_t)RT * MX * 2 * CP;       // S  [RT][MX][2][CP]
+  const size_t szStage = szS + (size_t)C * 2 * PX;   // h  [C][2][RT][XT]
+  const int tid = threadIdx.x, og = (tid >> 5) % OG, pg = (tid & 31) + 32 * ((tid >> 5) / OG);
   const int xt = blockIdx.x % a.nxt;                 // gridDim.x is a multiple of nxt
   for (int i = tid; i < C * CP; i += NT) {
     const int ci = i / CP, co = i % CP;
@@ -453,8 +517,8 @@ synth(SynthArgs a) {
     sTs[i] = t.y;
   }
   const int pr = 2 * pg;                             // this thread's first pair
-  const bool on = pr < PX;
-  const int rl = on ? pr / XT : 0, xl = on ? pr % XT : 0;
+  const bool on = FULL || pr < PX;
+  const int rl = FULL || !on ? 0 : pr / XT, xl = FULL ? pr : (on ? pr % XT : 0);
   float bias[8], lsum[8][3];
 #pragma unroll
   for (int o = 0; o < 8; ++o) {
@@ -462,25 +526,39 @@ synth(SynthArgs a) {
     lsum[o][0] = lsum[o][1] = lsum[o][2] = 0.f;
   }
   const int nyb = N / RT;
-  for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+  const int lxq = 31 - __clz(XT / 4), lrt = 31 - __clz(RT);  // powers of two
+  auto stage = [&](int u, int st) {
+    if (u < a.units) {
+      const int t = u / a.nxt, y0 = (t % nyb) * RT, b = t / nyb;
+      float* dS = sStage + st * szStage;
+      float* dH = dS + szS;
+      for (int i = tid; i < C << (lxq + lrt + 1); i += NT) {
+        const int xq = i & ((1 << lxq) - 1), r = (i >> lxq) & (RT - 1), h = (i >> (lxq + lrt)) & 1,
+                  c = i >> (lxq + lrt + 1);
+        wf::cp_async16(dH + 4 * (size_t)i,
+                       a.in + ((size_t)b * C + c) * P + (size_t)(y0 + r) * N + h * (N / 2) + xt * XT + 4 * xq);
+      }
+      const float* gs = a.S + ((size_t)b * N + y0) * MX * 2 * CP;
+      for (int i = tid; i < (int)(szS / 4); i += NT) wf::cp_async16(dS + 4 * i, gs + 4 * i);
+    }
+    wf::cp_async_commit();
+  };
+  stage(blockIdx.x, 0);
+  int cur = 0;
+  for (int u = blockIdx.x; u < a.units; u += gridDim.x, cur ^= 1) {
     const int t = u / a.nxt, yb = t % nyb, b = t / nyb;
     const int y0 = yb * RT;
-    __syncthreads();  // the tables are written; the last step's tiles are read
-    const int XQ = XT / 4;
-    for (int i = tid; i < C * 2 * RT * XQ; i += NT) {
-      const int xq = i % XQ, r = (i / XQ) % RT, h = (i / (XQ * RT)) & 1, c = i / (XQ * RT * 2);
-      wf::cp_async16(sH + 4 * (size_t)i,
-                     a.in + ((size_t)b * C + c) * P + (size_t)(y0 + r) * N + h * (N / 2) + xt * XT + 4 * xq);
-    }
-    const float* gs = a.S + ((size_t)b * N + y0) * MX * 2 * CP;
-    for (int i = tid; i < RT * MX * 2 * CP / 4; i += NT) wf::cp_async16(sS + 4 * i, gs + 4 * i);
-    wf::cp_async_commit();
-    wf::cp_async_wait<0>();
+    // the stage filled next was read in the last step (barrier at its end)
+    stage(u + gridDim.x, cur ^ 1);
+    wf::cp_async_wait<1>();
     __syncthreads();
-    float z[8][4];  // [channel][x, x + 1, x + N/2, x + N/2 + 1]
+    const float* sS = sStage + cur * szStage;
+    float* sH = sStage + cur * szStage + szS;
+    // [channel pair][x, x + 1, x + N/2, x + N/2 + 1]
+    unsigned long long zz[4][4];
 #pragma unroll
-    for (int o = 0; o < 8; ++o) z[o][0] = z[o][1] = z[o][2] = z[o][3] = 0.f;
-    // modes: even k into z[.][0..1], odd k into z[.][2..3]
+    for (int o = 0; o < 4; ++o) zz[o][0] = zz[o][1] = zz[o][2] = zz[o][3] = 0ull;
+    // modes: even k into [.][0..1], odd k into [.][2..3]
     const float* s = sS + (size_t)rl * MX * 2 * CP + og * 8;
 #pragma unroll 2
     for (int k = 0; k < MX; k += 2) {
@@ -489,43 +567,55 @@ synth(SynthArgs a) {
         if (k + h < MX) {
           const float2 c = *reinterpret_cast<const float2*>(sTc + (k + h) * XT + xl);
           const float2 sn = *reinterpret_cast<const float2*>(sTs + (k + h) * XT + xl);
-          const float4* sr = reinterpret_cast<const float4*>(s + (k + h) * 2 * CP);
-          const float4* si = reinterpret_cast<const float4*>(s + (k + h) * 2 * CP + CP);
-          const float4 r0 = sr[0], r1 = sr[1], i0 = si[0], i1 = si[1];
-          const float re[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-          const float im[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+          const ulonglong2* sr = reinterpret_cast<const ulonglong2*>(s + (k + h) * 2 * CP);
+          const ulonglong2* si = reinterpret_cast<const ulonglong2*>(s + (k + h) * 2 * CP + CP);
+          const ulonglong2 r0 = sr[0], r1 = sr[1], i0 = si[0], i1 = si[1];
+          const unsigned long long re[4] = {r0.x, r0.y, r1.x, r1.y}, im[4] = {i0.x, i0.y, i1.x, i1.y};
+          const unsigned long long cx = dup2(c.x), cy = dup2(c.y), sx = dup2(sn.x), sy = dup2(sn.y);
 #pragma unroll
-          for (int o = 0; o < 8; ++o) {
-            z[o][2 * h] = fmaf(re[o], c.x, fmaf(im[o], sn.x, z[o][2 * h]));
-            z[o][2 * h + 1] = fmaf(re[o], c.y, fmaf(im[o], sn.y, z[o][2 * h + 1]));
+          for (int o = 0; o < 4; ++o) {
+            zz[o][2 * h] = fma2(re[o], cx, fma2(im[o], sx, zz[o][2 * h]));
+            zz[o][2 * h + 1] = fma2(re[o], cy, fma2(im[o], sy, zz[o][2 * h + 1]));
           }
         }
       }
     }
 #pragma unroll
-    for (int o = 0; o < 8; ++o) {
-      const float e0 = z[o][0], e1 = z[o][1], d0 = z[o][2], d1 = z[o][3];
-      z[o][0] = e0 + d0 + bias[o];
-      z[o][1] = e1 + d1 + bias[o];
-      z[o][2] = e0 - d0 + bias[o];
-      z[o][3] = e1 - d1 + bias[o];
+    for (int o = 0; o < 4; ++o) {
+      float2 e0 = unpack2(zz[o][0]), e1 = unpack2(zz[o][1]), d0 = unpack2(zz[o][2]), d1 = unpack2(zz[o][3]);
+      const float b0 = bias[2 * o], b1 = bias[2 * o + 1];
+      zz[o][0] = pack2(e0.x + d0.x + b0, e0.y + d0.y + b1);
+      zz[o][1] = pack2(e1.x + d1.x + b0, e1.y + d1.y + b1);
+      zz[o][2] = pack2(e0.x - d0.x + b0, e0.y - d0.y + b1);
+      zz[o][3] = pack2(e1.x - d1.x + b0, e1.y - d1.y + b1);
     }
     const float* hp = sH + (on ? pr : 0);
 #pragma unroll 4
     for (int c = 0; c < C; ++c) {
       const float2 h0 = *reinterpret_cast<const float2*>(hp + (size_t)c * 2 * PX);
       const float2 h1 = *reinterpret_cast<const float2*>(hp + (size_t)c * 2 * PX + PX);
-      const float4* wp = reinterpret_cast<const float4*>(sW + c * CP + og * 8);
-      const float4 w0 = wp[0], w1 = wp[1];
-      const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+      const ulonglong2* wp = reinterpret_cast<const ulonglong2*>(sW + c * CP + og * 8);
+      const ulonglong2 w0 = wp[0], w1 = wp[1];
+      const unsigned long long w[4] = {w0.x, w0.y, w1.x, w1.y};
+      const unsigned long long a0 = dup2(h0.x), a1 = dup2(h0.y), b0 = dup2(h1.x), b1 = dup2(h1.y);
 #pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        z[o][0] = fmaf(w[o], h0.x, z[o][0]);
-        z[o][1] = fmaf(w[o], h0.y, z[o][1]);
-        z[o][2] = fmaf(w[o], h1.x, z[o][2]);
-        z[o][3] = fmaf(w[o], h1.y, z[o][3]);
+      for (int o = 0; o < 4; ++o) {
+        zz[o][0] = fma2(w[o], a0, zz[o][0]);
+        zz[o][1] = fma2(w[o], a1, zz[o][1]);
+        zz[o][2] = fma2(w[o], b0, zz[o][2]);
+        zz[o][3] = fma2(w[o], b1, zz[o][3]);
       }
     }
+    __syncthreads();  // the tile is read: the next step's copies may overwrite it
+    float z[8][4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 v = unpack2(zz[o][e]);
+        z[2 * o][e] = v.x;
+        z[2 * o + 1][e] = v.y;
+      }
     const size_t px = (size_t)(y0 + rl) * N + xt * XT + xl;  // and px + N/2
     if constexpr (!ADJ) {
       float yv[4] = {0.f, 0.f, 0.f, 0.f};
@@ -544,11 +634,11 @@ synth(SynthArgs a) {
               float g[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                const float zz = z[o][e];
-                const float Phi = 0.5f * (1.f + erff(zz * 0.70710678118654752f));
+                const float v = z[o][e];
+                const float Phi = 0.5f * (1.f + erff(v * 0.70710678118654752f));
                 // d/dz [z Phi(z)] = Phi(z) + z phi(z)
-                if (a.dact) g[e] = fmaf(zz, 0.3989422804014327f * __expf(-0.5f * zz * zz), Phi);
-                z[o][e] = zz * Phi;
+                if (a.dact) g[e] = fmaf(v, 0.3989422804014327f * __expf(-0.5f * v * v), Phi);
+                z[o][e] = v * Phi;
               }
               if (a.dact) {
                 *reinterpret_cast<float2*>(a.dact + idx) = make_float2(g[0], g[1]);
@@ -562,12 +652,18 @@ synth(SynthArgs a) {
           }
         }
       }
-      if (a.Q) {  // sum the channel groups (neighbouring lanes)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-          for (int sft = 1; sft < OG; sft <<= 1) yv[e] += __shfl_xor_sync(0xffffffffu, yv[e], sft);
+      if (a.Q) {  // sum the channel groups (the warps of these pixels) in order
+        if (on) *reinterpret_cast<float4*>(sH + (og * PG + pg) * 4) = make_float4(yv[0], yv[1], yv[2], yv[3]);
+        __syncthreads();
         if (on && og == 0) {
+#pragma unroll
+          for (int g = 1; g < OG; ++g) {
+            const float4 v = *reinterpret_cast<const float4*>(sH + (g * PG + pg) * 4);
+            yv[0] += v.x;
+            yv[1] += v.y;
+            yv[2] += v.z;
+            yv[3] += v.w;
+          }
           float* yo = a.y + (size_t)b * P + px;
           const float q = a.q[0];
           yo[0] = yv[0] + q;
@@ -575,6 +671,7 @@ synth(SynthArgs a) {
           yo[N / 2] = yv[2] + q;
           yo[N / 2 + 1] = yv[3] + q;
         }
+        __syncthreads();
       }
     } else if (on) {
       float xv[2][4];
@@ -618,6 +715,7 @@ synth(SynthArgs a) {
   }
   if constexpr (ADJ) {
     if (a.x) {  // the block's sums over its pixels: a fixed tree
+      wf::cp_async_wait<0>();
       __syncthreads();
 #pragma unroll
       for (int o = 0; o < 8; ++o)
@@ -625,20 +723,19 @@ synth(SynthArgs a) {
         for (int i = 0; i < 3; ++i) {
           float v = lsum[o][i];
 #pragma unroll
-          for (int sft = OG; sft < 32; sft <<= 1) v += __shfl_xor_sync(0xffffffffu, v, sft);
+          for (int sft = 16; sft > 0; sft >>= 1) v += __shfl_xor_sync(0xffffffffu, v, sft);
           lsum[o][i] = v;
         }
-      float* red = sm_sy;  // [warps][CP][3] over the tables, which are done with
-      const int warp = tid >> 5, lane = tid & 31;
-      if (lane < OG)
+      float* red = sm_sy;  // [warps][8][3] over the tables, which are done with
+      if ((tid & 31) == 0)
 #pragma unroll
         for (int o = 0; o < 8; ++o)
 #pragma unroll
-          for (int i = 0; i < 3; ++i) red[(warp * CP + lane * 8 + o) * 3 + i] = lsum[o][i];
+          for (int i = 0; i < 3; ++i) red[((tid >> 5) * 8 + o) * 3 + i] = lsum[o][i];
       __syncthreads();
       for (int i = tid; i < CP * 3; i += NT) {
-        float v = 0.f;
-        for (int w = 0; w < NT / 32; ++w) v += red[w * CP * 3 + i];
+        float v = 0.f;  // channel i / 3: the warps of group (i / 3) / 8
+        for (int w = i / 24; w < NT / 32; w += OG) v += red[w * 24 + i % 24];
         a.lpart[(size_t)blockIdx.x * CP * 3 + i] = v;
       }
     }
@@ -658,9 +755,7 @@ weight_grad(const float* __restrict__ gz, const float* __restrict__ in, float* _
             int P) {
   constexpr int G = CP / 4, GT = G * G;
   constexpr int SPLITS = 256 / GT < 32 ? 256 / GT : 32;  // at most one per 16-byte piece of a tile
-  extern __shared__ __align__(16) float sm_wg[];
-  float* sg = sm_wg;
-  float* sh = sm_wg + CP * kWgStride;
+  extern __shared__ __align__(16) float sm_wg[];  // two stages of a g and an h tile
   const int tid = threadIdx.x, grp = tid % GT, sp = tid / GT;
   const int og = grp / G, ig = grp % G;
   const bool on = sp < SPLITS;
@@ -671,20 +766,31 @@ weight_grad(const float* __restrict__ gz, const float* __restrict__ in, float* _
 #pragma unroll
     for (int i = 0; i < 4; ++i) tot[o][i] = 0.f;
   for (int c = C; c < CP; ++c)
-    for (int x = tid; x < kWgPx; x += blockDim.x) sg[c * kWgStride + x] = sh[c * kWgStride + x] = 0.f;
-  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int b = t / tiles_b, p0 = (t - b * tiles_b) * kWgPx;
-    __syncthreads();
-    for (int i = tid; i < C * (kWgPx / 4); i += blockDim.x) {
-      const int c = i / (kWgPx / 4), xq = i % (kWgPx / 4);
-      const size_t o = ((size_t)b * C + c) * P + p0 + 4 * xq;
-      wf::cp_async16(sg + c * kWgStride + 4 * xq, gz + o);
-      wf::cp_async16(sh + c * kWgStride + 4 * xq, in + o);
+    for (int x = tid; x < kWgPx; x += blockDim.x)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sm_wg[(q * CP + c) * kWgStride + x] = 0.f;
+  auto stage = [&](int t, int st) {
+    if (t < tiles) {
+      const int b = t / tiles_b, p0 = (t - b * tiles_b) * kWgPx;
+      float* d = sm_wg + 2 * st * CP * kWgStride;
+      for (int i = tid; i < C * (kWgPx / 4); i += 256) {
+        const int c = i / (kWgPx / 4), xq = i % (kWgPx / 4);
+        const size_t o = ((size_t)b * C + c) * P + p0 + 4 * xq;
+        wf::cp_async16(d + c * kWgStride + 4 * xq, gz + o);
+        wf::cp_async16(d + (CP + c) * kWgStride + 4 * xq, in + o);
+      }
     }
     wf::cp_async_commit();
-    wf::cp_async_wait<0>();
+  };
+  stage(blockIdx.x, 0);
+  int st = 0;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x, st ^= 1) {
+    stage(t + gridDim.x, st ^ 1);
+    wf::cp_async_wait<1>();
     __syncthreads();
     if (on) {
+      const float* sg = sm_wg + 2 * st * CP * kWgStride;
+      const float* sh = sg + CP * kWgStride;
       float acc[4][4];
 #pragma unroll
       for (int o = 0; o < 4; ++o)
@@ -707,7 +813,9 @@ weight_grad(const float* __restrict__ gz, const float* __restrict__ in, float* _
 #pragma unroll
         for (int i = 0; i < 4; ++i) tot[o][i] += acc[o][i];
     }
+    __syncthreads();  // the stage is read before it is filled again
   }
+  wf::cp_async_wait<0>();
   __syncthreads();
   float* red = sm_wg;  // [SPLITS][CP][CP]: at most 2 CP kWgStride floats (checked below)
   static_assert((CP >= 32 ? SPLITS : 8) * CP * CP <= 2 * CP * kWgStride, "reduction fits the tiles");
@@ -737,25 +845,26 @@ weight_grad(const float* __restrict__ gz, const float* __restrict__ in, float* _
   }
 }
 
-// out[i * stride_out ...]: sums of nblk partial vectors of n values, one warp
-// lane per value and eight partial sums per value (fixed order).  map = 0:
+// Sums of nblk partial vectors of n values, a lane per value and 32 partial
+// sums per value (fixed order).  map = 0:
 // out[k]; map = 1: the lift's (o, {x0, x1, 1}) triples into gP [C][2] and gp
 // [C]; map = 2: C values into out, then one into out2.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 sum_partials(const float* __restrict__ partial, int nblk, int n, float* __restrict__ out, float* __restrict__ out2,
              int map, int C) {
-  __shared__ float red[8][32];
+  __shared__ float red[32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int k = blockIdx.x * 32 + lane;
   float s = 0.f;
   if (k < n)
-    for (int b = w; b < nblk; b += 8) s += partial[(size_t)b * n + k];
+#pragma unroll 4
+    for (int b = w; b < nblk; b += 32) s += partial[(size_t)b * n + k];
   red[w][lane] = s;
   __syncthreads();
   if (w != 0 || k >= n) return;
   s = 0.f;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) s += red[i][lane];
+  for (int i = 0; i < 32; ++i) s += red[i][lane];
   if (map == 0) {
     out[k] = s;
   } else if (map == 1) {
@@ -785,17 +894,24 @@ proj_bwd(const float* __restrict__ y, const float* __restrict__ t, const float* 
   float acc[CP], sg = 0.f;
 #pragma unroll
   for (int o = 0; o < CP; ++o) acc[o] = 0.f;
-  const size_t total = (size_t)B * P;
+  const size_t total = (size_t)B * P / 4;  // four pixels a step (P is a multiple of 256)
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(g / P), p = (int)(g % P);
-    const float gy = 2.f * (y[g] - t[g]) * inv[b];
-    sg += gy;
+    const size_t e = 4 * g;
+    const int b = (int)(e / P);
+    const float iv = inv[b];
+    // t is the caller's: no alignment beyond a float's
+    const float g0 = 2.f * (y[e] - t[e]) * iv, g1 = 2.f * (y[e + 1] - t[e + 1]) * iv,
+                g2 = 2.f * (y[e + 2] - t[e + 2]) * iv, g3 = 2.f * (y[e + 3] - t[e + 3]) * iv;
+    sg += (g0 + g1) + (g2 + g3);
+    const size_t base = (size_t)b * C * P + (e - (size_t)b * P);
 #pragma unroll
     for (int o = 0; o < CP; ++o)
       if (o < C) {
-        const size_t idx = ((size_t)b * C + o) * P + p;
-        acc[o] = fmaf(gy, hL[idx], acc[o]);
-        gz[idx] = sQ[o] * gy;
+        const size_t idx = base + (size_t)o * P;
+        const float4 h = *reinterpret_cast<const float4*>(hL + idx);
+        acc[o] += fmaf(g0, h.x, g1 * h.y) + fmaf(g2, h.z, g3 * h.w);
+        const float q = sQ[o];
+        *reinterpret_cast<float4*>(gz + idx) = make_float4(q * g0, q * g1, q * g2, q * g3);
       }
   }
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -845,14 +961,15 @@ __global__ void loss_partial(const float* __restrict__ y, const float* __restric
   }
 }
 
-// loss = mean_b num_b / den_b; inv[b] = 1 / (B den_b).  One warp: lane k sums
-// block k of every map (nblk = 32), then a fixed tree.
+// loss = mean_b num_b / den_b; inv[b] = 1 / (B den_b).  A warp per map: lane k
+// sums block k (nblk = 32), then a fixed tree.
 __global__ void loss_fin(const double* __restrict__ part, int nblk, int B, double* __restrict__ loss,
                          float* __restrict__ inv) {
-  double L = 0.0;
-  for (int b = 0; b < B; ++b) {
+  __shared__ double rel[64];  // B <= 64
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < B; b += blockDim.x >> 5) {
     double n = 0.0, d = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += 32) {
+    for (int k = lane; k < nblk; k += 32) {
       n += part[((size_t)b * nblk + k) * 2];
       d += part[((size_t)b * nblk + k) * 2 + 1];
     }
@@ -861,10 +978,17 @@ __global__ void loss_fin(const double* __restrict__ part, int nblk, int B, doubl
       d += __shfl_xor_sync(0xffffffffu, d, s);
     }
     d = d > 0.0 ? d : 1.0;
-    L += n / d;
-    if (threadIdx.x == 0) inv[b] = (float)(1.0 / (B * d));
+    if (lane == 0) {
+      rel[b] = n / d;
+      inv[b] = (float)(1.0 / (B * d));
+    }
   }
-  if (threadIdx.x == 0) *loss = L / B;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double L = 0.0;
+    for (int b = 0; b < B; ++b) L += rel[b];
+    *loss = L / B;
+  }
 }
 
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -956,7 +1080,7 @@ struct wf_fno_s {
   float* S = nullptr;         // [B][N][MX][2][CP]
   float2 *tw_x = nullptr, *tw_y = nullptr, *tw_k = nullptr;
   float* wpart = nullptr;
-  int OG = 1, KG = 1, sms = 1, synth_per_sm = 1, adj_per_sm = 1;
+  int OG = 1, KW = 1, sms = 1, synth_per_sm = 1, adj_per_sm = 1;
   double* lpart = nullptr;
   double* dloss = nullptr;
   float* inv = nullptr;
@@ -980,23 +1104,35 @@ size_t P_(const wf_fno_s* F) { return (size_t)F->n * F->n; }
 size_t act_(const wf_fno_s* F) { return (size_t)F->batch * F->lay.width * P_(F); }
 size_t modes_(const wf_fno_s* F) { return (size_t)2 * F->lay.my * F->lay.mx; }
 int an_blocks(int n) { return (n / 2) / (std::min(kAnRows, n) / 2); }
-int an_threads(int n, int KG) { return (std::min(kAnRows, n) / 4 * 2 * KG + 31) / 32 * 32; }
-size_t an_smem(int KG, int MX) {
-  return std::max(sizeof(float) * 2 * kAnX * kAnRows + sizeof(float4) * kAnX * 2 * KG, sizeof(float2) * kAnRows * MX);
+size_t an_smem(int KS, int KW, int MX) {
+  return sizeof(float) * std::max((size_t)KS * (2 * kAnX * kAnRows + kAnX * 2 * KW * 16), (size_t)2 * (kAnRows + 1) * MX);
 }
 size_t cols_smem(int MY2, int CP) { return sizeof(float2) * MY2 * (kColY + CP); }
 
-// pixels or gradients [B][C][N][N] -> partial sums of the retained modes in Xp
+// pixels or gradients [B][C][N][N] -> partial sums of the retained modes in Xp.
+// Few blocks: four groups of warps each, from N = 256 on (every group then has
+// its own 32 pixels of a half row): 26 us against 44 us for one 512^2 map of
+// 32 channels (256 blocks).  From four blocks per SM on, one group, whose
+// smaller stage lets more blocks share an SM: 39 us against 60 us for eight
+// 256^2 maps (1024 blocks).
+template <int KW>
+void launch_analysis_kw(wf_fno_s* F, const float* in, int B, float s0, float s1) {
+  const int C = F->lay.width, N = F->n, MX = F->lay.mx, MY2 = 2 * F->lay.my;
+  const int grid = B * C * an_blocks(N);
+  if (N >= 256 && grid < 4 * F->sms)
+    analysis<4, KW><<<grid, 256 * KW, an_smem(4, KW, MX), F->stream>>>(in, F->Xp, F->tw_k, F->tw_y, N, MX, MY2, s0, s1);
+  else
+    analysis<1, KW><<<grid, 64 * KW, an_smem(1, KW, MX), F->stream>>>(in, F->Xp, F->tw_k, F->tw_y, N, MX, MY2, s0, s1);
+}
 void launch_analysis(wf_fno_s* F, const float* in, int B, float s0, float s1) {
-  const int C = F->lay.width, N = F->n, MX = F->lay.mx;
-  analysis<<<B * C * an_blocks(N), an_threads(N, F->KG), an_smem(F->KG, MX), F->stream>>>(
-      in, F->Xp, F->tw_k, F->tw_y, N, MX, 2 * F->lay.my, F->KG, s0, s1);
+  if (F->KW == 1) launch_analysis_kw<1>(F, in, B, s0, s1);
+  else launch_analysis_kw<2>(F, in, B, s0, s1);
 }
 
 void launch_mix(wf_fno_s* F, int l, float2* X, int B, int bwd) {
   const int C = F->lay.width, NM = (int)modes_(F);
   const __half2* R = reinterpret_cast<const __half2*>(F->half + F->lay.oR[l]);
-  mix<<<dim3((NM + kMixModes - 1) / kMixModes, B), kThreads, 0, F->stream>>>(F->Xp, an_blocks(F->n), R, X, F->Y, C,
+  mix<<<dim3((NM + kMixModes - 1) / kMixModes, B), 2 * kThreads, 0, F->stream>>>(F->Xp, an_blocks(F->n), R, X, F->Y, C,
                                                                              8 * F->OG, NM, bwd);
 }
 
@@ -1014,6 +1150,13 @@ int synth_grid(const wf_fno_s* F, const SynthGeom& g) {
   return std::max(g.nxt, n / g.nxt * g.nxt);
 }
 
+template <int OG, bool ADJ>
+void launch_synth_og(wf_fno_s* F, const SynthArgs& a, const SynthGeom& g, int grid) {
+  constexpr int nt = OG * synth_pg(OG);
+  if (a.C == 8 * OG && g.RT == 1 && g.XT == 2 * synth_pg(OG)) synth<OG, ADJ, true><<<grid, nt, g.smem, F->stream>>>(a);
+  else synth<OG, ADJ, false><<<grid, nt, g.smem, F->stream>>>(a);
+}
+
 template <bool ADJ>
 int launch_synth(wf_fno_s* F, SynthArgs a, int B) {
   const SynthGeom g = synth_geom(F->OG, B, F->lay.width, F->n, F->lay.mx);
@@ -1029,24 +1172,30 @@ int launch_synth(wf_fno_s* F, SynthArgs a, int B) {
   a.tw_x = F->tw_x;
   const int grid = synth_grid<ADJ>(F, g);
   switch (F->OG) {
-    case 1: synth<1, ADJ><<<grid, 1 * synth_pg(1), g.smem, F->stream>>>(a); break;
-    case 2: synth<2, ADJ><<<grid, 2 * synth_pg(2), g.smem, F->stream>>>(a); break;
-    case 4: synth<4, ADJ><<<grid, 4 * synth_pg(4), g.smem, F->stream>>>(a); break;
-    default: synth<8, ADJ><<<grid, 8 * synth_pg(8), g.smem, F->stream>>>(a); break;
+    case 1: launch_synth_og<1, ADJ>(F, a, g, grid); break;
+    case 2: launch_synth_og<2, ADJ>(F, a, g, grid); break;
+    case 4: launch_synth_og<4, ADJ>(F, a, g, grid); break;
+    default: launch_synth_og<8, ADJ>(F, a, g, grid); break;
   }
   return grid;
 }
 
 template <int OG, bool ADJ>
 cudaError_t prepare_synth(size_t smem, int* per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(synth<OG, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int n0 = 0, n1 = 0;
+  cudaError_t e = cudaFuncSetAttribute(synth<OG, ADJ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, synth<OG, ADJ>, OG * synth_pg(OG), smem);
+    e = cudaFuncSetAttribute(synth<OG, ADJ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n0, synth<OG, ADJ, false>, OG * synth_pg(OG), smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, synth<OG, ADJ, true>, OG * synth_pg(OG), smem);
+  *per_sm = std::min(n0, n1);
   if (e == cudaSuccess && *per_sm < 1) e = cudaErrorInvalidConfiguration;
   return e;
 }
 
-constexpr size_t wg_smem(int CP) { return sizeof(float) * 2 * CP * kWgStride; }
+constexpr size_t wg_smem(int CP) { return sizeof(float) * 4 * CP * kWgStride; }
 
 // shared-memory sizes and blocks per SM of this network's kernels
 cudaError_t prepare_kernels(wf_fno_s* F) {
@@ -1070,8 +1219,13 @@ cudaError_t prepare_kernels(wf_fno_s* F) {
       default: e = prepare_synth<8, true>(sm, &F->adj_per_sm); break;
     }
   }
+  if (e == cudaSuccess && F->OG == 4)
+    e = cudaFuncSetAttribute(weight_grad<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wg_smem(32));
   if (e == cudaSuccess && F->OG == 8)
     e = cudaFuncSetAttribute(weight_grad<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wg_smem(64));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(F->KW == 1 ? analysis<4, 1> : analysis<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)an_smem(4, F->KW, F->lay.mx));
   return e;
 }
 
@@ -1115,7 +1269,7 @@ void weight_gradient(wf_fno_s* F, const float* in, int B, float* gW) {
     case 4: weight_grad<32><<<grid, 256, wg_smem(32), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
     default: weight_grad<64><<<grid, 256, wg_smem(64), F->stream>>>(F->gz, in, F->wpart, B, C, P); break;
   }
-  sum_partials<<<(C * C + 31) / 32, 256, 0, F->stream>>>(F->wpart, grid, C * C, gW, nullptr, 0, C);
+  sum_partials<<<(C * C + 31) / 32, 1024, 0, F->stream>>>(F->wpart, grid, C * C, gW, nullptr, 0, C);
 }
 
 // loss and gradient of the loss into F->grad (x, t device arrays), after
@@ -1125,10 +1279,10 @@ int backward(wf_fno_s* F, const float* x, const float* t, int B) {
   const int C = L.width, N = F->n, NM = (int)modes_(F), CP = 8 * F->OG;
   const int P = (int)P_(F);
   loss_partial<<<dim3(F->lblk, B), kThreads, 0, F->stream>>>(F->y, t, F->lpart, P);
-  loss_fin<<<1, 32, 0, F->stream>>>(F->lpart, F->lblk, B, F->dloss, F->inv);
+  loss_fin<<<1, 512, 0, F->stream>>>(F->lpart, F->lblk, B, F->dloss, F->inv);
   // projection Q, and g_z of the last layer
   const float* hL = F->h + (size_t)L.layers * act_(F);
-  const int pgrid = std::min(grid_for((size_t)B * P), 2 * F->sms);
+  const int pgrid = std::min(grid_for((size_t)B * P / 4), 2 * F->sms);
   const __half* Q = F->half + L.oQ;
   switch (F->OG) {
     case 1: proj_bwd<8><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
@@ -1136,7 +1290,7 @@ int backward(wf_fno_s* F, const float* x, const float* t, int B) {
     case 4: proj_bwd<32><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
     default: proj_bwd<64><<<pgrid, kThreads, 0, F->stream>>>(F->y, t, F->inv, Q, hL, F->gz, F->wpart, B, C, P); break;
   }
-  sum_partials<<<(CP + 32) / 32, 256, 0, F->stream>>>(F->wpart, pgrid, CP + 1, F->grad + L.oQ, F->grad + L.oq, 2, C);
+  sum_partials<<<(CP + 32) / 32, 1024, 0, F->stream>>>(F->wpart, pgrid, CP + 1, F->grad + L.oQ, F->grad + L.oq, 2, C);
   const float sc = 1.f / ((float)N * (float)N);
   for (int l = L.layers - 1; l >= 0; --l) {
     const float* hin = F->h + (size_t)l * act_(F);
@@ -1162,7 +1316,7 @@ int backward(wf_fno_s* F, const float* x, const float* t, int B) {
     }
     const int g = launch_synth<true>(F, a, B);
     if (l == 0)
-      sum_partials<<<(CP * 3 + 31) / 32, 256, 0, F->stream>>>(F->wpart, g, CP * 3, F->grad + L.oP, F->grad + L.op, 1,
+      sum_partials<<<(CP * 3 + 31) / 32, 1024, 0, F->stream>>>(F->wpart, g, CP * 3, F->grad + L.oP, F->grad + L.op, 1,
                                                               C);
   }
   return (int)cudaGetLastError();
@@ -1204,7 +1358,7 @@ int wf_fno_create(wf_fno_t* out, int n, int batch, int width, int mx, int my, in
   const size_t T = F->lay.total, P = (size_t)n * n;
   F->lblk = 32;
   F->OG = width <= 8 ? 1 : (width <= 16 ? 2 : (width <= 32 ? 4 : 8));
-  F->KG = ((mx + 1) / 2 + 1) / 2;  // pairs of modes of one parity
+  F->KW = ((mx + 1) / 2 + 7) / 8;  // sets of 8 modes of one parity
   const int CP = 8 * F->OG;
   if (prepare_kernels(F) != cudaSuccess) {
     cudaGetLastError();
@@ -1221,7 +1375,7 @@ int wf_fno_create(wf_fno_t* out, int n, int batch, int width, int mx, int my, in
             alloc(F, &F->X, (size_t)layers * batch * width * modes_(F)) &&
             alloc(F, &F->gY, (size_t)batch * width * modes_(F)) && alloc(F, &F->Y, (size_t)batch * CP * modes_(F)) &&
             alloc(F, &F->S, (size_t)batch * n * mx * 2 * CP) && alloc(F, &F->tw_x, (size_t)mx * n) &&
-            alloc(F, &F->tw_y, (size_t)2 * my * n) && alloc(F, &F->tw_k, (size_t)(n / 2) * 4 * F->KG) &&
+            alloc(F, &F->tw_y, (size_t)2 * my * n) && alloc(F, &F->tw_k, (size_t)(n / 2) * 16 * F->KW) &&
             alloc(F, &F->wpart, wpart) && alloc(F, &F->lpart, (size_t)batch * F->lblk * 2) &&
             alloc(F, &F->dloss, 1) && alloc(F, &F->inv, batch);
   if (!ok) {
@@ -1243,9 +1397,9 @@ int wf_fno_create(wf_fno_t* out, int n, int batch, int width, int mx, int my, in
     }
   }
   // the analysis's row table: [x][parity][k / 2], x < n/2, 0 beyond mx
-  std::vector<float2> tk((size_t)(n / 2) * 4 * F->KG, make_float2(0.f, 0.f));
+  std::vector<float2> tk((size_t)(n / 2) * 16 * F->KW, make_float2(0.f, 0.f));
   for (int x = 0; x < n / 2; ++x)
-    for (int k = 0; k < mx; ++k) tk[(size_t)x * 4 * F->KG + (k & 1) * 2 * F->KG + k / 2] = tx[(size_t)k * n + x];
+    for (int k = 0; k < mx; ++k) tk[(size_t)x * 16 * F->KW + (k & 1) * 8 * F->KW + k / 2] = tx[(size_t)k * n + x];
   const cudaMemcpyKind k = dev_ptr(params) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   ok = cudaMemcpy(F->tw_x, tx.data(), tx.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
        cudaMemcpy(F->tw_y, ty.data(), ty.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
