@@ -42,6 +42,7 @@ struct wf_plan_s {
   float2 *eig = nullptr, *eig_nyq = nullptr;
   float *pst = nullptr, *a2 = nullptr;
   float2 *twx = nullptr, *twy = nullptr, *twh = nullptr;  // twh: exp(-2 pi i k/(nx/2))
+  float2 *tws_row[2] = {}, *tws_col[2] = {};              // stage tables of the passes' shapes
   float2 *r_g = nullptr, *r_q = nullptr;
   double* part = nullptr;
   double* chi = nullptr;  // wf_chi2_aug: partial sums, then the value
@@ -83,6 +84,8 @@ struct wf_plan_s {
   // the state it restores after timing
   int row_variant = 0, col_variant = 0;
   bool tuned = false;
+  // the row pass's tensor maps of the column-tiled fields, per shape
+  CUtensorMap tm_t[2], tm_x[2];
   // the column pass hints the next wave's tiles into L2 (maps whose sweep
   // moves more bytes than L2 holds)
   bool l2_prefetch = false;
@@ -227,6 +230,48 @@ static bool sweep_above_l2(int ny, int nx) {
   return 40.0 * ny * nx > (double)l2;
 }
 
+// The stage table (StageTable in wf_device.cuh) of a transform whose threads
+// hold E values, from its table exp(-2 pi i k / L).
+static std::vector<float2> stage_table(const std::vector<float2>& tab, int E) {
+  const int L = (int)tab.size(), p2 = E & -E;
+  std::vector<float2> out;
+  for (int ns = 1, r = 0; ns < L; ns *= r) {
+    r = (ns == 1 && L % 3 == 0) ? E : std::min(p2, L / ns);
+    if (ns == 1) continue;
+    for (int q = 0; q == 0 || 4 * q < r; ++q)
+      for (int jm = 0; jm < ns; ++jm) out.push_back(tab[(size_t)jm * (L / (ns * r)) * (q ? 4 * q : 1)]);
+  }
+  return out;
+}
+
+// Tensor map of a column-tiled RF field for the row pass: a matrix of M / 4
+// tiles by 8 ny floats (a tile's rows are contiguous, 32 bytes each), copied in
+// boxes of `rows` rows by up to 256 tiles.
+static bool tile_map(CUtensorMap* map, const float2* field, int ny, int M, int rows) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static Encode encode = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      encode = reinterpret_cast<Encode>(fn);
+    else
+      cudaGetLastError();
+  });
+  if (!encode) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)ny * 2 * WF_TW, (cuuint64_t)(M / WF_TW)};
+  const cuuint64_t strides[1] = {(cuuint64_t)ny * WF_TW * sizeof(float2)};
+  const cuuint32_t box[2] = {(cuuint32_t)(rows * 2 * WF_TW), (cuuint32_t)std::min(M / WF_TW, 256)};
+  const cuuint32_t es[2] = {1, 1};
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float2*>(field), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Host-side validation shared by wf_plan_create and wf_batch_create (no CUDA call).
 int wf::check_plan_args(int ny, int nx, unsigned parts, const wf_params* p) {
   if (!size_supported(nx) || !size_supported(ny)) return WF_EUNSUPPORTED;
@@ -300,6 +345,10 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
   AL(P->twx, (size_t)nx);
   AL(P->twy, (size_t)ny);
   AL(P->twh, (size_t)(nx / 2));
+  for (int v = 0; v < 2; ++v) {
+    AL(P->tws_row[v], (size_t)nx);  // (the tables have fewer than twice the transform's values)
+    AL(P->tws_col[v], (size_t)2 * ny);
+  }
   AL(P->r_g, nh);
   AL(P->r_q, nh);
   AL(P->part, (size_t)3 * P->nrow + 4 * 256 + 64);
@@ -363,6 +412,17 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
     wf_plan_destroy(P);
     return WF_ECUDA;
   }
+  // tensor maps of the column-tiled fields the row pass copies
+  for (int v = 0; v < 2 && rc == WF_OK; ++v) {
+    const int rows = row_pass_rows(P->M, v);
+    if (!tile_map(&P->tm_t[v], P->has_rf ? P->f_t1 : P->f_y, ny, P->M, rows) ||
+        !tile_map(&P->tm_x[v], P->f_x, ny, P->M, rows))
+      rc = WF_ECUDA;
+  }
+  if (rc != WF_OK) {
+    wf_plan_destroy(P);
+    return rc;
+  }
   // one cooperative launch per R sweeps, when asked for
   if (prm.sweep_kernel == 1) {
     P->fused = fused_supported(ny, nx, P->has_rf, P->merge || !P->has_f, prm.dft_precision);
@@ -387,7 +447,15 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
   cudaError_t e1 = cudaMemcpy(P->twx, tx.data(), nx * sizeof(float2), cudaMemcpyHostToDevice);
   cudaError_t e2 = cudaMemcpy(P->twy, ty.data(), ny * sizeof(float2), cudaMemcpyHostToDevice);
   cudaError_t e3 = cudaMemcpy(P->twh, th.data(), nx / 2 * sizeof(float2), cudaMemcpyHostToDevice);
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
+  bool tabs = e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess;
+  for (int v = 0; v < 2 && tabs; ++v) {
+    const std::vector<float2> r = stage_table(th, row_pass_e(P->M, v)), c = stage_table(ty, col_pass_e(ny, v));
+    tabs = r.size() <= (size_t)nx && c.size() <= (size_t)2 * ny &&
+           cudaMemcpy(P->tws_row[v], r.data(), r.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
+           cudaMemcpy(P->tws_col[v], c.data(), c.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
+  }
+  if (!tabs) {
+    cudaGetLastError();
     wf_plan_destroy(P);
     return WF_ECUDA;
   }
@@ -401,6 +469,8 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
 static RowArgs row_args(wf_plan_s* P) {
   RowArgs a{};
   a.variant = P->row_variant;
+  a.tm_t = P->tm_t[P->row_variant];
+  a.tm_x = P->tm_x[P->row_variant];
   a.ny = P->ny;
   a.nx = P->nx;
   a.has_rf = P->has_rf;
@@ -413,6 +483,7 @@ static RowArgs row_args(wf_plan_s* P) {
   a.a2 = P->a2;
   a.twx = P->twx;
   a.twh = P->twh;
+  a.tws = P->tws_row[P->row_variant];
   a.st = P->st;
   a.r_g = P->r_g;
   a.r_q = P->r_q;
@@ -437,6 +508,7 @@ static ColArgs col_args(wf_plan_s* P, int parity) {
   a.eig = P->eig;
   a.eig_nyq = P->eig_nyq;
   a.twy = P->twy;
+  a.tws = P->tws_col[a.variant];
   a.st = P->st;
   a.r_g = P->r_g;
   a.r_q = P->r_q;

@@ -71,6 +71,28 @@ __device__ __forceinline__ float2 merged_mode(float2 v, float2 vp, float2 eg, fl
   }
 }
 
+// merged_mode for the CTA of the packed column 0, without a branch on the
+// lanes that hold it: with A and B the pair behind Z and its partner Zp = Z[-k],
+// fa A + i fb B = (fa + fb)/2 Z + (fa - fb)/2 conj(Zp), and the same for the
+// source.  Other columns pass their own value and eigenvalues as the partner's
+// (fb = fa).  That CTA is the last of a grid that fits on the device at once,
+// so its extra work is the pass's.
+template <bool SRC>
+__device__ __forceinline__ float2 merged_pair(float2 v, float2 vp, float2 eg, float2 egb, float off0, float Tl,
+                                              float2 jv, float2 jp) {
+  const float pa = eg.x + eg.y + off0, pb = egb.x + egb.y + off0;
+  const float ia = __fdividef(1.f, pa + Tl), ib = __fdividef(1.f, pb + Tl);
+  const float fa = pa * ia, fb = pb * ib;
+  const float hs = 0.5f * (fa + fb), hd = 0.5f * (fa - fb);
+  float2 r = make_float2(fmaf(hd, vp.x, hs * v.x), fmaf(-hd, vp.y, hs * v.y));
+  if constexpr (SRC) {
+    const float ga = Tl * eg.x * ia, gb = Tl * egb.x * ib;
+    const float gs = 0.5f * (ga + gb), gd = 0.5f * (ga - gb);
+    r = make_float2(fmaf(gs, jv.x, fmaf(gd, jp.x, r.x)), fmaf(gs, jv.y, fmaf(-gd, jp.y, r.y)));
+  }
+  return r;
+}
+
 // The column pass for one column length (wf_colpass.cu): modes COL_PASS_*.
 template <int L>
 int launch_col_pass_any(int mode, const ColArgs& a, cudaStream_t s);

@@ -9,6 +9,7 @@
 // and the 1/f noise are diagonal).
 #pragma once
 
+#include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -135,9 +136,36 @@ __device__ __forceinline__ void dft16(float2* a) {
   }
 }
 
+// 3 P-point DFT, P = 4 or 8, by the prime-factor split (3 and P are coprime, so
+// no twiddles): with n = (P n1 + 3 n2) mod 3P and k = (c k1 + 9 k2) mod 3P, c =
+// 1 mod 3 and 0 mod P, n k = P n1 k1 + 3 n2 k2 mod 3P -- P transforms of
+// length 3 over n1, then 3 of length P over n2.
+template <int P, bool INV>
+__device__ __forceinline__ void dft3P(float2* a) {
+  constexpr int N = 3 * P, c = (P % 3 == 1) ? P : 2 * P;
+  float2 b[3][P];
+#pragma unroll
+  for (int n2 = 0; n2 < P; ++n2) {
+    float2 x0 = a[(3 * n2) % N], x1 = a[(P + 3 * n2) % N], x2 = a[(2 * P + 3 * n2) % N];
+    dft3<INV>(x0, x1, x2);
+    b[0][n2] = x0;
+    b[1][n2] = x1;
+    b[2][n2] = x2;
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    if constexpr (P == 4) dft4<INV>(b[k1][0], b[k1][1], b[k1][2], b[k1][3]);
+    else dft8<INV>(b[k1]);
+#pragma unroll
+    for (int k2 = 0; k2 < P; ++k2) a[(c * k1 + 9 * k2) % N] = b[k1][k2];
+  }
+}
+
 template <int R, bool INV>
 __device__ __forceinline__ void dftR(float2* u) {
-  if constexpr (R == 3) dft3<INV>(u[0], u[1], u[2]);
+  if constexpr (R == 12) dft3P<4, INV>(u);
+  else if constexpr (R == 24) dft3P<8, INV>(u);
+  else if constexpr (R == 3) dft3<INV>(u[0], u[1], u[2]);
   else if constexpr (R == 2) dft2<INV>(u[0], u[1]);
   else if constexpr (R == 4) dft4<INV>(u[0], u[1], u[2], u[3]);
   else if constexpr (R == 8) dft8<INV>(u);
@@ -152,15 +180,33 @@ template <int L>
 struct SPad { static constexpr int size = L + L / 16; };
 
 // Radix of the stage that starts with sub-transform length NS.  Lengths are
-// 2^k or 3 * 2^k: a factor 3 is taken by the first stage (E then holds a
-// factor 3 too), the rest by powers of two up to the largest one dividing E.
+// 2^k or 3 * 2^k: of the latter, the first stage takes all E = 12 or 24 values
+// of a thread at once (one exchange fewer than a radix-3 stage of its own),
+// the rest go by powers of two up to the largest one dividing E.
 template <int L, int E, int NS>
 struct StageRadix {
   static_assert(L % 3 != 0 || E % 3 == 0, "lengths 3*2^k need a factor 3 in E");
   static constexpr int P2 = E & -E;  // largest power of two dividing E
   static constexpr int rem = L / NS;
-  static constexpr int value = (NS == 1 && L % 3 == 0) ? 3 : (rem >= P2 ? P2 : rem);
+  static constexpr int value = (NS == 1 && L % 3 == 0) ? E : (rem >= P2 ? P2 : rem);
+  static_assert(L % 3 != 0 || E == 12 || E == 24, "3 * 2^k: 12 or 24 values per thread");
 };
+
+// Twiddles of one transform in the order its stages read them: for every stage
+// after the first (sub-transform length NS, radix R) and q = 0, 1, ...
+// (the powers 1, 4, 8, 12 below R), NS values W_{NS R}^{jm q'} over jm.  The lanes
+// of a warp read consecutive ones, where the table exp(-2 pi i k / L) has them
+// 8 lines apart.  Built by stage_table (wf_api.cu).
+template <int R>
+struct StageQ { static constexpr int n = R <= 4 ? 1 : (R == 8 ? 2 : (R == 12 ? 3 : 4)); };
+template <int L, int E, int NS = 1>
+struct StageTable {
+  static constexpr int R = StageRadix<L, E, NS>::value;
+  static constexpr int here = NS == 1 ? 0 : NS * StageQ<R>::n;
+  static constexpr int size = here + StageTable<L, E, NS * R>::size;
+};
+template <int L, int E>
+struct StageTable<L, E, L> { static constexpr int size = 0; };
 
 // (L - k) mod L for 0 <= k < L: the index of the mode -k.
 template <int L>
@@ -365,6 +411,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, int max
 // try_wait already suspends for a hardware-chosen interval per attempt; this
 // many attempts is far beyond the microseconds a bulk copy takes.
 constexpr int WF_WAIT_TRIES = 1 << 20;
+
+// 2D tensor copies (cp.async.bulk.tensor) of a box at (x, y) of the map: shared
+// addresses on 128 bytes, x a multiple of 16 bytes.  Loads complete on an
+// mbarrier; the storing thread waits until its stores are written.
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+__device__ __forceinline__ void tma2d_g2s(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tma2d_s2g(const CUtensorMap* map, int x, int y, const void* src) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y), "r"(smem_u32(src))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() {
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
 
 // Ampere-style asynchronous copies (16 or 8 bytes per thread) for strided tiles.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -626,13 +696,16 @@ __device__ __forceinline__ void tc5_teardown() {
 // Inputs are the "natural" layout (thread t holds x[t + m*TPF], m =
 // b + r*(E/R)); outputs go to shared memory at their autosort positions, or,
 // for the last stage, back to the registers in the natural layout.
-// twtab holds exp(-2 pi i k / (L*twstride)), k < L*twstride.  PREC != 0 runs
-// the radix-16 stages of 16-value threads on the tensor cores (above).
-template <int L, int E, int NS, bool INV, bool WARP, bool TWS = false, int PREC = 0>
+// twtab holds exp(-2 pi i k / (L*twstride)), k < L*twstride, or, with OFF >= 0,
+// the stage table of this transform (OFF: where this stage's part starts).
+// PREC != 0 runs the radix-16 stages of 16-value threads on the tensor cores
+// (above).
+template <int L, int E, int NS, bool INV, bool WARP, bool TWS = false, int PREC = 0, int OFF = -1>
 struct FFTStages {
+  static constexpr int R = StageRadix<L, E, NS>::value;
+  static constexpr int NEXT = OFF < 0 ? -1 : OFF + (NS == 1 ? 0 : NS * StageQ<R>::n);
   static __device__ __forceinline__ void run(float2 (&v)[E], float2* sb, int t,
                                              const float2* __restrict__ twtab, int twstride) {
-    constexpr int R = StageRadix<L, E, NS>::value;
     constexpr int TPF = L / E;
     constexpr bool LAST = (NS * R == L);
     constexpr bool TC = (PREC != 0 && R == 16 && E == 16 && !WARP);
@@ -643,7 +716,7 @@ struct FFTStages {
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = sb[spad(t + m * TPF)];
       fft_sync<WARP>();
-      if constexpr (!LAST) FFTStages<L, E, NS * R, INV, WARP, TWS, PREC>::run(v, sb, t, twtab, twstride);
+      if constexpr (!LAST) FFTStages<L, E, NS * R, INV, WARP, TWS, PREC, NEXT>::run(v, sb, t, twtab, twstride);
     } else {
       stage_fp32(v, sb, t, twtab, twstride);
     }
@@ -651,7 +724,6 @@ struct FFTStages {
 
   static __device__ __forceinline__ void stage_fp32(float2 (&v)[E], float2* sb, int t,
                                                     const float2* __restrict__ twtab, int twstride) {
-    constexpr int R = StageRadix<L, E, NS>::value;
     constexpr int TPF = L / E;
     constexpr int B = E / R;
     constexpr bool LAST = (NS * R == L);
@@ -665,12 +737,15 @@ struct FFTStages {
       if constexpr (NS > 1) {
         // twiddles W_{NS R}^{jm r}: exact table values every 4th power,
         // products in between (at most 3 multiplications deep)
-        const int step = jm * (L / (NS * R)) * twstride;
-        float2 w1 = tw_dir<INV>(tw_load<TWS>(twtab, step));
+        const int step = OFF < 0 ? jm * (L / (NS * R)) * twstride : 0;
+        auto tw = [&](int r) {
+          return tw_dir<INV>(tw_load<TWS>(twtab, OFF < 0 ? step * r : OFF + (r / 4) * NS + jm));
+        };
+        float2 w1 = tw(1);
         float2 wr = w1;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          if ((r & 3) == 0) wr = tw_dir<INV>(tw_load<TWS>(twtab, step * r));
+          if ((r & 3) == 0) wr = tw(r);
           u[r] = cmul(u[r], wr);
           wr = cmul(wr, w1);
         }
@@ -690,7 +765,7 @@ struct FFTStages {
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = sb[spad(t + m * TPF)];
       fft_sync<WARP>();
-      FFTStages<L, E, NS * R, INV, WARP, TWS, PREC>::run(v, sb, t, twtab, twstride);
+      FFTStages<L, E, NS * R, INV, WARP, TWS, PREC, NEXT>::run(v, sb, t, twtab, twstride);
     }
   }
 };
@@ -702,6 +777,11 @@ template <int L, int E, bool INV, bool WARP = false, bool TWS = false, int PREC 
 __device__ __forceinline__ void fft_block(float2 (&v)[E], float2* sb, int t,
                                           const float2* __restrict__ twtab, int twstride) {
   FFTStages<L, E, 1, INV, WARP, TWS, PREC>::run(v, sb, t, twtab, twstride);
+}
+// The same with the transform's stage table.
+template <int L, int E, bool INV, bool WARP = false, bool TWS = false>
+__device__ __forceinline__ void fft_staged(float2 (&v)[E], float2* sb, int t, const float2* __restrict__ table) {
+  FFTStages<L, E, 1, INV, WARP, TWS, 0, 0>::run(v, sb, t, table, 1);
 }
 
 // W_N^k (N = 2M) for the k = t + m*(M/E) a thread handles in c2r_pre and
@@ -738,6 +818,28 @@ __device__ __forceinline__ void c2r_pre_w(float2 (&v)[E], float2* sb, int t, con
       float2 Xm = cconj(sb[spad(M - k)]);
       float2 Ek = cadd(X, Xm);
       float2 Ok = cmul(csub(X, Xm), cconj(wk[m]));
+      v[m] = make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
+    }
+  }
+  fft_sync<WARP>();
+}
+
+// The same with X in shared memory (at(k) gives X[k]), possibly the transform's
+// own buffer: every value and its partner are read from there, then it is free.
+template <int M, int E, bool WARP, typename At>
+__device__ __forceinline__ void c2r_pre_in(float2 (&v)[E], int t, const float2* __restrict__ twx, const At& at) {
+  constexpr int TPF = M / E;
+  const float s = 0.5f / (float)M;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int k = t + m * TPF;
+    const float2 X = at(k);
+    if (k == 0) {
+      v[m] = make_float2((X.x + X.y) * s, (X.x - X.y) * s);
+    } else {
+      const float2 Xm = cconj(at(M - k));
+      const float2 Ek = cadd(X, Xm);
+      const float2 Ok = cmul(csub(X, Xm), cconj(__ldg(&twx[k])));
       v[m] = make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
     }
   }

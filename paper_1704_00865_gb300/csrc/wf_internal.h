@@ -2,6 +2,7 @@
 // translation units of libwf (not part of the public ABI).
 #pragma once
 
+#include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -29,11 +30,6 @@ constexpr int WF_TW = 4;
 // anything the iteration writes.
 #ifndef WF_PDL
 #define WF_PDL 1
-#endif
-// 1: the passes release the next kernel at entry; 0: after their last
-// transform, before the stores
-#ifndef WF_PDL_EARLY
-#define WF_PDL_EARLY 0
 #endif
 template <typename... KArgs, typename... Args>
 inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -97,7 +93,8 @@ struct RowArgs {
   const float* pst;           // [nx/2+1] stripe eigenvalues
   const float* a2;            // [ny] a(y)^2 or nullptr
   const float2* twx;          // exp(-2 pi i k/nx), k < nx
-  const float2* twh;          // exp(-2 pi i k/(nx/2)), k < nx/2 (row pass)
+  const float2* twh;          // exp(-2 pi i k/(nx/2)), k < nx/2
+  const float2* tws;          // row pass: stage table of its shape (StageTable)
   WfState* st;
   float2* r_g;                // residual scratch (RF)
   float2* r_q;
@@ -110,6 +107,8 @@ struct RowArgs {
   const float2* src_px;       // source j on masked pixels (pairs) or nullptr
   float2* gm_out;             // S^-1 s on masked pixels (pairs), 0 elsewhere, or nullptr
   int variant;                // row pass shape (0 or 1), chosen by the autotuner
+  CUtensorMap tm_t;           // row pass: t_RF (or t_PX) and the signal-side field as tiles
+  CUtensorMap tm_x;           // (tile_map, rows of the pass's shape)
 };
 
 struct ColArgs {
@@ -125,6 +124,7 @@ struct ColArgs {
   const float2* eig;          // [ny][nx/2] (C, P1f) for kx = col
   const float2* eig_nyq;      // [ny] (C, P1f) at kx = nx/2
   const float2* twy;          // exp(-2 pi i k/ny), k < ny
+  const float2* tws;          // column pass: stage table of its shape
   WfState* st;
   float2* r_g;
   float2* r_q;
@@ -137,6 +137,9 @@ struct ColArgs {
   int prefetch;               // column pass: hint the tiles of the CTA one wave ahead into L2
   int pf;                     // (set by the launcher) that distance in CTAs, 0 = off
 };
+
+// Dynamic shared memory per CTA and per SM (1 KB of it reserved per CTA).
+constexpr size_t kMaxDynSmem = 227 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024;
 
 // CTAs of a kernel resident at once on the current device (SMs x CTAs per
 // SM for the block and dynamic shared memory), or 0 if the query fails: the
@@ -168,6 +171,7 @@ bool col_tc_supported(int L);
 bool col_tc5_supported(int L);  // tcgen05 stages (dft_precision 3, 4)
 // values per thread of the row / column pass shape `variant` for a length
 int row_pass_e(int M, int variant);
+int row_pass_rows(int M, int variant);  // rows per CTA
 int col_pass_e(int L, int variant);
 
 // The whole sweep, nsweeps times, in one cooperative launch (wf_fused.cu):

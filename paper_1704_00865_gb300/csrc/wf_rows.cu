@@ -181,11 +181,13 @@ row_kernel(RowArgs a) {
 // units that the SMs finish within one row of each other.
 // Values per thread of the two shapes the autotuner chooses between (one
 // where both coincide): 8 (two warps per 1024-point row) measured fastest at
-// 1024^2 and above, 4 at 512^2 and below; 3 * 2^k rows take 12.
+// 1024^2 and above (16 values: 20.1 against 19.0 us at 2048^2, 97 against 90 at
+// 4096^2), 4 at 512^2 and below; 3 * 2^k rows take 12 (13.0 -> 17.0 us at 1536^2)
+// or 24 (the other way round from 768^2 down).
 template <int M>
 struct RowPassE {
   static constexpr int v0 = (M % 3 == 0) ? 12 : 8;
-  static constexpr int v1 = (M % 3 == 0) ? 12 : 4;
+  static constexpr int v1 = (M % 3 == 0) ? 24 : 4;
 };
 template <int M, int EV>
 struct RowPassCfg {
@@ -196,172 +198,215 @@ struct RowPassCfg {
   static constexpr bool WARP = (THREADS == 32);
 };
 
+// Shared memory of the row pass.  The tiles of the column-tiled fields keep
+// their order, [tile][row][4 columns].  EARLY (rows up to 512 values, whose
+// CTAs all fit at once): every input has its own buffer and is requested at the
+// start.  Longer rows: the field of the first transform lands in the
+// transform's own buffer (its values and their partners -k are read from there
+// before the first exchange overwrites them), and t_RF and the signal-side
+// field take the pixel table's place once the pixel update has read it -- 50
+// instead of 99 KB at 2048 values, so four CTAs of an SM overlap one
+// another's loads and transforms.
 template <int M, int MODE, int EV>
 struct RowPassSmem {
   static constexpr int ROWS = RowPassCfg<M, EV>::ROWS;
+  static constexpr int NT = RowPassCfg<M, EV>::THREADS;
   static constexpr bool RF = (MODE == ROW_PASS_RF);
-  static constexpr size_t a_off = 16;
-  static constexpr size_t dn_off = a_off + (size_t)ROWS * M * 8;
-  static constexpr size_t t1_off = dn_off + (size_t)ROWS * M * 16;
-  static constexpr size_t x_off = t1_off + (RF ? (size_t)ROWS * M * 8 : 0);
-  static constexpr size_t tw_off = x_off + (RF ? (size_t)ROWS * M * 8 : 0);  // twh, M values
-  static constexpr size_t fft_bytes = (size_t)ROWS * SPad<M>::size * 8;
-  // the transform twiddles are staged too where that costs no CTA per SM
-  // (228 KB per SM, 1 KB reserved per CTA); up to 512-point rows a whole
-  // 1024^2 row pass is resident either way, and staging measured faster
-  static constexpr size_t kSM = 228 * 1024, kRes = 1024;
-  static constexpr size_t base_bytes = tw_off + fft_bytes;
-  static constexpr bool TWS =
-      M <= 512 || kSM / (base_bytes + (size_t)M * 8 + kRes) == kSM / (base_bytes + kRes);
-  static constexpr size_t fft_off = tw_off + (TWS ? (size_t)M * 8 : 0);
-  static constexpr size_t bytes = fft_off + fft_bytes;
+  static constexpr bool EARLY = M <= 512;
+  static constexpr size_t al(size_t n) { return (n + 127) / 128 * 128; }
+  static constexpr size_t field = (size_t)ROWS * M * 8;
+  static constexpr size_t fft_off = 128;
+  static constexpr size_t dn_off = fft_off + al((size_t)ROWS * SPad<M>::size * 8);
+  static constexpr size_t in_off = EARLY ? dn_off + 2 * field : fft_off;  // the first transform's field
+  static constexpr size_t t_off = !RF ? dn_off : (EARLY ? in_off + field : dn_off);  // t_RF, then the signal side
+  static constexpr size_t tw_off = EARLY ? in_off + field + (RF ? 2 * field : 0) : dn_off + 2 * field;
+  // the transform twiddles are staged too for short rows
+  static constexpr bool TWS = M <= 512;
+  static constexpr uint32_t tw_bytes = StageTable<M, EV>::size * 8;  // a multiple of 16
+  static constexpr size_t bytes = tw_off + (TWS ? tw_bytes : 0);
+  // resident CTAs the registers are held to: 64 a thread for long rows, 102
+  // and 170 for 12 and 24 values
+  static constexpr int min_ctas =
+      EV == 12 ? 640 / NT : (EV == 24 ? 384 / NT : (M >= 768 ? 1024 / NT : 1));
+  // position of value k of row r in a tiled buffer
+  static __device__ __forceinline__ int tpos(int r, int k) {
+    return (k / WF_TW) * (ROWS * WF_TW) + r * WF_TW + (k % WF_TW);
+  }
 };
 
-// Gather rows y0 .. y0+nrows-1 of a column-tiled RF field into row-major
-// shared memory, 16 bytes (two complex values) per asynchronous copy.
-template <int M, int THREADS>
-__device__ __forceinline__ void gather_tiled_rows(float2* dst, const float2* src, int y0, int nrows, int ny) {
-  for (int i = threadIdx.x; i < nrows * (M / 2); i += THREADS) {
-    const int r = i / (M / 2);
-    const int k = (i - r * (M / 2)) * 2;
-    cp_async16(dst + r * M + k, src + tidx(y0 + r, k, ny));
-  }
-}
+constexpr int kBoxTiles = 256;  // column tiles of one tensor copy
 
 // The row pass (Sec. 2: eq. 2mess_t1 analogue in pixels between the inverse
-// and forward row DFTs, then the stripe-basis updates).  Row-major inputs
-// (d_RF, the pixel table) arrive by TMA bulk copies on an mbarrier, the
-// column-tiled ones (t_RF, the signal-side field) by 16-byte asynchronous
-// copies; the first transform starts as soon as its own field is in.  Waits
-// are bounded; on a timeout the CTA records WF_ERR_TIMEOUT, drains its
+// and forward row DFTs, then the stripe-basis updates).  Every copy is the
+// TMA's: row-major inputs (d_RF, the pixel table) by bulk copies, the
+// column-tiled ones (t_RF, the signal-side field) and the new t_RF by 2D tensor
+// copies of all the row's 32-byte pieces.  (Gathered by 16-byte asynchronous
+// copies and stored by 8-byte stores, those pieces took a shared-memory
+// wavefront each: 66 % of the load-store pipe at 4096^2, the pass's bound.)
+// Waits are bounded; on a timeout the CTA records WF_ERR_TIMEOUT, drains its
 // copies (bounded) and returns.
 template <int M, int MODE, int EV>
-__global__ void __launch_bounds__(RowPassCfg<M, EV>::THREADS)
-row_pass_kernel(RowArgs a) {
+__global__ void __launch_bounds__(RowPassCfg<M, EV>::THREADS, RowPassSmem<M, MODE, EV>::min_ctas)
+row_pass_kernel(const __grid_constant__ RowArgs a) {
   using Cfg = RowPassCfg<M, EV>;
   using SM = RowPassSmem<M, MODE, EV>;
-  constexpr int E = Cfg::E, TPF = Cfg::TPF, ROWS = Cfg::ROWS, NT = Cfg::THREADS;
+  constexpr int E = Cfg::E, TPF = Cfg::TPF, ROWS = Cfg::ROWS;
   constexpr bool W = Cfg::WARP;
-  constexpr bool RF = SM::RF;
-  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool RF = SM::RF, EARLY = SM::EARLY;
+  constexpr uint32_t kField = (uint32_t)SM::field;
+  extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-  float2* s_a = reinterpret_cast<float2*>(smem + SM::a_off);
-  float4* s_dn = reinterpret_cast<float4*>(smem + SM::dn_off);
-  float2* s_t1 = reinterpret_cast<float2*>(smem + SM::t1_off);
-  float2* s_x = reinterpret_cast<float2*>(smem + SM::x_off);
-  float2* s_tw = reinterpret_cast<float2*>(smem + SM::tw_off);
   float2* s_fft = reinterpret_cast<float2*>(smem + SM::fft_off);
+  float4* s_dn = reinterpret_cast<float4*>(smem + SM::dn_off);
+  float2* s_in = reinterpret_cast<float2*>(smem + SM::in_off);
+  float2* s_t1 = reinterpret_cast<float2*>(smem + SM::t_off);
+  float2* s_x = s_t1 + ROWS * M;
+  float2* s_tw = reinterpret_cast<float2*>(smem + SM::tw_off);
 
   const int g = threadIdx.x / TPF;
   const int t = threadIdx.x - g * TPF;
-  const int y0 = blockIdx.x * ROWS;
-  const int nval = min(ROWS, a.ny - y0);
+  const int y0 = blockIdx.x * ROWS;  // ny is a multiple of ROWS
   const int y = y0 + g;
-  const bool valid = g < nval;
   float2* sb = s_fft + g * SPad<M>::size;
+
+  // one row group of a column-tiled field into (or out of) a tiled buffer
+  auto load_tiled = [&](float2* dst, const CUtensorMap* map, uint64_t* b) {
+#pragma unroll
+    for (int j = 0; j < M / WF_TW; j += kBoxTiles)
+      tma2d_g2s(dst + j * ROWS * WF_TW, map, y0 * 2 * WF_TW, j, b);
+  };
 
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+    mbar_init(&bar[2], 1);
     mbar_fence_init();
+    // before the previous kernel has finished: the pixel table (fixed during
+    // a solve) and the transform twiddles
+    mbar_expect_tx(&bar[1], 2 * kField + (SM::TWS ? SM::tw_bytes : 0));
+    if constexpr (SM::TWS) bulk_g2s(s_tw, a.tws, SM::tw_bytes, &bar[1]);
+    bulk_g2s(s_dn, a.dn + (size_t)y0 * M, 2 * kField, &bar[1]);
+    tma_prefetch_map(&a.tm_t);
+    tma_prefetch_map(&a.tm_x);
   }
-  fft_sync<W>();
-  if constexpr (WF_PDL_EARLY) pdl_trigger();
-  // before the previous kernel has finished: the pixel table (fixed during a
-  // solve) and the transform twiddles
-  if (threadIdx.x == 0) {
-    mbar_expect_tx(&bar[1], (uint32_t)(nval * M * 16 + (SM::TWS ? M * 8 : 0)));
-    if constexpr (SM::TWS) bulk_g2s(s_tw, a.twh, (uint32_t)(M * 8), &bar[1]);
-    for (int r = 0; r < nval; ++r) bulk_g2s(s_dn + r * M, a.dn + (size_t)(y0 + r) * M, M * 16, &bar[1]);
-  }
-  float2 wk[E];
-  load_rtw<M, E>(wk, t, a.twx);
+  float2 wk[EARLY ? E : 1];
+  if constexpr (EARLY) load_rtw<M, E>(wk, t, a.twx);
   // stripe spectrum a(y)^2 Pst(k) of this thread's modes (fixed during a solve)
-  float pk[RF ? E : 1];
+  float pk[RF && EARLY ? E : 1];
   float a2y = 1.f, pkn = 0.f;  // pkn: Pst at kx = M, packed with kx = 0
   if constexpr (RF) {
-    if (a.a2 != nullptr && valid) a2y = __ldg(&a.a2[y]);
+    if (a.a2 != nullptr) a2y = __ldg(&a.a2[y]);
+    if constexpr (EARLY) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) pk[m] = __ldg(&a.pst[t + m * TPF]);
+      for (int m = 0; m < E; ++m) pk[m] = __ldg(&a.pst[t + m * TPF]);
+    }
     if (t == 0) pkn = __ldg(&a.pst[M]);
   }
   pdl_wait();
   // the fields the previous kernels wrote
   if (threadIdx.x == 0) {
+    mbar_expect_tx(&bar[0], kField);
     if constexpr (RF) {
-      mbar_expect_tx(&bar[0], (uint32_t)(nval * M * 8));
-      for (int r = 0; r < nval; ++r) bulk_g2s(s_a + r * M, a.f_d1 + (size_t)(y0 + r) * M, M * 8, &bar[0]);
+      if constexpr (EARLY) {
+        bulk_g2s(s_in, a.f_d1 + (size_t)y0 * M, kField, &bar[0]);
+        mbar_expect_tx(&bar[2], 2 * kField);
+        load_tiled(s_t1, &a.tm_t, &bar[2]);
+        load_tiled(s_x, &a.tm_x, &bar[2]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) bulk_g2s(s_in + r * M, a.f_d1 + (size_t)(y0 + r) * M, M * 8, &bar[0]);
+      }
     } else {
-      mbar_expect_tx(&bar[0], 0u);  // nothing on this barrier: completes at once
+      load_tiled(s_in, &a.tm_x, &bar[0]);
     }
   }
-  if constexpr (RF) {
-    gather_tiled_rows<M, NT>(s_t1, a.f_t1, y0, nval, a.ny);
-    gather_tiled_rows<M, NT>(s_x, a.f_x, y0, nval, a.ny);
-  } else {
-    gather_tiled_rows<M, NT>(s_a, a.f_x, y0, nval, a.ny);
-  }
-  cp_async_commit();
   // link covariances of this lambda level (written by the controller)
   const float T2 = a.st->Tf[2];
   const float T1 = RF ? a.st->Tf[1] : 0.f;
   const float off1 = RF ? (float)a.st->off[1] : 0.f;
+  const bool done = a.check_done && a.st->done;  // uniform: set only between launches
+  __syncthreads();  // the barriers are initialised
 
+  // the copies requested so far, for a CTA that leaves early
   auto drain = [&]() {
     const bool ok0 = mbar_wait(&bar[0], 0, WF_WAIT_TRIES);
     const bool ok1 = mbar_wait(&bar[1], 0, WF_WAIT_TRIES);
-    cp_async_wait<0>();
-    if (!(ok0 && ok1)) atomicOr(&a.st->err, WF_ERR_TIMEOUT);
+    const bool ok2 = !(RF && EARLY) || mbar_wait(&bar[2], 0, WF_WAIT_TRIES);
+    if (!(ok0 && ok1 && ok2)) atomicOr(&a.st->err, WF_ERR_TIMEOUT);
   };
-  // uniform: the flag is set only between launches; the copies above are
-  // already in flight, so they land before the block exits
-  if (a.check_done && a.st->done) {
+  if (done) {
     drain();
     return;
   }
-  bool ok = mbar_wait(&bar[0], 0, WF_WAIT_TRIES) && mbar_wait(&bar[1], 0, WF_WAIT_TRIES);
-  if constexpr (!RF) cp_async_wait<0>();
+  const bool ok = mbar_wait(&bar[0], 0, WF_WAIT_TRIES) && mbar_wait(&bar[1], 0, WF_WAIT_TRIES);
   if (__syncthreads_or(!ok)) {
     drain();
     return;
   }
 
   float2 v[E];
+  if constexpr (EARLY) {
 #pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = s_a[g * M + t + m * TPF];
-  c2r_pre_w<M, E, W>(v, sb, t, wk);
-  fft_block<M, E, true, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.twh, 1);
+    for (int m = 0; m < E; ++m) {
+      const int k = t + m * TPF;
+      v[m] = RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)];
+    }
+    c2r_pre_w<M, E, W>(v, sb, t, wk);
+  } else {
+    c2r_pre_in<M, E, W>(v, t, a.twx, [&](int k) { return RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)]; });
+  }
+  fft_staged<M, E, true, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
   // eq. (2mess_t1) analogue in pixel space, two pixels per complex value
 #pragma unroll
   for (int m = 0; m < E; ++m) {
     const float4 q = s_dn[g * M + t + m * TPF];
     v[m] = make_float2(tpx_update(q.x, q.y, v[m].x, T2), tpx_update(q.z, q.w, v[m].y, T2));
   }
-  fft_block<M, E, false, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.twh, 1);
-  r2c_post_w<M, E, W>(v, sb, t, wk);
-  if constexpr (!WF_PDL_EARLY) pdl_trigger();
-  if constexpr (RF) {
-    cp_async_wait<0>();
-    fft_sync<W>();
+  if constexpr (RF && !EARLY) {
+    __syncthreads();  // the pixel table is read
+    if (threadIdx.x == 0) {
+      mbar_expect_tx(&bar[2], 2 * kField);
+      load_tiled(s_t1, &a.tm_t, &bar[2]);
+      load_tiled(s_x, &a.tm_x, &bar[2]);
+    }
   }
-  if (!valid) return;
-  const size_t row0 = (size_t)y * M;
-  if constexpr (!RF) {
-#pragma unroll
-    for (int m = 0; m < E; ++m) a.f_y[tidx(y, t + m * TPF, a.ny)] = v[m];
-  } else {
+  fft_staged<M, E, false, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
+  if constexpr (EARLY) r2c_post_w<M, E, W>(v, sb, t, wk);
+  else r2c_post<M, E, W>(v, sb, t, a.twx);
+  pdl_trigger();
+  if constexpr (RF) {
+    if (__syncthreads_or(!mbar_wait(&bar[2], 0, WF_WAIT_TRIES))) {
+      drain();
+      if (!mbar_wait(&bar[2], 0, WF_WAIT_TRIES) || threadIdx.x == 0) atomicOr(&a.st->err, WF_ERR_TIMEOUT);
+      return;
+    }
     // eqs. (2mess_d0), (2mess_t0) analogues in the stripe basis
+    const size_t row0 = (size_t)y * M;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const int k = t + m * TPF;
-      const float2 t1o = s_t1[g * M + k];
-      const float2 xo = s_x[g * M + k];
+      const int k = t + m * TPF, i = SM::tpos(g, k);
+      const float2 t1o = s_t1[i];
+      const float2 xo = s_x[i];
       const float2 t2 = v[m];
+      const float pv = EARLY ? pk[EARLY ? m : 0] : __ldg(&a.pst[k]);
       float2 d1, t1;
-      stripe_update(k, t2, t1o, xo, a2y, pk[m], pkn, off1, T2, T1, d1, t1);
+      stripe_update(k, t2, t1o, xo, a2y, pv, pkn, off1, T2, T1, d1, t1);
       a.f_d1[row0 + k] = d1;
-      a.f_t1[tidx(y, k, a.ny)] = t1;
+      s_t1[i] = t1;
     }
+  } else {
+    if constexpr (!EARLY) __syncthreads();
+    else fft_sync<W>();
+#pragma unroll
+    for (int m = 0; m < E; ++m) s_t1[SM::tpos(g, t + m * TPF)] = v[m];
+  }
+  // the new messenger leaves by tensor copies
+  fence_async_smem();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < M / WF_TW; j += kBoxTiles) tma2d_s2g(&a.tm_t, y0 * 2 * WF_TW, j, s_t1 + j * ROWS * WF_TW);
+    bulk_store_wait();
   }
 }
 
@@ -377,7 +422,7 @@ static int launch_row_pass_e(const RowArgs& a, cudaStream_t s) {
                                    (int)bytes);
   });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
-  const dim3 grid((a.ny + Cfg::ROWS - 1) / Cfg::ROWS), block(Cfg::THREADS);
+  const dim3 grid(a.ny / Cfg::ROWS), block(Cfg::THREADS);
   return launch_pdl(row_pass_kernel<M, MODE, EV>, grid, block, bytes, s, a);
 }
 
@@ -443,6 +488,29 @@ int row_grid(int nx, int ny) {
     default: r = 1;
   }
   return (ny + r - 1) / r;
+}
+
+template <int M>
+static int row_rows(int v) {
+  return v == 1 ? RowPassCfg<M, RowPassE<M>::v1>::ROWS : RowPassCfg<M, RowPassE<M>::v0>::ROWS;
+}
+
+// rows per CTA of the row pass
+int row_pass_rows(int M, int v) {
+  switch (M) {
+    case 16: return row_rows<16>(v);
+    case 32: return row_rows<32>(v);
+    case 64: return row_rows<64>(v);
+    case 128: return row_rows<128>(v);
+    case 192: return row_rows<192>(v);
+    case 256: return row_rows<256>(v);
+    case 384: return row_rows<384>(v);
+    case 512: return row_rows<512>(v);
+    case 768: return row_rows<768>(v);
+    case 1024: return row_rows<1024>(v);
+    case 2048: return row_rows<2048>(v);
+    default: return 0;
+  }
 }
 
 template <int M>
