@@ -86,6 +86,7 @@ struct wf_plan_s {
   bool tuned = false;
   // the row pass's tensor maps of the column-tiled fields, per shape
   CUtensorMap tm_t[2], tm_x[2];
+  int sms = 0;              // SMs the passes' CTAs are spread over (0: other plans run beside this one)
   // the column pass hints the next wave's tiles into L2 (maps whose sweep
   // moves more bytes than L2 holds)
   bool l2_prefetch = false;
@@ -419,6 +420,12 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
         !tile_map(&P->tm_x[v], P->f_x, ny, P->M, rows))
       rc = WF_ECUDA;
   }
+  int dev = 0;
+  if (rc == WF_OK && (cudaGetDevice(&dev) != cudaSuccess ||
+                      cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)) {
+    cudaGetLastError();
+    rc = WF_ECUDA;
+  }
   if (rc != WF_OK) {
     wf_plan_destroy(P);
     return rc;
@@ -469,6 +476,7 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
 static RowArgs row_args(wf_plan_s* P) {
   RowArgs a{};
   a.variant = P->row_variant;
+  a.sms = P->sms;
   a.tm_t = P->tm_t[P->row_variant];
   a.tm_x = P->tm_x[P->row_variant];
   a.ny = P->ny;
@@ -496,6 +504,7 @@ static ColArgs col_args(wf_plan_s* P, int parity) {
   a.prec = P->p.dft_precision;
   a.variant = a.prec ? 0 : P->col_variant;  // the tensor-core stages use the 16-value shape
   a.prefetch = P->l2_prefetch;
+  a.sms = P->sms;
   a.ny = P->ny;
   a.nx = P->nx;
   a.has_rf = P->has_rf;
@@ -886,6 +895,7 @@ bool wf::plan_batch_ok(const wf_plan_t P) {
 }
 
 int wf::plan_size(const wf_plan_t P) { return P->ny; }
+void wf::plan_shares_gpu(wf_plan_t P) { P->sms = 0; }
 int wf::plan_autotune(const wf_plan_t P) { return P->p.autotune; }
 
 // Runs the iteration of several loaded plans together (wf_run for each, with
@@ -1122,7 +1132,8 @@ static int run_setup(wf_plan_t P, const wf_schedule* sch, double tol, CtrlArgs* 
         !(sch->snap >= 1.0))
       return WF_EINVAL;
     c.mode = 1;
-    c.ratio = sch->ratio;
+    c.rate_lo = sch->ratio < 1.0 ? pow(1.0 - sch->ratio, R) : 0.0;
+    c.rate_hi = pow(1.0 + sch->ratio, R);
     c.expo = sch->expo;
     c.snap = sch->snap;
     lam0 = sch->lam0;
@@ -1183,7 +1194,7 @@ static int wf_run_on(wf_plan_t P, const wf_schedule* sch, double tol, wf_stats* 
     key.insert(key.end(), b, b + n);
   };
   const long long par = it0 & 1, src = P->has_src ? 1 : 0;
-  put(&c.tol, 8); put(&c.tol_u, 8); put(&c.ratio, 8); put(&c.expo, 8); put(&c.snap, 8);
+  put(&c.tol, 8); put(&c.tol_u, 8); put(&c.rate_lo, 8); put(&c.rate_hi, 8); put(&c.expo, 8); put(&c.snap, 8);
   put(&c.mode, 4); put(&c.nlevels, 4); put(&c.R, 4); put(&c.max_iters, 4); put(&c.count_iters, 4);
   put(&c.skip_fixed, 4);
   put(&par, 8); put(&src, 8);

@@ -32,6 +32,7 @@
 #include <mutex>
 #include <numeric>
 #include <thread>
+
 #include <vector>
 
 #include "../../include/wf.h"
@@ -320,6 +321,7 @@ int wf_batch_create(wf_batch_t* out, int nmaps, const int* ny, const int* nx, un
         destroy(B);
         return rc;
       }
+      if (B->lanes > 1 && nmaps > 1) wf::plan_shares_gpu(B->plans[i]);
     }
   }
   if (!ok) {

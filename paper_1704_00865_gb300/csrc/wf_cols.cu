@@ -11,6 +11,8 @@
 // Column 0 packs the two real-signal columns kx = 0 and kx = nx/2 as
 // Z = A + i B (see wf_cols_common.cuh), treated as separate modes with their
 // own eigenvalues.
+#include <mutex>
+
 #include "wf_cols_common.cuh"
 
 namespace wf {
@@ -19,8 +21,9 @@ template <int L>
 struct ColCfg {
   static constexpr int E = (L % 3 == 0) ? 12 : ((L >= 2048) ? 16 : 8);
   static constexpr int TPC = L / E;
-  static constexpr int W0 = 256 / TPC;
-  static constexpr int W = W0 < 1 ? 1 : (W0 > 32 ? 32 : W0);
+  // whole tiles, 32-byte pieces of the row-major fields (half of that at 4096,
+  // where four columns would not fit)
+  static constexpr int W = TPC < 16 ? 64 / TPC : (L >= 4096 ? 2 : WF_TW);
   static constexpr int THREADS = W * TPC;
   // Stride between the per-column FFT buffers (complex values): a half-warp
   // covers W columns x 16/W consecutive indices, which are bank-conflict free
@@ -28,16 +31,22 @@ struct ColCfg {
   static constexpr int SP = SPad<L>::size;
   static constexpr int WANT = (W >= 32) ? 1 : (16 / W) % 16;
   static constexpr int STRIDE = SP + ((WANT - SP % 16) + 16) % 16;
+  static constexpr size_t bytes = (size_t)W * STRIDE * 8;
 };
 
+// the plain transforms are held to 64 registers a thread, so that two CTAs of
+// long columns share an SM
 template <int L, int MODE>
-__global__ void __launch_bounds__(ColCfg<L>::THREADS)
+constexpr int col_min_ctas() {
+  return (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED) && L >= 1024 ? 1024 / ColCfg<L>::THREADS : 1;
+}
+
+template <int L, int MODE>
+__global__ void __launch_bounds__(ColCfg<L>::THREADS, col_min_ctas<L, MODE>())
 col_kernel(ColArgs a) {
   using Cfg = ColCfg<L>;
   constexpr int E = Cfg::E, TPC = Cfg::TPC, W = Cfg::W;
-  __shared__ float2 sbuf[W][Cfg::STRIDE];
-  pdl_trigger();
-  pdl_wait();
+  extern __shared__ __align__(16) float2 sbuf[];  // [W][STRIDE]
 
   const int c = threadIdx.x % W;
   const int t = threadIdx.x / W;
@@ -45,11 +54,23 @@ col_kernel(ColArgs a) {
   const int col = blockIdx.x * W + c;
   const bool valid = col < ncols;
   const int colv = valid ? col : 0;
-  float2* sb = sbuf[c];
+  float2* sb = sbuf + c * Cfg::STRIDE;
 
+  pdl_trigger();
+  // the eigenvalues, fixed during a solve, while the previous kernel drains
+  constexpr bool EIG = (MODE == COL_RESID_A || MODE == COL_RESID_C || MODE == COL_G_FROM_S), PRE = EIG && E <= 12;
+  float2 eg0[PRE ? E : 1];
+  if constexpr (PRE) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) eg0[m] = valid ? __ldg(&a.eig[tidx(t + m * TPC, colv, a.ny)]) : make_float2(1.f, 0.f);
+  }
+  pdl_wait();
   // uniform: both flags are set only between launches
   if ((a.check_done && a.st->done) || (a.skip_ok && a.st->skip_resid)) return;
 
+  auto eig_at = [&](int m) -> float2 {
+    return PRE ? eg0[PRE ? m : 0] : (valid ? a.eig[tidx(t + m * TPC, colv, a.ny)] : make_float2(1.f, 0.f));
+  };
   auto at = [&](int k) -> size_t { return (size_t)k * ncols + colv; };       // row-major
   auto att = [&](int k) -> size_t { return tidx(k, colv, a.ny); };           // column-tiled
   float2 v[E];
@@ -89,7 +110,7 @@ col_kernel(ColArgs a) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
         const int k = t + m * TPC;
-        const float2 eg = valid ? a.eig[att(k)] : make_float2(1.f, 1.f);
+        const float2 eg = eig_at(m);
         // with a source j: g = (y + (N0 + T) j^) / (C + N0 + T)
         const float2 jv = (a.src != nullptr && valid) ? a.src[att(k)] : make_float2(0.f, 0.f);
         if (blockIdx.x == 0 && c == 0) {
@@ -128,7 +149,7 @@ col_kernel(ColArgs a) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
         const int k = t + m * TPC;
-        const float2 eg = valid ? a.eig[att(k)] : make_float2(1.f, 1.f);
+        const float2 eg = eig_at(m);
         if (blockIdx.x == 0 && c == 0) {
           const int kp = neg_mod<L>(k);
           const float2 egb = a.eig_nyq[k];
@@ -164,7 +185,7 @@ col_kernel(ColArgs a) {
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const int k = t + m * TPC;
-      const float2 eg = valid ? a.eig[att(k)] : make_float2(0.f, 0.f);
+      const float2 eg = eig_at(m);
       if (blockIdx.x == 0 && c == 0) {
         float2 A, B;
         unpack_pair(v[m], vp[m], A, B);
@@ -193,7 +214,7 @@ col_kernel(ColArgs a) {
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const int k = t + m * TPC;
-      const float2 eg = valid ? a.eig[att(k)] : make_float2(1.f, 1.f);
+      const float2 eg = eig_at(m);
       if (blockIdx.x == 0 && c == 0) {
         float2 A, B;
         unpack_pair(v[m], vp[m], A, B);
@@ -265,24 +286,35 @@ col_kernel(ColArgs a) {
   }
 }
 
+template <int L, int MODE>
+static int launch_col_kernel(const ColArgs& a, cudaStream_t s) {
+  using Cfg = ColCfg<L>;
+  // once per instantiation and process (plans may run on several host threads)
+  static std::once_flag once;
+  static cudaError_t cfg_err = cudaSuccess;
+  std::call_once(once, [] {
+    cfg_err = cudaFuncSetAttribute(col_kernel<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes);
+  });
+  if (cfg_err != cudaSuccess) return (int)cfg_err;
+  const dim3 grid((a.nx / 2 + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);
+  return launch_pdl(col_kernel<L, MODE>, grid, block, Cfg::bytes, s, a);
+}
+
 template <int L>
 static int launch_col_L(int mode, const ColArgs& a, cudaStream_t s) {
-  using Cfg = ColCfg<L>;
-  const int ncols = a.nx / 2;
-  const dim3 grid((ncols + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);
   switch (mode) {
     case COL_PASS_2DF:
     case COL_PASS_NO2DF:
     case COL_PASS_MERGE:
     case COL_PASS_MERGE_SRC: return launch_col_pass_any<L>(mode, a, s);
-    case COL_RESID_A: return launch_pdl(col_kernel<L, COL_RESID_A>, grid, block, 0, s, a);
-    case COL_RESID_C: return launch_pdl(col_kernel<L, COL_RESID_C>, grid, block, 0, s, a);
-    case COL_FWD: return launch_pdl(col_kernel<L, COL_FWD>, grid, block, 0, s, a);
-    case COL_INV: return launch_pdl(col_kernel<L, COL_INV>, grid, block, 0, s, a);
-    case COL_G_FROM_S: return launch_pdl(col_kernel<L, COL_G_FROM_S>, grid, block, 0, s, a);
-    case COL_UNTILE: return launch_pdl(col_kernel<L, COL_UNTILE>, grid, block, 0, s, a);
-    case COL_FWD_TILED: return launch_pdl(col_kernel<L, COL_FWD_TILED>, grid, block, 0, s, a);
-    case COL_WARM: return launch_pdl(col_kernel<L, COL_WARM>, grid, block, 0, s, a);
+    case COL_RESID_A: return launch_col_kernel<L, COL_RESID_A>(a, s);
+    case COL_RESID_C: return launch_col_kernel<L, COL_RESID_C>(a, s);
+    case COL_FWD: return launch_col_kernel<L, COL_FWD>(a, s);
+    case COL_INV: return launch_col_kernel<L, COL_INV>(a, s);
+    case COL_G_FROM_S: return launch_col_kernel<L, COL_G_FROM_S>(a, s);
+    case COL_UNTILE: return launch_col_kernel<L, COL_UNTILE>(a, s);
+    case COL_FWD_TILED: return launch_col_kernel<L, COL_FWD_TILED>(a, s);
+    case COL_WARM: return launch_col_kernel<L, COL_WARM>(a, s);
     default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();

@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(CTRL_THREADS) ctrl_kernel(CtrlArgs a) {
   // the residual kernels of this checkpoint returned at once (uniform: the
   // flag changes below only after every thread has read it)
   const bool skipped = a.count_iters && st->skip_resid;
+  const WfState c = *st;  // all fields at once, while the sums are loaded
   __syncthreads();
   double gm2 = 0.0, g2 = 0.0, r2 = 0.0;
   if (!skipped) {
@@ -327,85 +328,95 @@ __global__ void __launch_bounds__(CTRL_THREADS) ctrl_kernel(CtrlArgs a) {
     r2 = block_add<CTRL_THREADS>(r2, red);
   }
   if (threadIdx.x != 0) return;
+  double rel_u = c.rel_u, rel_m = c.rel_m;
   if (!skipped) {
+    rel_u = c.du2 > 0 ? sqrt(r2 / c.du2) : 0.0;
+    rel_m = g2 > 0 ? sqrt(gm2 / g2) : 0.0;
     st->gm2 = gm2;
     st->g2 = g2;
     st->rho2 = r2;
-    st->rel_u = st->du2 > 0 ? sqrt(r2 / st->du2) : 0.0;
-    st->rel_m = g2 > 0 ? sqrt(gm2 / g2) : 0.0;
+    st->rel_u = rel_u;
+    st->rel_m = rel_m;
   }
   if (!a.count_iters) return;  // residual only
-  st->iter += a.R;
-  st->in_level += a.R;
-  st->checkpoints += 1;
+  const int iter = c.iter + a.R, in_level = c.in_level + a.R;
+  st->iter = iter;
+  st->in_level = in_level;
+  st->checkpoints = c.checkpoints + 1;
   if (a.trace != nullptr) {
     // one record per checkpoint: sweeps, the lambda they ran at, the
     // residual terms, chi^2_aug, the run
     const int i = *a.trace_n;
     if (i < a.trace_cap) {
       double* r = a.trace + (size_t)WF_TRACE_FIELDS * i;
-      r[0] = (double)st->iter;
-      r[1] = st->lam;
-      r[2] = skipped ? nan("") : st->rel_u;
-      r[3] = skipped ? nan("") : st->rel_m;
+      r[0] = (double)iter;
+      r[1] = c.lam;
+      r[2] = skipped ? nan("") : rel_u;
+      r[3] = skipped ? nan("") : rel_m;
       r[4] = a.chi_val != nullptr ? *a.chi_val : nan("");
       r[5] = (double)a.run_index;
       *a.trace_n = i + 1;
     }
   }
-  if (!skipped && a.tol > 0 && st->lam == 1.0 && st->rel_u <= a.tol_u && st->rel_m <= a.tol) {
+  if (!skipped && a.tol > 0 && c.lam == 1.0 && rel_u <= a.tol_u && rel_m <= a.tol) {
     st->done = 1;
     st->status = 0;
     return;
   }
-  if (st->iter >= a.max_iters) {
+  if (iter >= a.max_iters) {
     st->done = 1;
     st->status = a.tol > 0 ? 3 : 0;  // WF_ENOCONV
     return;
   }
   // stagnation at lambda = 1: an FP32 iteration stops improving once the
   // slow links move their fields by less than one unit in the last place
-  if (a.stall > 0 && a.tol > 0 && st->lam == 1.0) {
-    if (st->stall_ref <= 0.0 || r2 < 0.99 * st->stall_ref) {
+  if (a.stall > 0 && a.tol > 0 && c.lam == 1.0) {
+    if (c.stall_ref <= 0.0 || r2 < 0.99 * c.stall_ref) {
       st->stall_ref = r2;
       st->stall_n = 0;
-    } else if (++st->stall_n >= a.stall) {
-      st->done = 1;
-      st->status = 4;  // WF_ESTALL
-      return;
+    } else {
+      st->stall_n = c.stall_n + 1;
+      if (c.stall_n + 1 >= a.stall) {
+        st->done = 1;
+        st->status = 4;  // WF_ESTALL
+        return;
+      }
     }
   }
+  auto move_to = [&](double lam) {
+    st->lam = lam;
+    st->in_level = 0;
+    st->stall_ref = -1.0;
+    st->stall_n = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) st->Tf[i] = (float)(lam * c.tau[i]);
+  };
   if (a.mode == 0) {
-    if (st->level < a.nlevels - 1 && st->in_level >= a.it_sched[st->level]) {
-      st->level += 1;
-      st->lam = a.lam_sched[st->level];
-      st->in_level = 0;
-      st->stall_ref = -1.0;
-      st->stall_n = 0;
-      set_T(st);
+    double lam = c.lam;
+    if (c.level < a.nlevels - 1 && in_level >= a.it_sched[c.level]) {
+      lam = a.lam_sched[c.level + 1];
+      st->level = c.level + 1;
+      move_to(lam);
     }
     // a fixed schedule uses the residual only at lambda = 1 (stop and stall
     // tests) and at the checkpoint that ends the run (the reported values):
     // the next checkpoint skips it otherwise
-    st->skip_resid = (a.skip_fixed && st->lam > 1.0 && st->iter + a.R < a.max_iters) ? 1 : 0;
-  } else if (st->lam > 1.0) {
+    st->skip_resid = (a.skip_fixed && lam > 1.0 && iter + a.R < a.max_iters) ? 1 : 0;
+  } else if (c.lam > 1.0) {
     // Sec. 3.3: lower lambda once Delta d^T Delta d changes by less than
-    // `ratio` per iteration
-    if (st->prev_rho2 > 0 && r2 > 0) {
-      const double rate = fabs(1.0 - pow(r2 / st->prev_rho2, 1.0 / a.R));
-      if (rate < a.ratio) {
-        double lam = pow(st->lam, a.expo);
+    // `ratio` per iteration, |1 - q^(1/R)| < ratio for q = rho2 / prev_rho2,
+    // i.e. q between (1 - ratio)^R and (1 + ratio)^R
+    double prev = r2;
+    if (c.prev_rho2 > 0 && r2 > 0) {
+      const double q = r2 / c.prev_rho2;
+      if (q > a.rate_lo && q < a.rate_hi) {
+        double lam = pow(c.lam, a.expo);
         if (lam < a.snap) lam = 1.0;
-        st->lam = lam;
-        st->in_level = 0;
-        st->prev_rho2 = -1.0;
-        st->stall_ref = -1.0;
-        st->stall_n = 0;
-        set_T(st);
-        return;
+        move_to(lam);
+        prev = -1.0;
       }
     }
-    st->prev_rho2 = r2;
+    st->prev_rho2 = prev;
   }
 }
 

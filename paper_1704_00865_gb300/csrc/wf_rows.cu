@@ -20,7 +20,10 @@ template <int M>
 struct RowCfg {
   static constexpr int E = (M % 3 == 0) ? 12 : ((M >= 2048) ? 16 : 8);
   static constexpr int TPF = M / E;
-  static constexpr int ROWS = (256 / TPF) >= 1 ? (256 / TPF) : 1;
+  // one row per CTA, or as many as a warp holds: a 512 x 384 map gives 256 CTAs
+  // (with 256 threads each it gave 32 and the residual's row steps took 27
+  // and 15 us there)
+  static constexpr int ROWS = TPF >= 32 ? 1 : 32 / TPF;
   static constexpr int THREADS = ROWS * TPF;
 };
 
@@ -48,8 +51,6 @@ row_kernel(RowArgs a) {
   constexpr int E = Cfg::E, TPF = Cfg::TPF, ROWS = Cfg::ROWS;
   __shared__ float2 sbuf[ROWS][SPad<M>::size];
   __shared__ double red[(Cfg::THREADS + 31) / 32];
-  pdl_trigger();
-  pdl_wait();
 
   const int g = threadIdx.x / TPF;
   const int t = threadIdx.x - g * TPF;
@@ -57,6 +58,15 @@ row_kernel(RowArgs a) {
   const bool valid = y < a.ny;
   const size_t row0 = (size_t)(valid ? y : 0) * M;
   float2* sb = sbuf[g];
+  pdl_trigger();
+  // the pixel table, fixed during a solve, while the previous kernel drains
+  constexpr bool PX = (MODE == ROW_RESID_B || MODE == ROW_RESID_D), PRE = PX && E <= 12;
+  float4 px[PRE ? E : 1];
+  if constexpr (PRE) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) px[m] = valid ? __ldg(&a.dn[row0 + t + m * TPF]) : make_float4(0.f, -1.f, 0.f, -1.f);
+  }
+  pdl_wait();
 
   // uniform: both flags are set only between launches
   if ((a.check_done && a.st->done) || (a.skip_ok && a.st->skip_resid)) return;
@@ -79,7 +89,7 @@ row_kernel(RowArgs a) {
     double gm2 = 0.0, g2 = 0.0;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const float4 q = valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f);
+      const float4 q = PRE ? px[PRE ? m : 0] : (valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f));
       const float2 jm = (valid && a.src_px != nullptr) ? a.src_px[row0 + t + m * TPF] : make_float2(0.f, 0.f);
       float gp[2], qp[2], go[2];
       const float gv[2] = {v[m].x, v[m].y}, sv[2] = {w[m].x, w[m].y};
@@ -141,7 +151,7 @@ row_kernel(RowArgs a) {
     double r2 = 0.0;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const float4 q = valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f);
+      const float4 q = PRE ? px[PRE ? m : 0] : (valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f));
       if (valid) {
         if (q.y >= 0.f) r2 += (double)v[m].x * (double)v[m].x;
         if (q.w >= 0.f) r2 += (double)v[m].y * (double)v[m].y;
@@ -419,11 +429,11 @@ static int launch_row_pass_e(const RowArgs& a, cudaStream_t s) {
   static cudaError_t cfg_err = cudaSuccess;
   std::call_once(once, [] {
     cfg_err = cudaFuncSetAttribute(row_pass_kernel<M, MODE, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)bytes);
+                                   (int)(bytes > kSpreadSmem ? bytes : kSpreadSmem));
   });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid(a.ny / Cfg::ROWS), block(Cfg::THREADS);
-  return launch_pdl(row_pass_kernel<M, MODE, EV>, grid, block, bytes, s, a);
+  return launch_pdl(row_pass_kernel<M, MODE, EV>, grid, block, spread_smem(grid.x, bytes, a.sms), s, a);
 }
 
 // a.variant selects the shape (0 or 1, RowPassE)
