@@ -73,60 +73,74 @@ __global__ void __launch_bounds__(kThreads) aa_dots_kernel(AADots a, size_t n4, 
 
 // The partials of all blocks summed in a fixed order -- warp j sums dot j,
 // lane k the partials of blocks k, k + 32, ..., then a shuffle tree -- and,
-// by one thread, the least-squares step: row and column `slot` of the Gram
+// by one warp, the least-squares step: row and column `slot` of the Gram
 // matrix G = Delta F^T Delta F (held in device memory across corrections)
 // take the new products, and (G + eps diag) gamma = Delta F^T f is solved by
 // Cholesky in FP64.  A column whose pivot falls below 1e-10 of the largest
-// diagonal (dependent on the others to FP32 accuracy) gets gamma = 0.
+// diagonal (dependent on the others to FP32 accuracy) gets gamma = 0.  Lane r
+// has row r, everything is in shared memory: the chain is one square root,
+// one division and one short sum per column.
 constexpr int kSolveThreads = 2 * WF_AA_MAX * 32;
 __global__ void __launch_bounds__(kSolveThreads) aa_solve_kernel(const double* part, int nblocks, int slot, int n,
                                                                  double* G, float* gamma) {
   __shared__ double dots[2 * WF_AA_MAX];
-  __shared__ double L[WF_AA_MAX][WF_AA_MAX];
+  __shared__ double L[WF_AA_MAX][WF_AA_MAX + 1];
+  __shared__ double A[WF_AA_MAX][WF_AA_MAX + 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < WF_AA_MAX * WF_AA_MAX) A[threadIdx.x / WF_AA_MAX][threadIdx.x % WF_AA_MAX] = G[threadIdx.x];
   double v = 0.0;
   for (int b = lane; b < nblocks; b += 32) v += part[(size_t)b * 2 * WF_AA_MAX + w];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   if (lane == 0) dots[w] = v;
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int k = 0; k < n; ++k) G[slot * WF_AA_MAX + k] = G[k * WF_AA_MAX + slot] = dots[k];
-  bool use[WF_AA_MAX];
-  double g[WF_AA_MAX], y[WF_AA_MAX];
-  double dmax = 0.0;
-  for (int i = 0; i < n; ++i) dmax = fmax(dmax, G[i * WF_AA_MAX + i]);
-  for (int i = 0; i < n; ++i) {
-    use[i] = false;
-    g[i] = y[i] = 0.0;
-    if (!(dmax > 0.0)) continue;
-    double d = G[i * WF_AA_MAX + i] * (1.0 + 1e-12);
-    for (int k = 0; k < i; ++k)
-      if (use[k]) d -= L[i][k] * L[i][k];
-    if (!(d > 1e-10 * dmax)) continue;
-    use[i] = true;
-    L[i][i] = sqrt(d);
-    for (int r = i + 1; r < n; ++r) {
-      double x = G[r * WF_AA_MAX + i];
-      for (int k = 0; k < i; ++k)
-        if (use[k]) x -= L[r][k] * L[i][k];
-      L[r][i] = x / L[i][i];
+  if (w != 0) return;
+  if (lane < n) {
+    A[slot][lane] = dots[lane];
+    G[slot * WF_AA_MAX + lane] = dots[lane];
+    if (lane != slot) {
+      A[lane][slot] = dots[lane];
+      G[lane * WF_AA_MAX + slot] = dots[lane];
     }
   }
+  __syncwarp();
+  unsigned use = 0;  // columns with a pivot (the same in every lane)
+  double dmax = 0.0;
+  for (int i = 0; i < n; ++i) dmax = fmax(dmax, A[i][i]);
+  const int r = lane;
   for (int i = 0; i < n; ++i) {
-    if (!use[i]) continue;
-    double x = dots[WF_AA_MAX + i];
+    if (!(dmax > 0.0)) break;
+    double d = A[i][i] * (1.0 + 1e-12);
     for (int k = 0; k < i; ++k)
-      if (use[k]) x -= L[i][k] * y[k];
-    y[i] = x / L[i][i];
+      if (use >> k & 1u) d -= L[i][k] * L[i][k];
+    if (!(d > 1e-10 * dmax)) continue;
+    use |= 1u << i;
+    const double p = sqrt(d);
+    __syncwarp();
+    if (r == i) L[i][i] = p;
+    if (r > i && r < n) {
+      double x = A[r][i];
+      for (int k = 0; k < i; ++k)
+        if (use >> k & 1u) x -= L[r][k] * L[i][k];
+      L[r][i] = x / p;
+    }
+    __syncwarp();
+  }
+  // forward and back substitution, column by column: lane r keeps its own
+  // right-hand side, the terms are subtracted in the order of the columns
+  double x = r < n ? dots[WF_AA_MAX + r] : 0.0, g = 0.0;
+  for (int i = 0; i < n; ++i) {
+    if (!(use >> i & 1u)) continue;
+    if (r == i) x = x / L[i][i];
+    const double y = __shfl_sync(0xffffffffu, x, i);
+    if (r > i && r < n) x -= L[r][i] * y;
   }
   for (int i = n - 1; i >= 0; --i) {
-    if (!use[i]) continue;
-    double x = y[i];
-    for (int k = i + 1; k < n; ++k)
-      if (use[k]) x -= L[k][i] * g[k];
-    g[i] = x / L[i][i];
+    if (!(use >> i & 1u)) continue;
+    if (r == i) g = x / L[i][i];
+    const double gi = __shfl_sync(0xffffffffu, g, i);
+    if (r < i) x -= L[i][r] * gi;
   }
-  for (int i = 0; i < WF_AA_MAX; ++i) gamma[i] = i < n ? (float)g[i] : 0.f;
+  if (lane < WF_AA_MAX) gamma[lane] = lane < n && (use >> lane & 1u) ? (float)g : 0.f;
 }
 
 // u = f - sum_j gamma_j (dx_j + df_j); x += u

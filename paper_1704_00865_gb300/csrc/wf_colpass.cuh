@@ -227,44 +227,64 @@ col_pass_kernel(ColArgs a) {
     else if constexpr (Cfg::SRC) return __ldg(&a.src[at0 + (size_t)k * WF_TW]);
     else return a.f_t0[(size_t)k * ncols + col];
   };
-  // partners of t_2DF are overwritten below: read them first
-  float2 tp[Cfg::T0 ? E : 1];
-  if constexpr (Cfg::T0 && !STAGED) {
-    if (blockIdx.x == 0) {
+  auto eig_of = [&](int k) -> float2 {
+    return STAGED ? s_eig[Cfg::sidx(k, c)] : __ldg(&a.eig[at0 + (size_t)k * WF_TW]);
+  };
+  if (blockIdx.x != 0) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int k = t + m * TPC;
+      const float2 e = eig_of(k);
+      if constexpr (MERGED) {
+        const float2 jv = Cfg::SRC ? third(k) : make_float2(0.f, 0.f);
+        v[m] = merged_mode<Cfg::SRC>(v[m], v[m], e, e, off0, Tl, false, jv, jv);
+      } else {
+        float2 t0n;
+        v[m] = mode_2df(v[m], third(k), e.x, e.y, off0, Tl, T0, T0s, t0n);
+        a.f_t0[(size_t)k * ncols + col] = t0n;
+      }
+    }
+  } else {
+    // the CTA of the packed column.  Partners of t_2DF are overwritten below:
+    // read them first
+    float2 tp[Cfg::T0 ? E : 1];
+    if constexpr (Cfg::T0 && !STAGED) {
       if (packed)
 #pragma unroll
         for (int m = 0; m < E; ++m) tp[m] = third(neg_mod<L>(t + m * TPC));
       __syncthreads();
     }
-  }
 #pragma unroll
-  for (int m = 0; m < E; ++m) {
-    const int k = t + m * TPC;
-    const float2 e = STAGED ? s_eig[Cfg::sidx(k, c)] : __ldg(&a.eig[at0 + (size_t)k * WF_TW]);
-    const float2 egn = packed ? (STAGED ? eq[STAGED ? m : 0] : __ldg(&a.eig_nyq[k])) : e;
-    const float2 vp = packed ? sb[spad(neg_mod<L>(k))] : v[m];
-    if constexpr (MERGED) {
-      constexpr bool SRC = Cfg::SRC;
-      const float2 jv = SRC ? third(k) : make_float2(0.f, 0.f);
-      const float2 jp = SRC ? (packed ? third(neg_mod<L>(k)) : jv) : make_float2(0.f, 0.f);
-      if (blockIdx.x == 0) v[m] = merged_pair<SRC>(v[m], vp, e, egn, off0, Tl, jv, jp);
-      else v[m] = merged_mode<SRC>(v[m], vp, e, egn, off0, Tl, false, jv, jp);
-    } else {
-      const float2 t0o = third(k);
-      float2 t0n, d0;
-      if (packed) {
-        float2 yA, yB, tA, tB, tnA, tnB;
-        unpack_pair(v[m], vp, yA, yB);
-        unpack_pair(t0o, STAGED ? third(neg_mod<L>(k)) : tp[Cfg::T0 ? m : 0], tA, tB);
-        const float2 dA = mode_2df(yA, tA, e.x, e.y, off0, Tl, T0, T0s, tnA);
-        const float2 dB = mode_2df(yB, tB, egn.x, egn.y, off0, Tl, T0, T0s, tnB);
-        d0 = repack_pair(dA, dB);
-        t0n = repack_pair(tnA, tnB);
+    for (int m = 0; m < E; ++m) {
+      const int k = t + m * TPC;
+      const float2 e = eig_of(k);
+      // (C, P1f) at kx = nx/2 for the packed column
+      const float2 egn = packed ? (STAGED ? eq[STAGED ? m : 0] : __ldg(&a.eig_nyq[k])) : e;
+      const float2 zp = sb[spad(neg_mod<L>(k))];
+      const float2 vp = make_float2(packed ? zp.x : v[m].x, packed ? zp.y : v[m].y);
+      if constexpr (MERGED) {
+        constexpr bool SRC = Cfg::SRC;
+        const float2 jv = SRC ? third(k) : make_float2(0.f, 0.f);
+        const float2 jn = SRC ? third(neg_mod<L>(k)) : jv;
+        const float2 jp = make_float2(packed ? jn.x : jv.x, packed ? jn.y : jv.y);
+        v[m] = merged_pair<SRC>(v[m], vp, e, egn, off0, Tl, jv, jp);
       } else {
-        d0 = mode_2df(v[m], t0o, e.x, e.y, off0, Tl, T0, T0s, t0n);
+        const float2 t0o = third(k);
+        float2 t0n, d0;
+        if (packed) {
+          float2 yA, yB, tA, tB, tnA, tnB;
+          unpack_pair(v[m], vp, yA, yB);
+          unpack_pair(t0o, STAGED ? third(neg_mod<L>(k)) : tp[Cfg::T0 ? m : 0], tA, tB);
+          const float2 dA = mode_2df(yA, tA, e.x, e.y, off0, Tl, T0, T0s, tnA);
+          const float2 dB = mode_2df(yB, tB, egn.x, egn.y, off0, Tl, T0, T0s, tnB);
+          d0 = repack_pair(dA, dB);
+          t0n = repack_pair(tnA, tnB);
+        } else {
+          d0 = mode_2df(v[m], t0o, e.x, e.y, off0, Tl, T0, T0s, t0n);
+        }
+        v[m] = d0;
+        a.f_t0[(size_t)k * ncols + col] = t0n;
       }
-      v[m] = d0;
-      a.f_t0[(size_t)k * ncols + col] = t0n;
     }
   }
   if constexpr (Cfg::T0) {

@@ -798,106 +798,74 @@ __device__ __forceinline__ void load_rtw(float2 (&wk)[E], int t, const float2* _
 // z[n] = x[2n] + i x[2n+1].  The packed half spectrum holds X[k] at k = 1..M-1
 // and (X[0], X[M]) -- both real -- as the pair in slot 0.
 
-// Before an inverse complex FFT: X (natural layout in v) -> Z so that
-// IFFT_M(Z) / M gives z.  Here the 1/N scaling of the inverse real DFT is
-// folded in.  twx = exp(-2 pi i k / N).
-template <int M, int E, bool WARP = false>
-__device__ __forceinline__ void c2r_pre_w(float2 (&v)[E], float2* sb, int t, const float2 (&wk)[E]) {
-  constexpr int TPF = M / E;
-  const float s = 0.5f / (float)M;
-#pragma unroll
-  for (int m = 0; m < E; ++m) sb[spad(t + m * TPF)] = v[m];
-  fft_sync<WARP>();
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
-    const int k = t + m * TPF;
-    float2 X = v[m];
-    if (k == 0) {
-      v[m] = make_float2((X.x + X.y) * s, (X.x - X.y) * s);
-    } else {
-      float2 Xm = cconj(sb[spad(M - k)]);
-      float2 Ek = cadd(X, Xm);
-      float2 Ok = cmul(csub(X, Xm), cconj(wk[m]));
-      v[m] = make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
-    }
-  }
-  fft_sync<WARP>();
+// Mode 0 is value m = 0 of thread t = 0 only.  The steps below take every mode
+// by the general formula and put mode 0 right by a select: a branch on k == 0
+// around each value would keep the loads of the next ones from overlapping
+// (the updates of 16 values then took as long as a transform).
+
+// partner index of mode k = t + m TPF: (M - k) mod M
+template <int M>
+__device__ __forceinline__ int partner(int k, int m, int t) {
+  return (m == 0 && t == 0) ? 0 : M - k;
+}
+// one mode of c2r_pre: X and its partner Xp = X[M - k], w = W_N^k
+__device__ __forceinline__ float2 c2r_mode(float2 X, float2 Xp, float2 w, float s) {
+  const float2 Xm = cconj(Xp);
+  const float2 Ek = cadd(X, Xm);
+  const float2 Ok = cmul(csub(X, Xm), cconj(w));
+  return make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
+}
+// one mode of r2c_post
+__device__ __forceinline__ float2 r2c_mode(float2 Z, float2 Zp, float2 w) {
+  const float2 Zm = cconj(Zp);
+  const float2 Ek = cscale(cadd(Z, Zm), 0.5f);
+  const float2 D = cscale(csub(Z, Zm), 0.5f);
+  return cadd(Ek, cmul(w, make_float2(D.y, -D.x)));
 }
 
-// The same with X in shared memory (at(k) gives X[k]), possibly the transform's
-// own buffer: every value and its partner are read from there, then it is free.
-template <int M, int E, bool WARP, typename At>
-__device__ __forceinline__ void c2r_pre_in(float2 (&v)[E], int t, const float2* __restrict__ twx, const At& at) {
-  constexpr int TPF = M / E;
-  const float s = 0.5f / (float)M;
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
-    const int k = t + m * TPF;
-    const float2 X = at(k);
-    if (k == 0) {
-      v[m] = make_float2((X.x + X.y) * s, (X.x - X.y) * s);
-    } else {
-      const float2 Xm = cconj(at(M - k));
-      const float2 Ek = cadd(X, Xm);
-      const float2 Ok = cmul(csub(X, Xm), cconj(__ldg(&twx[k])));
-      v[m] = make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
-    }
-  }
-  fft_sync<WARP>();
-}
-
-template <int M, int E, bool WARP = false>
-__device__ __forceinline__ void r2c_post_w(float2 (&v)[E], float2* sb, int t, const float2 (&wk)[E]) {
-  constexpr int TPF = M / E;
-#pragma unroll
-  for (int m = 0; m < E; ++m) sb[spad(t + m * TPF)] = v[m];
-  fft_sync<WARP>();
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
-    const int k = t + m * TPF;
-    float2 Z = v[m];
-    if (k == 0) {
-      v[m] = make_float2(Z.x + Z.y, Z.x - Z.y);
-    } else {
-      float2 Zm = cconj(sb[spad(M - k)]);
-      float2 Ek = cscale(cadd(Z, Zm), 0.5f);
-      float2 D = cscale(csub(Z, Zm), 0.5f);
-      float2 Ok = make_float2(D.y, -D.x);
-      v[m] = cadd(Ek, cmul(wk[m], Ok));
-    }
-  }
-  fft_sync<WARP>();
-}
-
-template <int M, int E, bool WARP = false>
-__device__ __forceinline__ void c2r_pre(float2 (&v)[E], float2* sb, int t,
-                                        const float2* __restrict__ twx) {
+// Before an inverse complex FFT: X (natural layout; at(k) gives X[k]) -> Z so
+// that IFFT_M(Z) / M gives z.  Here the 1/N scaling of the inverse real DFT is
+// folded in.  w(m, k) = W_N^k, W_N = exp(-2 pi i / N).
+template <int M, int E, typename At, typename Wk>
+__device__ __forceinline__ void c2r_pre_at(float2 (&v)[E], int t, const At& at, const Wk& w) {
   constexpr int TPF = M / E;
   const float s = 0.5f / (float)M;  // 1/(2M) = 1/N, times the 1/2 of E and O
 #pragma unroll
-  for (int m = 0; m < E; ++m) sb[spad(t + m * TPF)] = v[m];
-  fft_sync<WARP>();
-#pragma unroll
   for (int m = 0; m < E; ++m) {
     const int k = t + m * TPF;
-    float2 X = v[m];
-    if (k == 0) {
-      v[m] = make_float2((X.x + X.y) * s * 1.0f, (X.x - X.y) * s);
-    } else {
-      float2 Xm = cconj(sb[spad(M - k)]);
-      float2 Ek = cadd(X, Xm);
-      float2 Ok = cmul(csub(X, Xm), cconj(__ldg(&twx[k])));
-      // Z = E + i O
-      v[m] = make_float2((Ek.x - Ok.y) * s, (Ek.y + Ok.x) * s);
+    const float2 X = at(k), Xp = at(partner<M>(k, m, t));
+    float2 z = c2r_mode(X, Xp, w(m, k), s);
+    if (m == 0) {
+      z.x = t == 0 ? (X.x + X.y) * s : z.x;
+      z.y = t == 0 ? (X.x - X.y) * s : z.y;
     }
+    v[m] = z;
   }
-  fft_sync<WARP>();
 }
 
-// After a forward complex FFT: Z (natural layout) -> packed X.
+// The same from the registers, through the transform's buffer.
+template <int M, int E, bool WARP, typename Wk>
+__device__ __forceinline__ void c2r_pre_regs(float2 (&v)[E], float2* sb, int t, const Wk& w) {
+  constexpr int TPF = M / E;
+#pragma unroll
+  for (int m = 0; m < E; ++m) sb[spad(t + m * TPF)] = v[m];
+  fft_sync<WARP>();
+  c2r_pre_at<M, E>(v, t, [&](int k) { return sb[spad(k)]; }, w);
+  fft_sync<WARP>();
+}
 template <int M, int E, bool WARP = false>
-__device__ __forceinline__ void r2c_post(float2 (&v)[E], float2* sb, int t,
-                                         const float2* __restrict__ twx) {
+__device__ __forceinline__ void c2r_pre(float2 (&v)[E], float2* sb, int t, const float2* __restrict__ twx) {
+  c2r_pre_regs<M, E, WARP>(v, sb, t, [&](int, int k) { return __ldg(&twx[k]); });
+}
+template <int M, int E, bool WARP = false>
+__device__ __forceinline__ void c2r_pre_w(float2 (&v)[E], float2* sb, int t, const float2 (&wk)[E]) {
+  c2r_pre_regs<M, E, WARP>(v, sb, t, [&](int m, int) { return wk[m]; });
+}
+
+// After a forward complex FFT: Z (natural layout) -> packed X.  LAST: the
+// buffer is not used again before the caller's next barrier.
+template <int M, int E, bool WARP, bool LAST, typename Wk>
+__device__ __forceinline__ void r2c_post_regs(float2 (&v)[E], float2* sb, int t, const Wk& w) {
   constexpr int TPF = M / E;
 #pragma unroll
   for (int m = 0; m < E; ++m) sb[spad(t + m * TPF)] = v[m];
@@ -905,18 +873,23 @@ __device__ __forceinline__ void r2c_post(float2 (&v)[E], float2* sb, int t,
 #pragma unroll
   for (int m = 0; m < E; ++m) {
     const int k = t + m * TPF;
-    float2 Z = v[m];
-    if (k == 0) {
-      v[m] = make_float2(Z.x + Z.y, Z.x - Z.y);
-    } else {
-      float2 Zm = cconj(sb[spad(M - k)]);
-      float2 Ek = cscale(cadd(Z, Zm), 0.5f);
-      float2 D = cscale(csub(Z, Zm), 0.5f);
-      float2 Ok = make_float2(D.y, -D.x);  // D / i
-      v[m] = cadd(Ek, cmul(__ldg(&twx[k]), Ok));
+    const float2 Z = v[m];
+    float2 x = r2c_mode(Z, sb[spad(partner<M>(k, m, t))], w(m, k));
+    if (m == 0) {
+      x.x = t == 0 ? Z.x + Z.y : x.x;
+      x.y = t == 0 ? Z.x - Z.y : x.y;
     }
+    v[m] = x;
   }
-  fft_sync<WARP>();
+  if constexpr (!LAST) fft_sync<WARP>();
+}
+template <int M, int E, bool WARP = false, bool LAST = false>
+__device__ __forceinline__ void r2c_post(float2 (&v)[E], float2* sb, int t, const float2* __restrict__ twx) {
+  r2c_post_regs<M, E, WARP, LAST>(v, sb, t, [&](int, int k) { return __ldg(&twx[k]); });
+}
+template <int M, int E, bool WARP = false, bool LAST = false>
+__device__ __forceinline__ void r2c_post_w(float2 (&v)[E], float2* sb, int t, const float2 (&wk)[E]) {
+  r2c_post_regs<M, E, WARP, LAST>(v, sb, t, [&](int m, int) { return wk[m]; });
 }
 
 // ---------------------------------------------------------------- state

@@ -355,16 +355,9 @@ row_pass_kernel(const __grid_constant__ RowArgs a) {
   }
 
   float2 v[E];
-  if constexpr (EARLY) {
-#pragma unroll
-    for (int m = 0; m < E; ++m) {
-      const int k = t + m * TPF;
-      v[m] = RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)];
-    }
-    c2r_pre_w<M, E, W>(v, sb, t, wk);
-  } else {
-    c2r_pre_in<M, E, W>(v, t, a.twx, [&](int k) { return RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)]; });
-  }
+  c2r_pre_at<M, E>(v, t, [&](int k) { return RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)]; },
+                   [&](int m, int k) { return EARLY ? wk[EARLY ? m : 0] : __ldg(&a.twx[k]); });
+  if constexpr (!EARLY) fft_sync<W>();  // read before the first exchange overwrites it
   fft_staged<M, E, true, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
   // eq. (2mess_t1) analogue in pixel space, two pixels per complex value
 #pragma unroll
@@ -381,8 +374,8 @@ row_pass_kernel(const __grid_constant__ RowArgs a) {
     }
   }
   fft_staged<M, E, false, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
-  if constexpr (EARLY) r2c_post_w<M, E, W>(v, sb, t, wk);
-  else r2c_post<M, E, W>(v, sb, t, a.twx);
+  if constexpr (EARLY) r2c_post_w<M, E, W, true>(v, sb, t, wk);
+  else r2c_post<M, E, W, true>(v, sb, t, a.twx);
   pdl_trigger();
   if constexpr (RF) {
     if (__syncthreads_or(!mbar_wait(&bar[2], 0, WF_WAIT_TRIES))) {
@@ -400,7 +393,8 @@ row_pass_kernel(const __grid_constant__ RowArgs a) {
       const float2 t2 = v[m];
       const float pv = EARLY ? pk[EARLY ? m : 0] : __ldg(&a.pst[k]);
       float2 d1, t1;
-      stripe_update(k, t2, t1o, xo, a2y, pv, pkn, off1, T2, T1, d1, t1);
+      stripe_mode(t2, t1o, xo, fmaf(a2y, pv, off1), T2, T1, d1, t1);
+      if (m == 0 && t == 0) stripe_update(0, t2, t1o, xo, a2y, pv, pkn, off1, T2, T1, d1, t1);
       a.f_d1[row0 + k] = d1;
       s_t1[i] = t1;
     }

@@ -14,6 +14,16 @@ __device__ __forceinline__ float tpx_update(float d, float nb, float u, float T2
   return nb < 0.f ? u : __fdividef(fmaf(T2, d, nb * u), nb + T2);
 }
 
+// Stripe-basis updates of one row-DFT mode other than 0 (see stripe_update),
+// nb its Nbar_RF.
+__device__ __forceinline__ void stripe_mode(float2 t2, float2 t1o, float2 xo, float nb, float T2, float T1, float2& d1,
+                                            float2& t1) {
+  const float wa = __fdividef(nb, nb + T2);      // weight of t_PX
+  d1 = make_float2(fmaf(wa, t2.x - t1o.x, t1o.x), fmaf(wa, t2.y - t1o.y, t1o.y));
+  const float wb = __fdividef(nb, nb + T1);      // weight of x
+  t1 = make_float2(fmaf(wb, xo.x - d1.x, d1.x), fmaf(wb, xo.y - d1.y, d1.y));
+}
+
 // Stripe-basis updates of one row-DFT mode k (eqs. 2mess_d0 and 2mess_t0
 // analogues): d_RF between t_PX (link T_PX) and the old t_RF (link Nbar_RF),
 // then t_RF between the new d_RF (link T_RF) and the signal-side field x
@@ -30,11 +40,7 @@ __device__ __forceinline__ void stripe_update(int k, float2 t2, float2 t1o, floa
     t1.x = __fdividef(fmaf(T1, d1.x, nr * xo.x), nr + T1);
     t1.y = __fdividef(fmaf(T1, d1.y, ni * xo.y), ni + T1);
   } else {
-    const float nb = fmaf(a2y, pk, off1);
-    const float wa = __fdividef(nb, nb + T2);      // weight of t_PX
-    d1 = make_float2(fmaf(wa, t2.x - t1o.x, t1o.x), fmaf(wa, t2.y - t1o.y, t1o.y));
-    const float wb = __fdividef(nb, nb + T1);      // weight of x
-    t1 = make_float2(fmaf(wb, xo.x - d1.x, d1.x), fmaf(wb, xo.y - d1.y, d1.y));
+    stripe_mode(t2, t1o, xo, fmaf(a2y, pk, off1), T2, T1, d1, t1);
   }
 }
 
