@@ -1323,10 +1323,12 @@ int wf_get_field(wf_plan_t P, int field, float* out) {
     case WF_FIELD_T_2DF: {
       if (!P->has_f || P->merge) return WF_EINVAL;
       ColArgs ca = col_args(P, 0);
-      ca.in = P->f_t0;
+      ca.in = P->f_t0;  // column-tiled: to row-major first, then in place
       ca.out = P->r_g;
+      CKI(launch_col(COL_UNTILE, ca, P->stream));
+      ca.in = P->r_g;
       CKI(launch_col(COL_INV, ca, P->stream));
-      P->launches += 1;
+      P->launches += 2;
       ra.in_rf = P->r_g;
       break;
     }

@@ -74,18 +74,6 @@ struct ColPassCfg {
   }
 };
 
-// Row-major source (t_2DF of the plain sweep): W columns by async copies.
-template <int L, int W, int THREADS>
-__device__ __forceinline__ void tile_load_rowmajor(float2* dst, const float2* src, int col0, int ncols) {
-  constexpr int VALS = W >= 2 ? 2 : 1;
-  for (int i = threadIdx.x; i < L * W / VALS; i += THREADS) {
-    const int ky = i / (W / VALS), j = (i - ky * (W / VALS)) * VALS;
-    const float2* g = src + (size_t)ky * ncols + col0 + j;
-    if constexpr (VALS == 2) cp_async16(dst + ky * W + j, g);
-    else cp_async8(dst + ky * W + j, g);
-  }
-}
-
 // Extra shared memory of the tcgen05 stages (PREC 3, 4) after the column
 // pass's own: 1 KB of alignment slack, the A tiles (16 KB per 128 threads,
 // twice for the split), the four 4 KB DFT matrices, the mbarrier.
@@ -120,7 +108,6 @@ col_pass_kernel(ColArgs a) {
 
   const int c = threadIdx.x % W;
   const int t = threadIdx.x / W;
-  const int ncols = a.nx / 2;
   const int col0 = blockIdx.x * W;
   const int col = col0 + c;
   float2* sb = s_fft + c * Cfg::STRIDE;
@@ -170,11 +157,10 @@ col_pass_kernel(ColArgs a) {
   float2 v[E];
   if constexpr (STAGED) {
     if (threadIdx.x == 0 && !done) {
-      mbar_expect_tx(&bar[0], (uint32_t)Cfg::tile);
+      mbar_expect_tx(&bar[0], (uint32_t)Cfg::tile * (Cfg::T0 ? 2 : 1));
       bulk_g2s(s_y, a.f_y + tile0, (uint32_t)Cfg::tile, &bar[0]);
+      if constexpr (Cfg::T0) bulk_g2s(s_t0, a.f_t0 + tile0, (uint32_t)Cfg::tile, &bar[0]);
     }
-    if constexpr (Cfg::T0)
-      if (!done) tile_load_rowmajor<L, W, Cfg::THREADS>(s_t0, a.f_t0, col0, ncols);
   } else if (!done) {
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = a.f_y[at0 + (size_t)(t + m * TPC) * WF_TW];
@@ -194,7 +180,6 @@ col_pass_kernel(ColArgs a) {
     // the copies land before the block exits on every path
     bool ok = mbar_wait(&bar[1], 0, WF_WAIT_TRIES);
     if (!done) ok = mbar_wait(&bar[0], 0, WF_WAIT_TRIES) && ok;
-    cp_async_wait<0>();
     const bool bad = __syncthreads_or(!ok);
     if (bad && threadIdx.x == 0) atomicOr(&a.st->err, WF_ERR_TIMEOUT);
     if (bad || done) return;
@@ -221,11 +206,11 @@ col_pass_kernel(ColArgs a) {
     __syncthreads();
   }
 
-  // value ky of this column of the third field (t_2DF is row-major)
+  // value ky of this column of the third field (t_2DF or the source)
   auto third = [&](int k) -> float2 {
-    if constexpr (STAGED) return Cfg::SRC ? s_t0[Cfg::sidx(k, c)] : s_t0[k * W + c];
+    if constexpr (STAGED) return s_t0[Cfg::sidx(k, c)];
     else if constexpr (Cfg::SRC) return __ldg(&a.src[at0 + (size_t)k * WF_TW]);
-    else return a.f_t0[(size_t)k * ncols + col];
+    else return a.f_t0[at0 + (size_t)k * WF_TW];
   };
   auto eig_of = [&](int k) -> float2 {
     return STAGED ? s_eig[Cfg::sidx(k, c)] : __ldg(&a.eig[at0 + (size_t)k * WF_TW]);
@@ -241,7 +226,7 @@ col_pass_kernel(ColArgs a) {
       } else {
         float2 t0n;
         v[m] = mode_2df(v[m], third(k), e.x, e.y, off0, Tl, T0, T0s, t0n);
-        a.f_t0[(size_t)k * ncols + col] = t0n;
+        a.f_t0[at0 + (size_t)k * WF_TW] = t0n;
       }
     }
   } else {
@@ -249,9 +234,8 @@ col_pass_kernel(ColArgs a) {
     // read them first
     float2 tp[Cfg::T0 ? E : 1];
     if constexpr (Cfg::T0 && !STAGED) {
-      if (packed)
 #pragma unroll
-        for (int m = 0; m < E; ++m) tp[m] = third(neg_mod<L>(t + m * TPC));
+      for (int m = 0; m < E; ++m) tp[m] = third(neg_mod<L>(t + m * TPC));
       __syncthreads();
     }
 #pragma unroll
@@ -270,20 +254,20 @@ col_pass_kernel(ColArgs a) {
         v[m] = merged_pair<SRC>(v[m], vp, e, egn, off0, Tl, jv, jp);
       } else {
         const float2 t0o = third(k);
-        float2 t0n, d0;
-        if (packed) {
-          float2 yA, yB, tA, tB, tnA, tnB;
-          unpack_pair(v[m], vp, yA, yB);
-          unpack_pair(t0o, STAGED ? third(neg_mod<L>(k)) : tp[Cfg::T0 ? m : 0], tA, tB);
-          const float2 dA = mode_2df(yA, tA, e.x, e.y, off0, Tl, T0, T0s, tnA);
-          const float2 dB = mode_2df(yB, tB, egn.x, egn.y, off0, Tl, T0, T0s, tnB);
-          d0 = repack_pair(dA, dB);
-          t0n = repack_pair(tnA, tnB);
-        } else {
-          d0 = mode_2df(v[m], t0o, e.x, e.y, off0, Tl, T0, T0s, t0n);
-        }
+        const float2 t0p = STAGED ? third(neg_mod<L>(k)) : tp[Cfg::T0 ? m : 0];
+        // (the pair is formed by every lane and kept by the packed column's)
+        float2 yA, yB, tA, tB, tnA, tnB;
+        unpack_pair(v[m], vp, yA, yB);
+        unpack_pair(t0o, t0p, tA, tB);
+        const float2 dB = mode_2df(yB, tB, egn.x, egn.y, off0, Tl, T0, T0s, tnB);
+        yA = make_float2(packed ? yA.x : v[m].x, packed ? yA.y : v[m].y);
+        tA = make_float2(packed ? tA.x : t0o.x, packed ? tA.y : t0o.y);
+        const float2 dA = mode_2df(yA, tA, e.x, e.y, off0, Tl, T0, T0s, tnA);
+        const float2 dp = repack_pair(dA, dB), tq = repack_pair(tnA, tnB);
+        const float2 d0 = make_float2(packed ? dp.x : dA.x, packed ? dp.y : dA.y);
+        const float2 t0n = make_float2(packed ? tq.x : tnA.x, packed ? tq.y : tnA.y);
         v[m] = d0;
-        a.f_t0[(size_t)k * ncols + col] = t0n;
+        a.f_t0[at0 + (size_t)k * WF_TW] = t0n;
       }
     }
   }

@@ -52,8 +52,8 @@ col_kernel(ColArgs a) {
   const int t = threadIdx.x / W;
   const int ncols = a.nx / 2;
   const int col = blockIdx.x * W + c;
-  const bool valid = col < ncols;
-  const int colv = valid ? col : 0;
+  constexpr bool valid = true;  // ncols is a multiple of W
+  const int colv = col;
   float2* sb = sbuf + c * Cfg::STRIDE;
 
   pdl_trigger();
@@ -89,6 +89,18 @@ col_kernel(ColArgs a) {
     __syncthreads();
   };
 
+  // Every mode through f(m, whether it belongs to the packed column): CTA 0
+  // has a loop of its own, so that the others' loads overlap.
+  auto each_mode = [&](auto&& f) {
+    if (blockIdx.x != 0) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) f(m, false);
+    } else {
+#pragma unroll
+      for (int m = 0; m < E; ++m) f(m, c == 0);
+    }
+  };
+
   if constexpr (MODE == COL_RESID_A) {
     // g = S^-1 s and s = C g in RF, for the residual and the export of s:
     // from the data-side messenger (merged 2DF block, or no 1/f part), or
@@ -107,13 +119,12 @@ col_kernel(ColArgs a) {
       for (int m = 0; m < E; ++m) v[m] = valid ? a.f_y[att(t + m * TPC)] : make_float2(0.f, 0.f);
       fft_block<L, E, false>(v, sb, t, a.twy, 1);
       if (blockIdx.x == 0) exchange0(v, vp);
-#pragma unroll
-      for (int m = 0; m < E; ++m) {
+      each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
         const float2 eg = eig_at(m);
         // with a source j: g = (y + (N0 + T) j^) / (C + N0 + T)
         const float2 jv = (a.src != nullptr && valid) ? a.src[att(k)] : make_float2(0.f, 0.f);
-        if (blockIdx.x == 0 && c == 0) {
+        if (pk) {
           const float2 egb = a.eig_nyq[k];
           const float2 jp = (a.src != nullptr) ? a.src[att(neg_mod<L>(k))] : make_float2(0.f, 0.f);
           float2 A, B, JA, JB;
@@ -131,7 +142,7 @@ col_kernel(ColArgs a) {
           v[m] = g;
           w[m] = cscale(g, eg.x);
         }
-      }
+      });
       fft_block<L, E, true>(v, sb, t, a.twy, 1);
       fft_block<L, E, true>(w, sb, t, a.twy, 1);
       if (valid) {
@@ -143,18 +154,17 @@ col_kernel(ColArgs a) {
       }
     } else if (a.has_f) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) v[m] = valid ? a.f_t0[at(t + m * TPC)] : make_float2(0.f, 0.f);
+      for (int m = 0; m < E; ++m) v[m] = valid ? a.f_t0[att(t + m * TPC)] : make_float2(0.f, 0.f);
       const float T0s = a.st->T0s[a.parity];
       float2 w[E];
-#pragma unroll
-      for (int m = 0; m < E; ++m) {
+      each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
         const float2 eg = eig_at(m);
-        if (blockIdx.x == 0 && c == 0) {
+        if (pk) {
           const int kp = neg_mod<L>(k);
           const float2 egb = a.eig_nyq[k];
           float2 A, B;
-          unpack_pair(v[m], a.f_t0[at(kp)], A, B);
+          unpack_pair(v[m], a.f_t0[att(kp)], A, B);
           const float ia = __fdividef(1.f, eg.x + T0s), ib = __fdividef(1.f, egb.x + T0s);
           const float2 gA = cscale(A, ia), gB = cscale(B, ib);
           v[m] = repack_pair(gA, gB);
@@ -164,7 +174,7 @@ col_kernel(ColArgs a) {
           v[m] = g;
           w[m] = cscale(g, eg.x);
         }
-      }
+      });
       fft_block<L, E, true>(v, sb, t, a.twy, 1);
       fft_block<L, E, true>(w, sb, t, a.twy, 1);
       if (valid) {
@@ -182,18 +192,17 @@ col_kernel(ColArgs a) {
     for (int m = 0; m < E; ++m) v[m] = valid ? a.r_g[at(t + m * TPC)] : make_float2(0.f, 0.f);
     fft_block<L, E, false>(v, sb, t, a.twy, 1);
     if (blockIdx.x == 0) exchange0(v, vp);
-#pragma unroll
-    for (int m = 0; m < E; ++m) {
+    each_mode([&](int m, bool pk) {
       const int k = t + m * TPC;
       const float2 eg = eig_at(m);
-      if (blockIdx.x == 0 && c == 0) {
+      if (pk) {
         float2 A, B;
         unpack_pair(v[m], vp[m], A, B);
         v[m] = repack_pair(cscale(A, eg.y), cscale(B, a.eig_nyq[k].y));
       } else {
         v[m] = cscale(v[m], eg.y);
       }
-    }
+    });
     fft_block<L, E, true>(v, sb, t, a.twy, 1);
     const float sc = 1.0f / (float)L;
     if (valid) {
@@ -211,18 +220,17 @@ col_kernel(ColArgs a) {
     for (int m = 0; m < E; ++m) v[m] = valid ? a.r_q[at(t + m * TPC)] : make_float2(0.f, 0.f);
     fft_block<L, E, false>(v, sb, t, a.twy, 1);
     if (blockIdx.x == 0) exchange0(v, vp);
-#pragma unroll
-    for (int m = 0; m < E; ++m) {
+    each_mode([&](int m, bool pk) {
       const int k = t + m * TPC;
       const float2 eg = eig_at(m);
-      if (blockIdx.x == 0 && c == 0) {
+      if (pk) {
         float2 A, B;
         unpack_pair(v[m], vp[m], A, B);
         v[m] = repack_pair(cscale(A, __fdividef(1.f, eg.x)), cscale(B, __fdividef(1.f, a.eig_nyq[k].x)));
       } else {
         v[m] = cscale(v[m], __fdividef(1.f, eg.x));
       }
-    }
+    });
     fft_block<L, E, true>(v, sb, t, a.twy, 1);
     const float sc = 1.0f / (float)L;
     if (valid) {
@@ -243,12 +251,11 @@ col_kernel(ColArgs a) {
       const float off0 = (float)a.st->off[0];
       fft_block<L, E, false>(v, sb, t, a.twy, 1);
       if (blockIdx.x == 0) exchange0(v, vp);
-#pragma unroll
-      for (int m = 0; m < E; ++m) {
+      each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
         const float2 eg = valid ? a.eig[att(k)] : make_float2(1.f, 0.f);
         const float fa = __fdividef(eg.x + eg.y + off0, eg.x);
-        if (blockIdx.x == 0 && c == 0) {
+        if (pk) {
           const float2 egb = a.eig_nyq[k];
           float2 A, B;
           unpack_pair(v[m], vp[m], A, B);
@@ -256,7 +263,7 @@ col_kernel(ColArgs a) {
         } else {
           v[m] = cscale(v[m], fa);
         }
-      }
+      });
       fft_block<L, E, true>(v, sb, t, a.twy, 1);
       const float sc = 1.0f / (float)L;
 #pragma unroll

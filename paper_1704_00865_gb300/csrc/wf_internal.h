@@ -14,9 +14,9 @@ namespace wf {
 
 struct WfState;
 
-// Fields that both passes touch -- the data-side messenger in RF (t_RF, or
-// t_PX without stripes), the field next to it on the signal side (d_2DF, or
-// s without a 1/f part), and the (C, P1f) table -- are stored in column
+// Fields that the column pass touches -- the data-side messenger in RF (t_RF,
+// or t_PX without stripes), the field next to it on the signal side (d_2DF, or
+// s without a 1/f part), t_2DF, and the (C, P1f) table -- are stored in column
 // tiles of WF_TW complex columns: element (y, kx) lives at
 //   (kx / WF_TW) * ny * WF_TW + y * WF_TW + kx % WF_TW,
 // so a column pass reads whole tiles contiguously and a row pass reads
@@ -121,7 +121,7 @@ struct ColArgs {
   int parity;                 // slot of T0s holding the stored t_2DF's T_0
   const float2* f_y;          // data-side messenger in RF (t_RF or t_PX)
   float2* f_x;                // output in RF (d_2DF or s)
-  float2* f_t0;               // t_2DF [ny][nx/2] (2D Fourier)
+  float2* f_t0;               // t_2DF (2D Fourier, column-tiled)
   const float2* eig;          // [ny][nx/2] (C, P1f) for kx = col
   const float2* eig_nyq;      // [ny] (C, P1f) at kx = nx/2
   const float2* twy;          // exp(-2 pi i k/ny), k < ny

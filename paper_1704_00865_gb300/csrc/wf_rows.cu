@@ -97,18 +97,17 @@ row_kernel(RowArgs a) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const double gd = (double)gv[h];
-        if (valid) g2 += gd * gd;
-        if (nv[h] < 0.f) {  // masked: the residual there is S^-1 s (minus a source)
-          const double rm = gd - (double)jv[h];
-          if (valid) gm2 += rm * rm;
-          gp[h] = 0.f;
-          qp[h] = 0.f;
-          go[h] = gv[h];
-        } else {             // N_PX g' + s - d with the full pixel variance
-          gp[h] = gv[h];
-          qp[h] = fmaf(nv[h] + vshift, gv[h], sv[h] - dv[h]);
-          go[h] = 0.f;
+        const bool masked = nv[h] < 0.f;  // the residual there is S^-1 s (minus a source)
+        const double rm = masked ? gd - (double)jv[h] : 0.0;
+        if (valid) {
+          g2 += gd * gd;
+          gm2 += rm * rm;
         }
+        // N_PX g' + s - d with the full pixel variance
+        const float qu = fmaf(nv[h] + vshift, gv[h], sv[h] - dv[h]);
+        gp[h] = masked ? 0.f : gv[h];
+        qp[h] = masked ? 0.f : qu;
+        go[h] = masked ? gv[h] : 0.f;
       }
       if (valid && a.gm_out != nullptr) a.gm_out[row0 + t + m * TPF] = make_float2(go[0], go[1]);
       v[m] = make_float2(gp[0], gp[1]);
@@ -153,8 +152,9 @@ row_kernel(RowArgs a) {
     for (int m = 0; m < E; ++m) {
       const float4 q = PRE ? px[PRE ? m : 0] : (valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f));
       if (valid) {
-        if (q.y >= 0.f) r2 += (double)v[m].x * (double)v[m].x;
-        if (q.w >= 0.f) r2 += (double)v[m].y * (double)v[m].y;
+        const double r0 = q.y >= 0.f ? (double)v[m].x : 0.0, r1 = q.w >= 0.f ? (double)v[m].y : 0.0;
+        r2 += r0 * r0;
+        r2 += r1 * r1;
         // optional map of Delta d on unmasked pixels (defect correction)
         if (a.out_px != nullptr)
           a.out_px[row0 + t + m * TPF] = make_float2(q.y >= 0.f ? v[m].x : 0.f, q.w >= 0.f ? v[m].y : 0.f);
