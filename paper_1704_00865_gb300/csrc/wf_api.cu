@@ -343,13 +343,33 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
   AL(P->eig_nyq, (size_t)ny);
   AL(P->pst, (size_t)P->M + 1);
   AL(P->a2, (size_t)ny);
-  AL(P->twx, (size_t)nx);
-  AL(P->twy, (size_t)ny);
-  AL(P->twh, (size_t)(nx / 2));
-  for (int v = 0; v < 2; ++v) {
-    AL(P->tws_row[v], (size_t)nx);  // (the tables have fewer than twice the transform's values)
-    AL(P->tws_col[v], (size_t)2 * ny);
+  // twiddle tables exp(-2 pi i k / n), computed in double on the host; the
+  // half-length row transform's is every other entry of twx; the stage tables
+  // of the passes' shapes; each padded to a multiple of 16 bytes
+  std::vector<float2> tx(nx), ty(ny), th(nx / 2), tabs;
+  for (int k = 0; k < nx; ++k) {
+    const double a = 2.0 * M_PI * (double)k / (double)nx;
+    tx[k] = make_float2((float)cos(a), (float)-sin(a));
   }
+  for (int k = 0; k < ny; ++k) {
+    const double a = 2.0 * M_PI * (double)k / (double)ny;
+    ty[k] = make_float2((float)cos(a), (float)-sin(a));
+  }
+  for (int k = 0; k < nx / 2; ++k) th[k] = tx[2 * k];
+  size_t tab_off[7], ntab = 0;
+  auto add_table = [&](const std::vector<float2>& t) {
+    tab_off[ntab++] = tabs.size();
+    tabs.insert(tabs.end(), t.begin(), t.end());
+    if (tabs.size() % 2) tabs.push_back(make_float2(0.f, 0.f));
+  };
+  add_table(tx);
+  add_table(ty);
+  add_table(th);
+  for (int v = 0; v < 2; ++v) {
+    add_table(stage_table(th, row_pass_e(P->M, v)));
+    add_table(stage_table(ty, col_pass_e(ny, v)));
+  }
+  AL(P->twx, tabs.size());
   AL(P->r_g, nh);
   AL(P->r_q, nh);
   AL(P->part, (size_t)3 * P->nrow + 4 * 256 + 64);
@@ -438,33 +458,16 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
       return WF_EUNSUPPORTED;
     }
   }
-  // twiddle tables exp(-2 pi i k / n), computed in double on the host
-  std::vector<float2> tx(nx), ty(ny);
-  for (int k = 0; k < nx; ++k) {
-    const double a = 2.0 * M_PI * (double)k / (double)nx;
-    tx[k] = make_float2((float)cos(a), (float)-sin(a));
-  }
-  for (int k = 0; k < ny; ++k) {
-    const double a = 2.0 * M_PI * (double)k / (double)ny;
-    ty[k] = make_float2((float)cos(a), (float)-sin(a));
-  }
-  // the half-length row transform's table is every other entry of twx
-  std::vector<float2> th(nx / 2);
-  for (int k = 0; k < nx / 2; ++k) th[k] = tx[2 * k];
-  cudaError_t e1 = cudaMemcpy(P->twx, tx.data(), nx * sizeof(float2), cudaMemcpyHostToDevice);
-  cudaError_t e2 = cudaMemcpy(P->twy, ty.data(), ny * sizeof(float2), cudaMemcpyHostToDevice);
-  cudaError_t e3 = cudaMemcpy(P->twh, th.data(), nx / 2 * sizeof(float2), cudaMemcpyHostToDevice);
-  bool tabs = e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess;
-  for (int v = 0; v < 2 && tabs; ++v) {
-    const std::vector<float2> r = stage_table(th, row_pass_e(P->M, v)), c = stage_table(ty, col_pass_e(ny, v));
-    tabs = r.size() <= (size_t)nx && c.size() <= (size_t)2 * ny &&
-           cudaMemcpy(P->tws_row[v], r.data(), r.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
-           cudaMemcpy(P->tws_col[v], c.data(), c.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
-  }
-  if (!tabs) {
+  if (cudaMemcpy(P->twx, tabs.data(), tabs.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
     wf_plan_destroy(P);
     return WF_ECUDA;
+  }
+  P->twy = P->twx + tab_off[1];
+  P->twh = P->twx + tab_off[2];
+  for (int v = 0; v < 2; ++v) {
+    P->tws_row[v] = P->twx + tab_off[3 + 2 * v];
+    P->tws_col[v] = P->twx + tab_off[4 + 2 * v];
   }
   *out = P;
   return WF_OK;

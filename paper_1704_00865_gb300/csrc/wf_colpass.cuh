@@ -55,8 +55,11 @@ struct ColPassCfg {
   static constexpr size_t al(size_t n) { return (n + 15) / 16 * 16; }
   static constexpr size_t tile = STAGED ? (size_t)L * W * 8 : 0;
   static constexpr size_t fft_off = 16;
-  static constexpr size_t y_off = LAND ? fft_off : fft_off + al((size_t)W * STRIDE * 8);
-  static constexpr size_t eig_off = LAND ? fft_off + al((size_t)W * STRIDE * 8) : y_off + tile;
+  // PP: the messenger's tile, once read, is the second exchange buffer
+  static constexpr bool PP = STAGED && !LAND && PREC == 0;
+  static constexpr size_t fft_bytes = al((size_t)W * STRIDE * 8);
+  static constexpr size_t y_off = LAND ? fft_off : fft_off + fft_bytes;
+  static constexpr size_t eig_off = LAND ? fft_off + fft_bytes : y_off + (PP ? fft_bytes : tile);
   static constexpr size_t t0_off = eig_off + tile;
   static constexpr size_t tw_off = t0_off + (EXTRA ? tile : 0);
   // the twiddle table too where it costs no CTA per SM
@@ -98,6 +101,7 @@ col_pass_kernel(ColArgs a) {
   constexpr int E = Cfg::E, TPC = Cfg::TPC, W = Cfg::W;
   constexpr bool STAGED = Cfg::STAGED, MERGED = (MODE == COL_PASS_MERGE || MODE == COL_PASS_MERGE_SRC);
   static_assert(!STAGED || Cfg::TILED, "whole tiles are staged");
+  static_assert(!Cfg::PP || Cfg::fft_bytes >= Cfg::tile, "the second exchange buffer holds the tile");
   extern __shared__ __align__(16) unsigned char smem[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
   float2* s_fft = reinterpret_cast<float2*>(smem + Cfg::fft_off);
@@ -111,6 +115,7 @@ col_pass_kernel(ColArgs a) {
   const int col0 = blockIdx.x * W;
   const int col = col0 + c;
   float2* sb = s_fft + c * Cfg::STRIDE;
+  float2* sb2 = s_y + c * Cfg::STRIDE;  // PP
   const size_t at0 = tidx(0, col, a.ny);  // (ky, this column) in the tiled fields: at0 + 4 ky
   const size_t tile0 = tidx(0, col0, a.ny);
   const bool packed = (blockIdx.x == 0 && c == 0);
@@ -195,12 +200,13 @@ col_pass_kernel(ColArgs a) {
     tc5_setup<L, PREC>(smem + Cfg::bytes, tc5_mbar<L, MODE, EV, PREC>(smem), Cfg::TWS ? s_tw : a.twy, 1);
 
   if constexpr (PREC) fft_block<L, E, false, false, Cfg::TWS, PREC>(v, sb, t, Cfg::TWS ? s_tw : a.twy, 1);
+  else if constexpr (Cfg::PP) fft_pingpong<L, E, false, false, Cfg::TWS>(v, sb, sb2, t, Cfg::TWS ? s_tw : a.tws);
   else fft_staged<L, E, false, false, Cfg::TWS>(v, sb, t, Cfg::TWS ? s_tw : a.tws);
 
   // partner values Z[-k] for the packed column 0, read below from shared
   // memory (CTA 0 only; uniform)
   if (blockIdx.x == 0) {
-    __syncthreads();
+    if constexpr (!Cfg::PP) __syncthreads();
 #pragma unroll
     for (int m = 0; m < E; ++m) sb[spad(t + m * TPC)] = v[m];
     __syncthreads();
@@ -275,8 +281,17 @@ col_pass_kernel(ColArgs a) {
     // publish the T_0 that the new t_2DF was made with (implicit s)
     if (blockIdx.x == 0 && threadIdx.x == 0) a.st->T0s[a.parity ^ 1] = T0;
   }
-  if (blockIdx.x == 0) __syncthreads();  // the partners are read
+  if (blockIdx.x == 0) {
+    if constexpr (Cfg::PP) {  // its partners are still being read: the other buffer
+      float2* x = sb;
+      sb = sb2;
+      sb2 = x;
+    } else {
+      __syncthreads();  // the partners are read
+    }
+  }
   if constexpr (PREC) fft_block<L, E, true, false, Cfg::TWS, PREC>(v, sb, t, Cfg::TWS ? s_tw : a.twy, 1);
+  else if constexpr (Cfg::PP) fft_pingpong<L, E, true, false, Cfg::TWS>(v, sb, sb2, t, Cfg::TWS ? s_tw : a.tws);
   else fft_staged<L, E, true, false, Cfg::TWS>(v, sb, t, Cfg::TWS ? s_tw : a.tws);
   if constexpr (PREC >= 3) {
     tc5_teardown();

@@ -722,8 +722,10 @@ struct FFTStages {
     }
   }
 
-  static __device__ __forceinline__ void stage_fp32(float2 (&v)[E], float2* sb, int t,
-                                                    const float2* __restrict__ twtab, int twstride) {
+  // the stage's butterflies: inputs from the registers, outputs to the buffer
+  // (or, of the last stage, back to the registers)
+  static __device__ __forceinline__ void butterflies(float2 (&v)[E], float2* sb, int t,
+                                                     const float2* __restrict__ twtab, int twstride) {
     constexpr int TPF = L / E;
     constexpr int B = E / R;
     constexpr bool LAST = (NS * R == L);
@@ -760,15 +762,43 @@ struct FFTStages {
         for (int r = 0; r < R; ++r) sb[spad(base + r * NS)] = u[r];
       }
     }
-    if constexpr (!LAST) {
+  }
+
+  static __device__ __forceinline__ void stage_fp32(float2 (&v)[E], float2* sb, int t,
+                                                    const float2* __restrict__ twtab, int twstride) {
+    butterflies(v, sb, t, twtab, twstride);
+    if constexpr (NS * R != L) {
       fft_sync<WARP>();
 #pragma unroll
-      for (int m = 0; m < E; ++m) v[m] = sb[spad(t + m * TPF)];
+      for (int m = 0; m < E; ++m) v[m] = sb[spad(t + m * (L / E))];
       fft_sync<WARP>();
       FFTStages<L, E, NS * R, INV, WARP, TWS, PREC, NEXT>::run(v, sb, t, twtab, twstride);
     }
   }
 };
+
+// The stages with two exchange buffers in turn, from stage table `table`: a
+// barrier between the stores and the loads of an exchange is enough, since the
+// next one goes to the other buffer (whose readers have passed this barrier).
+template <int L, int E, int NS, bool INV, bool WARP, bool TWS, int OFF>
+struct FFTStagesPP {
+  using S = FFTStages<L, E, NS, INV, WARP, TWS, 0, OFF>;
+  static constexpr int R = StageRadix<L, E, NS>::value;
+  static constexpr bool LAST = (NS * R == L);
+  static constexpr int exchanges = LAST ? 0 : 1 + FFTStagesPP<L, E, LAST ? L : NS * R, INV, WARP, TWS, 0>::exchanges;
+  static __device__ __forceinline__ void run(float2 (&v)[E], float2* sb, float2* other, int t,
+                                             const float2* __restrict__ table) {
+    S::butterflies(v, sb, t, table, 1);
+    if constexpr (!LAST) {
+      fft_sync<WARP>();
+#pragma unroll
+      for (int m = 0; m < E; ++m) v[m] = sb[spad(t + m * (L / E))];
+      FFTStagesPP<L, E, NS * R, INV, WARP, TWS, S::NEXT>::run(v, other, sb, t, table);
+    }
+  }
+};
+template <int L, int E, bool INV, bool WARP, bool TWS, int OFF>
+struct FFTStagesPP<L, E, L, INV, WARP, TWS, OFF> { static constexpr int exchanges = 0; };
 
 // Full complex DFT of length L (no scaling).  Every thread of the block (or
 // of the warp, WARP = true) must call it; sb is this transform's own padded
@@ -782,6 +812,20 @@ __device__ __forceinline__ void fft_block(float2 (&v)[E], float2* sb, int t,
 template <int L, int E, bool INV, bool WARP = false, bool TWS = false>
 __device__ __forceinline__ void fft_staged(float2 (&v)[E], float2* sb, int t, const float2* __restrict__ table) {
   FFTStages<L, E, 1, INV, WARP, TWS, 0, 0>::run(v, sb, t, table, 1);
+}
+
+// The same with two buffers in turn, the first exchange through sb: `sb` and
+// `other` are swapped on return so that sb is the next one to use.
+template <int L, int E, bool INV, bool WARP = false, bool TWS = false>
+__device__ __forceinline__ void fft_pingpong(float2 (&v)[E], float2*& sb, float2*& other, int t,
+                                             const float2* __restrict__ table) {
+  using F = FFTStagesPP<L, E, 1, INV, WARP, TWS, 0>;
+  F::run(v, sb, other, t, table);
+  if constexpr (F::exchanges % 2 != 0) {
+    float2* x = sb;
+    sb = other;
+    other = x;
+  }
 }
 
 // W_N^k (N = 2M) for the k = t + m*(M/E) a thread handles in c2r_pre and

@@ -211,7 +211,8 @@ struct RowPassCfg {
 // Shared memory of the row pass.  The tiles of the column-tiled fields keep
 // their order, [tile][row][4 columns].  EARLY (rows up to 512 values, whose
 // CTAs all fit at once): every input has its own buffer and is requested at the
-// start.  Longer rows: the field of the first transform lands in the
+// start, and the first transform's field's, once read, is the second exchange
+// buffer (one barrier per exchange instead of two).  Longer rows: the field of the first transform lands in the
 // transform's own buffer (its values and their partners -k are read from there
 // before the first exchange overwrites them), and t_RF and the signal-side
 // field take the pixel table's place once the pixel update has read it -- 50
@@ -226,10 +227,11 @@ struct RowPassSmem {
   static constexpr size_t al(size_t n) { return (n + 127) / 128 * 128; }
   static constexpr size_t field = (size_t)ROWS * M * 8;
   static constexpr size_t fft_off = 128;
-  static constexpr size_t dn_off = fft_off + al((size_t)ROWS * SPad<M>::size * 8);
+  static constexpr size_t fft_bytes = al((size_t)ROWS * SPad<M>::size * 8);
+  static constexpr size_t dn_off = fft_off + fft_bytes;
   static constexpr size_t in_off = EARLY ? dn_off + 2 * field : fft_off;  // the first transform's field
-  static constexpr size_t t_off = !RF ? dn_off : (EARLY ? in_off + field : dn_off);  // t_RF, then the signal side
-  static constexpr size_t tw_off = EARLY ? in_off + field + (RF ? 2 * field : 0) : dn_off + 2 * field;
+  static constexpr size_t t_off = !RF ? dn_off : (EARLY ? in_off + fft_bytes : dn_off);  // t_RF, then the signal side
+  static constexpr size_t tw_off = EARLY ? in_off + fft_bytes + (RF ? 2 * field : 0) : dn_off + 2 * field;
   // the transform twiddles are staged too for short rows
   static constexpr bool TWS = M <= 512;
   static constexpr uint32_t tw_bytes = StageTable<M, EV>::size * 8;  // a multiple of 16
@@ -358,7 +360,9 @@ row_pass_kernel(const __grid_constant__ RowArgs a) {
   c2r_pre_at<M, E>(v, t, [&](int k) { return RF ? s_in[g * M + k] : s_in[SM::tpos(g, k)]; },
                    [&](int m, int k) { return EARLY ? wk[EARLY ? m : 0] : __ldg(&a.twx[k]); });
   if constexpr (!EARLY) fft_sync<W>();  // read before the first exchange overwrites it
-  fft_staged<M, E, true, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
+  float2* sb2 = s_in + g * SPad<M>::size;  // EARLY: the second exchange buffer
+  if constexpr (EARLY) fft_pingpong<M, E, true, W, SM::TWS>(v, sb, sb2, t, s_tw);
+  else fft_staged<M, E, true, W, SM::TWS>(v, sb, t, a.tws);
   // eq. (2mess_t1) analogue in pixel space, two pixels per complex value
 #pragma unroll
   for (int m = 0; m < E; ++m) {
@@ -373,7 +377,8 @@ row_pass_kernel(const __grid_constant__ RowArgs a) {
       load_tiled(s_x, &a.tm_x, &bar[2]);
     }
   }
-  fft_staged<M, E, false, W, SM::TWS>(v, sb, t, SM::TWS ? s_tw : a.tws);
+  if constexpr (EARLY) fft_pingpong<M, E, false, W, SM::TWS>(v, sb, sb2, t, s_tw);
+  else fft_staged<M, E, false, W, SM::TWS>(v, sb, t, a.tws);
   if constexpr (EARLY) r2c_post_w<M, E, W, true>(v, sb, t, wk);
   else r2c_post<M, E, W, true>(v, sb, t, a.twx);
   pdl_trigger();
