@@ -43,6 +43,7 @@ struct wf_plan_s {
   float *pst = nullptr, *a2 = nullptr;
   float2 *twx = nullptr, *twy = nullptr, *twh = nullptr;  // twh: exp(-2 pi i k/(nx/2))
   float2 *tws_row[2] = {}, *tws_col[2] = {};              // stage tables of the passes' shapes
+  float2 *twk_row = nullptr, *twk_col = nullptr;          // and of the other kernels
   float2 *r_g = nullptr, *r_q = nullptr;
   double* part = nullptr;
   double* chi = nullptr;  // wf_chi2_aug: partial sums, then the value
@@ -345,7 +346,7 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
   AL(P->a2, (size_t)ny);
   // twiddle tables exp(-2 pi i k / n), computed in double on the host; the
   // half-length row transform's is every other entry of twx; the stage tables
-  // of the passes' shapes; each padded to a multiple of 16 bytes
+  // of the passes' shapes and of the other kernels; each padded to a multiple of 16 bytes
   std::vector<float2> tx(nx), ty(ny), th(nx / 2), tabs;
   for (int k = 0; k < nx; ++k) {
     const double a = 2.0 * M_PI * (double)k / (double)nx;
@@ -356,7 +357,7 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
     ty[k] = make_float2((float)cos(a), (float)-sin(a));
   }
   for (int k = 0; k < nx / 2; ++k) th[k] = tx[2 * k];
-  size_t tab_off[7], ntab = 0;
+  size_t tab_off[9], ntab = 0;
   auto add_table = [&](const std::vector<float2>& t) {
     tab_off[ntab++] = tabs.size();
     tabs.insert(tabs.end(), t.begin(), t.end());
@@ -369,6 +370,8 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
     add_table(stage_table(th, row_pass_e(P->M, v)));
     add_table(stage_table(ty, col_pass_e(ny, v)));
   }
+  add_table(stage_table(th, row_kernel_e(P->M)));
+  add_table(stage_table(ty, col_kernel_e(ny)));
   AL(P->twx, tabs.size());
   AL(P->r_g, nh);
   AL(P->r_q, nh);
@@ -469,6 +472,8 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
     P->tws_row[v] = P->twx + tab_off[3 + 2 * v];
     P->tws_col[v] = P->twx + tab_off[4 + 2 * v];
   }
+  P->twk_row = P->twx + tab_off[7];
+  P->twk_col = P->twx + tab_off[8];
   *out = P;
   return WF_OK;
 }
@@ -495,6 +500,7 @@ static RowArgs row_args(wf_plan_s* P) {
   a.twx = P->twx;
   a.twh = P->twh;
   a.tws = P->tws_row[P->row_variant];
+  a.twk = P->twk_row;
   a.st = P->st;
   a.r_g = P->r_g;
   a.r_q = P->r_q;
@@ -521,6 +527,7 @@ static ColArgs col_args(wf_plan_s* P, int parity) {
   a.eig_nyq = P->eig_nyq;
   a.twy = P->twy;
   a.tws = P->tws_col[a.variant];
+  a.twk = P->twk_col;
   a.st = P->st;
   a.r_g = P->r_g;
   a.r_q = P->r_q;

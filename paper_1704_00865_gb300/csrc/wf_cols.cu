@@ -19,7 +19,7 @@ namespace wf {
 
 template <int L>
 struct ColCfg {
-  static constexpr int E = (L % 3 == 0) ? 12 : ((L >= 2048) ? 16 : 8);
+  static constexpr int E = col_kernel_e(L);
   static constexpr int TPC = L / E;
   // whole tiles, 32-byte pieces of the row-major fields (half of that at 4096,
   // where four columns would not fit)
@@ -117,7 +117,7 @@ col_kernel(ColArgs a) {
       float2 w[E];
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = valid ? a.f_y[att(t + m * TPC)] : make_float2(0.f, 0.f);
-      fft_block<L, E, false>(v, sb, t, a.twy, 1);
+      fft_staged<L, E, false>(v, sb, t, a.twk);
       if (blockIdx.x == 0) exchange0(v, vp);
       each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
@@ -143,8 +143,8 @@ col_kernel(ColArgs a) {
           w[m] = cscale(g, eg.x);
         }
       });
-      fft_block<L, E, true>(v, sb, t, a.twy, 1);
-      fft_block<L, E, true>(w, sb, t, a.twy, 1);
+      fft_staged<L, E, true>(v, sb, t, a.twk);
+      fft_staged<L, E, true>(w, sb, t, a.twk);
       if (valid) {
 #pragma unroll
         for (int m = 0; m < E; ++m) {
@@ -175,8 +175,8 @@ col_kernel(ColArgs a) {
           w[m] = cscale(g, eg.x);
         }
       });
-      fft_block<L, E, true>(v, sb, t, a.twy, 1);
-      fft_block<L, E, true>(w, sb, t, a.twy, 1);
+      fft_staged<L, E, true>(v, sb, t, a.twk);
+      fft_staged<L, E, true>(w, sb, t, a.twk);
       if (valid) {
 #pragma unroll
         for (int m = 0; m < E; ++m) {
@@ -190,7 +190,7 @@ col_kernel(ColArgs a) {
     float2 vp[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.r_g[at(t + m * TPC)] : make_float2(0.f, 0.f);
-    fft_block<L, E, false>(v, sb, t, a.twy, 1);
+    fft_staged<L, E, false>(v, sb, t, a.twk);
     if (blockIdx.x == 0) exchange0(v, vp);
     each_mode([&](int m, bool pk) {
       const int k = t + m * TPC;
@@ -203,7 +203,7 @@ col_kernel(ColArgs a) {
         v[m] = cscale(v[m], eg.y);
       }
     });
-    fft_block<L, E, true>(v, sb, t, a.twy, 1);
+    fft_staged<L, E, true>(v, sb, t, a.twk);
     const float sc = 1.0f / (float)L;
     if (valid) {
 #pragma unroll
@@ -218,7 +218,7 @@ col_kernel(ColArgs a) {
     float2 vp[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.r_q[at(t + m * TPC)] : make_float2(0.f, 0.f);
-    fft_block<L, E, false>(v, sb, t, a.twy, 1);
+    fft_staged<L, E, false>(v, sb, t, a.twk);
     if (blockIdx.x == 0) exchange0(v, vp);
     each_mode([&](int m, bool pk) {
       const int k = t + m * TPC;
@@ -231,7 +231,7 @@ col_kernel(ColArgs a) {
         v[m] = cscale(v[m], __fdividef(1.f, eg.x));
       }
     });
-    fft_block<L, E, true>(v, sb, t, a.twy, 1);
+    fft_staged<L, E, true>(v, sb, t, a.twk);
     const float sc = 1.0f / (float)L;
     if (valid) {
 #pragma unroll
@@ -249,7 +249,7 @@ col_kernel(ColArgs a) {
     }
     if (a.has_f) {
       const float off0 = (float)a.st->off[0];
-      fft_block<L, E, false>(v, sb, t, a.twy, 1);
+      fft_staged<L, E, false>(v, sb, t, a.twk);
       if (blockIdx.x == 0) exchange0(v, vp);
       each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
@@ -264,7 +264,7 @@ col_kernel(ColArgs a) {
           v[m] = cscale(v[m], fa);
         }
       });
-      fft_block<L, E, true>(v, sb, t, a.twy, 1);
+      fft_staged<L, E, true>(v, sb, t, a.twk);
       const float sc = 1.0f / (float)L;
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = cscale(v[m], sc);
@@ -281,7 +281,7 @@ col_kernel(ColArgs a) {
   } else if constexpr (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED) {
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.in[at(t + m * TPC)] : make_float2(0.f, 0.f);
-    fft_block<L, E, MODE == COL_INV>(v, sb, t, a.twy, 1);
+    fft_staged<L, E, MODE == COL_INV>(v, sb, t, a.twk);
     const float sc = (MODE == COL_INV) ? 1.0f / (float)L : 1.0f;
     if (valid) {
 #pragma unroll

@@ -95,6 +95,7 @@ struct RowArgs {
   const float2* twx;          // exp(-2 pi i k/nx), k < nx
   const float2* twh;          // exp(-2 pi i k/(nx/2)), k < nx/2
   const float2* tws;          // row pass: stage table of its shape (StageTable)
+  const float2* twk;          // the other row kernels' stage table
   WfState* st;
   float2* r_g;                // residual scratch (RF)
   float2* r_q;
@@ -126,6 +127,7 @@ struct ColArgs {
   const float2* eig_nyq;      // [ny] (C, P1f) at kx = nx/2
   const float2* twy;          // exp(-2 pi i k/ny), k < ny
   const float2* tws;          // column pass: stage table of its shape
+  const float2* twk;          // the other column kernels' stage table
   WfState* st;
   float2* r_g;
   float2* r_q;
@@ -189,6 +191,14 @@ int launch_col_pass_tc(int L, int mode, const ColArgs& a, cudaStream_t s);
 int launch_col_dft_tc(int inverse, const ColArgs& a, cudaStream_t s);
 bool col_tc_supported(int L);
 bool col_tc5_supported(int L);  // tcgen05 stages (dft_precision 3, 4)
+// values per thread of the residual's and the plain transforms' kernels
+// (they read their twiddles from stage tables as the passes do: from the table
+// exp(-2 pi i k / L), whose entries lanes read lines apart, a forward and an
+// inverse 2048^2 transform took 76.0 us instead of 72.4, a 512 x 384 run with a
+// residual every second sweep 2199 instead of 2100; 2048-value rows take 8
+// values, 16 before)
+constexpr int row_kernel_e(int M) { return M % 3 == 0 ? 12 : 8; }
+constexpr int col_kernel_e(int L) { return L % 3 == 0 ? 12 : (L >= 2048 ? 16 : 8); }
 // values per thread of the row / column pass shape `variant` for a length
 int row_pass_e(int M, int variant);
 int row_pass_rows(int M, int variant);  // rows per CTA

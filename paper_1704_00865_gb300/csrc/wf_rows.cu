@@ -18,7 +18,7 @@ namespace wf {
 
 template <int M>
 struct RowCfg {
-  static constexpr int E = (M % 3 == 0) ? 12 : ((M >= 2048) ? 16 : 8);
+  static constexpr int E = row_kernel_e(M);
   static constexpr int TPF = M / E;
   // one row per CTA, or as many as a warp holds: a 512 x 384 map gives 256 CTAs
   // (with 256 threads each it gave 32 and the residual's row steps took 27
@@ -82,9 +82,9 @@ row_kernel(RowArgs a) {
       w[m] = valid ? a.r_q[row0 + t + m * TPF] : make_float2(0.f, 0.f);
     }
     c2r_pre<M, E>(v, sb, t, a.twx);
-    fft_block<M, E, true>(v, sb, t, a.twx, 2);
+    fft_staged<M, E, true>(v, sb, t, a.twk);
     c2r_pre<M, E>(w, sb, t, a.twx);
-    fft_block<M, E, true>(w, sb, t, a.twx, 2);
+    fft_staged<M, E, true>(w, sb, t, a.twk);
     const float vshift = (float)a.st->var_shift;
     double gm2 = 0.0, g2 = 0.0;
 #pragma unroll
@@ -113,9 +113,9 @@ row_kernel(RowArgs a) {
       v[m] = make_float2(gp[0], gp[1]);
       w[m] = make_float2(qp[0], qp[1]);
     }
-    fft_block<M, E, false>(v, sb, t, a.twx, 2);
+    fft_staged<M, E, false>(v, sb, t, a.twk);
     r2c_post<M, E>(v, sb, t, a.twx);
-    fft_block<M, E, false>(w, sb, t, a.twx, 2);
+    fft_staged<M, E, false>(w, sb, t, a.twk);
     r2c_post<M, E>(w, sb, t, a.twx);
     if (valid) {
       const float a2y = (a.a2 != nullptr) ? a.a2[y] : 1.f;
@@ -146,7 +146,7 @@ row_kernel(RowArgs a) {
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.r_q[row0 + t + m * TPF] : make_float2(0.f, 0.f);
     c2r_pre<M, E>(v, sb, t, a.twx);
-    fft_block<M, E, true>(v, sb, t, a.twx, 2);
+    fft_staged<M, E, true>(v, sb, t, a.twk);
     double r2 = 0.0;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -166,7 +166,7 @@ row_kernel(RowArgs a) {
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.in_rf[row0 + t + m * TPF] : make_float2(0.f, 0.f);
     c2r_pre<M, E>(v, sb, t, a.twx);
-    fft_block<M, E, true>(v, sb, t, a.twx, 2);
+    fft_staged<M, E, true>(v, sb, t, a.twk);
     if (valid) {
 #pragma unroll
       for (int m = 0; m < E; ++m) a.out_px[row0 + t + m * TPF] = v[m];
@@ -174,7 +174,7 @@ row_kernel(RowArgs a) {
   } else if constexpr (MODE == ROW_R2C) {
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = valid ? a.in_px[row0 + t + m * TPF] : make_float2(0.f, 0.f);
-    fft_block<M, E, false>(v, sb, t, a.twx, 2);
+    fft_staged<M, E, false>(v, sb, t, a.twk);
     r2c_post<M, E>(v, sb, t, a.twx);
     if (valid) {
 #pragma unroll
@@ -192,8 +192,8 @@ row_kernel(RowArgs a) {
 // Values per thread of the two shapes the autotuner chooses between (one
 // where both coincide): 8 (two warps per 1024-point row) measured fastest at
 // 1024^2 and above (16 values: 20.1 against 19.0 us at 2048^2, 97 against 90 at
-// 4096^2), 4 at 512^2 and below; 3 * 2^k rows take 12 (13.0 -> 17.0 us at 1536^2)
-// or 24 (the other way round from 768^2 down).
+// 4096^2), 4 at 512^2 and below; 3 * 2^k rows take 24 (13.0 against 17.0 us at 1536^2)
+// or 12 (faster from 768^2 down).
 template <int M>
 struct RowPassE {
   static constexpr int v0 = (M % 3 == 0) ? 12 : 8;

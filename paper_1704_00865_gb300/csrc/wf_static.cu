@@ -24,12 +24,14 @@
 
 namespace {
 
-constexpr int kMaxSide = 4096;                 // twiddle table length per axis
+constexpr int kMaxSide = 4096;                 // row twiddle table, and both stage tables
 constexpr size_t kMaxSpectrum = (size_t)1 << 19;  // complex values: ny * nx / 2 <= 2^19
 constexpr size_t kStaticComplex = 2 * (size_t)kMaxSide + kMaxSpectrum;  // 4 MiB + 64 KiB
 
-// [0, 4096): exp(-2 pi i k / nx); [4096, 8192): exp(-2 pi i k / ny);
-// [8192, ...): the row-transformed spectrum between the two passes.
+// [0, 4096): exp(-2 pi i k / nx); [4096, 6144) and [6144, 8192): the stage tables
+// (StageTable in wf_device.cuh, at most 1088 values) of the column and the row
+// transform; [8192, ...): the row-transformed spectrum between the two passes.
+constexpr int kColTable = kMaxSide, kRowTable = kMaxSide + kMaxSide / 2;
 static __device__ __align__(256) float2 wf_static_scratch[kStaticComplex];
 
 constexpr int kMaxDevices = 64;
@@ -37,17 +39,35 @@ std::mutex g_mu;
 float2* g_addr[kMaxDevices] = {};
 
 // twiddles in double precision (sincospi), rounded once to float
-__global__ void static_twiddles(float2* tw, int nx, int ny) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nx) {
-    double s, c;
-    sincospi(2.0 * (double)i / (double)nx, &s, &c);
-    tw[i] = make_float2((float)c, (float)-s);
+__device__ float2 twiddle(int k, int n) {
+  double s, c;
+  sincospi(2.0 * (double)k / (double)n, &s, &c);
+  return make_float2((float)c, (float)-s);
+}
+
+// entry i of the stage table of a length-L transform with E values per thread
+__device__ void stage_entry(float2* tab, int i, int L, int E) {
+  const int p2 = E & -E;
+  int off = 0;
+  for (int ns = 1, r = 0; ns < L; ns *= r) {
+    r = (ns == 1 && L % 3 == 0) ? E : min(p2, L / ns);
+    if (ns == 1) continue;
+    const int n = ns * max(1, r / 4);
+    if (i < off + n) {
+      const int q = (i - off) / ns, jm = (i - off) % ns;
+      tab[i] = twiddle(jm * (L / (ns * r)) * (q ? 4 * q : 1), L);
+      return;
+    }
+    off += n;
   }
-  if (i < ny) {
-    double s, c;
-    sincospi(2.0 * (double)i / (double)ny, &s, &c);
-    tw[kMaxSide + i] = make_float2((float)c, (float)-s);
+}
+
+__global__ void static_twiddles(float2* tw, int nx, int ny, int row_e, int col_e) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nx) tw[i] = twiddle(i, nx);
+  if (i < kMaxSide / 2) {
+    stage_entry(tw + kColTable, i, ny, col_e);
+    stage_entry(tw + kRowTable, i, nx / 2, row_e);
   }
 }
 
@@ -94,25 +114,27 @@ extern "C" int wf_fft2_noalloc(int ny, int nx, const float* in, float* out, int 
   if (rc != WF_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   float2* twx = base;
-  float2* twy = base + kMaxSide;
   float2* spec = base + 2 * kMaxSide;
-  const int nmax = nx > ny ? nx : ny;
+  const int nmax = nx > kMaxSide / 2 ? nx : kMaxSide / 2;
   // launched with cudaLaunchKernelEx, whose return value is this launch's
   // own status (an error some earlier call left pending is not collected)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((nmax + 255) / 256);
   cfg.blockDim = dim3(256);
   cfg.stream = s;
-  if (cudaLaunchKernelEx(&cfg, static_twiddles, base, nx, ny) != cudaSuccess) return WF_ECUDA;
+  if (cudaLaunchKernelEx(&cfg, static_twiddles, base, nx, ny, wf::row_kernel_e(nx / 2), wf::col_kernel_e(ny)) !=
+      cudaSuccess)
+    return WF_ECUDA;
 
   wf::RowArgs ra{};
   ra.ny = ny;
   ra.nx = nx;
   ra.twx = twx;
+  ra.twk = base + kRowTable;
   wf::ColArgs ca{};
   ca.ny = ny;
   ca.nx = nx;
-  ca.twy = twy;
+  ca.twk = base + kColTable;
   if (!inverse) {
     ra.in_px = (const float2*)in;
     ra.out_rf = spec;
