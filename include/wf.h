@@ -153,10 +153,10 @@ typedef struct {
  *                  place.  With refine > 0 a stalled first solve goes on to
  *                  the corrections, and wf_solve then reports WF_OK when the
  *                  refined s passes the stop test.  0 (default): never.
- *  autotune        1 (default): the first problem a plan loads times both
- *                  compiled shapes of each pass (values per thread) on the
- *                  plan's buffers and keeps the faster, cached per device and
- *                  map shape for the process (see wf_plan_shapes); 0: the
+ *  autotune        1 (default): the first problem a plan loads times sweeps
+ *                  with both compiled shapes of each pass (values per thread)
+ *                  on the plan's buffers and keeps the fastest pair, cached per
+ *                  device and map shape for the process (see wf_plan_shapes); 0: the
  *                  first shapes; 2: the second shapes, untimed.  The shape
  *                  changes only the rounding order.
  *  refine_extra    further corrections after the refine ones, each run only
