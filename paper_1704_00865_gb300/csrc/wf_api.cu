@@ -221,8 +221,8 @@ void wf_plan_destroy(wf_plan_t P) {
 
 // True when one sweep's fields (40 bytes per pixel: the row pass's 28 and
 // the column pass's 12) exceed the current device's L2; then the column
-// pass issues L2 prefetch hints one wave ahead (measured at 4096^2: 99.6 ->
-// 96.0 us; the same hints in the row pass made 2048^2 slower).
+// pass issues L2 prefetch hints one wave ahead (measured at 4096^2 with one CTA
+// per SM: 99.6 -> 96.0 us; the same hints in the row pass made 2048^2 slower).
 static bool sweep_above_l2(int ny, int nx) {
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
