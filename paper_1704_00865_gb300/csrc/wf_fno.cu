@@ -1182,12 +1182,17 @@ int launch_synth(wf_fno_s* F, SynthArgs a, int B) {
   return grid;
 }
 
+// Blocks per SM of this network's synthesis (smem a block).  The limit belongs
+// to the kernel on the device, not to the network: every network sets the same
+// one, the most a block can have, or a network of a smaller footprint would
+// take the launches of an earlier one away.
 template <int OG, bool ADJ>
 cudaError_t prepare_synth(size_t smem, int* per_sm) {
   int n0 = 0, n1 = 0;
-  cudaError_t e = cudaFuncSetAttribute(synth<OG, ADJ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e =
+      cudaFuncSetAttribute(synth<OG, ADJ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf::kMaxDynSmem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(synth<OG, ADJ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(synth<OG, ADJ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf::kMaxDynSmem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n0, synth<OG, ADJ, false>, OG * synth_pg(OG), smem);
   if (e == cudaSuccess)
