@@ -1150,8 +1150,7 @@ static int run_setup(wf_plan_t P, const wf_schedule* sch, double tol, CtrlArgs* 
         !(sch->snap >= 1.0))
       return WF_EINVAL;
     c.mode = 1;
-    c.rate_lo = sch->ratio < 1.0 ? pow(1.0 - sch->ratio, R) : 0.0;
-    c.rate_hi = pow(1.0 + sch->ratio, R);
+    c.rate = rate_bounds(sch->ratio, R);
     c.expo = sch->expo;
     c.snap = sch->snap;
     lam0 = sch->lam0;
@@ -1212,7 +1211,7 @@ static int wf_run_on(wf_plan_t P, const wf_schedule* sch, double tol, wf_stats* 
     key.insert(key.end(), b, b + n);
   };
   const long long par = it0 & 1, src = P->has_src ? 1 : 0;
-  put(&c.tol, 8); put(&c.tol_u, 8); put(&c.rate_lo, 8); put(&c.rate_hi, 8); put(&c.expo, 8); put(&c.snap, 8);
+  put(&c.tol, 8); put(&c.tol_u, 8); put(&c.rate, sizeof(c.rate)); put(&c.expo, 8); put(&c.snap, 8);
   put(&c.mode, 4); put(&c.nlevels, 4); put(&c.R, 4); put(&c.max_iters, 4); put(&c.count_iters, 4);
   put(&c.skip_fixed, 4);
   put(&par, 8); put(&src, 8);

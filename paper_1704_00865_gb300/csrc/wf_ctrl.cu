@@ -404,12 +404,10 @@ __global__ void __launch_bounds__(CTRL_THREADS) ctrl_kernel(CtrlArgs a) {
     st->skip_resid = (a.skip_fixed && lam > 1.0 && iter + a.R < a.max_iters) ? 1 : 0;
   } else if (c.lam > 1.0) {
     // Sec. 3.3: lower lambda once Delta d^T Delta d changes by less than
-    // `ratio` per iteration, |1 - q^(1/R)| < ratio for q = rho2 / prev_rho2,
-    // i.e. q between (1 - ratio)^R and (1 + ratio)^R
+    // `ratio` per iteration
     double prev = r2;
     if (c.prev_rho2 > 0 && r2 > 0) {
-      const double q = r2 / c.prev_rho2;
-      if (q > a.rate_lo && q < a.rate_hi) {
+      if (rate_below(a.rate, r2 / c.prev_rho2)) {
         double lam = pow(c.lam, a.expo);
         if (lam < a.snap) lam = 1.0;
         move_to(lam);

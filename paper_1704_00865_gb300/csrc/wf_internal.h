@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/wf.h"
+#include "wf_rate.h"
 
 namespace wf {
 
@@ -356,7 +357,7 @@ struct CtrlArgs {
   const double* lam_sched;    // fixed: device arrays
   const int* it_sched;
   int nlevels;
-  double rate_lo, rate_hi;    // adaptive: (1 -+ ratio)^R
+  RateBounds rate;            // adaptive
   double expo, snap;
   int count_iters;            // add R to iter (0 for a residual-only call)
   int skip_fixed;             // fixed schedule: skip residuals nothing uses (st->skip_resid)
