@@ -23,8 +23,6 @@
 // between them (wf_batch.cu).
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "wf_cols_common.cuh"
 #include "wf_device.cuh"
 #include "wf_internal.h"
@@ -373,10 +371,9 @@ int batch_item_shape(int cls, int* rows_per_item, int* cols_per_item, int* row_v
 // CTAs of a persistent batch launch on the current device (all resident:
 // the cooperative launch requires it), or 0 if it cannot be launched
 int batch_grid() {
-  static std::once_flag once;
-  static cudaError_t cfg_err = cudaSuccess;
-  std::call_once(once, [] {
-    cfg_err = cudaFuncSetAttribute(batch_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
+  static DeviceOnce once;
+  const cudaError_t cfg_err = once.run([](int*) {
+    return cudaFuncSetAttribute(batch_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
   });
   if (cfg_err != cudaSuccess) return 0;
   int dev = 0, sms = 0, coop = 0, per_sm = 0;

@@ -11,8 +11,6 @@
 // barriers an exchange and, at 4096^2, one CTA per SM.
 #pragma once
 
-#include <mutex>
-
 #include "wf_cols_common.cuh"
 
 namespace wf {
@@ -314,15 +312,17 @@ static int launch_col_pass_e(const ColArgs& a, cudaStream_t s) {
   constexpr size_t kBytes = Cfg::bytes + Tc5Smem<L, MODE, EV, PREC>::bytes;
   static_assert(kBytes <= kMaxDynSmem, "column pass staging exceeds shared memory");
   static_assert(PREC < 3 || Cfg::THREADS % 128 == 0, "tcgen05 tiles are 128 threads");
-  // once per instantiation and process (plans may run on several host threads)
-  static std::once_flag once;
-  static cudaError_t cfg_err = cudaSuccess;
-  static int dist = 0;  // CTAs one wave ahead
-  std::call_once(once, [] {
-    cfg_err = cudaFuncSetAttribute(col_pass_kernel<L, MODE, EV, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(kBytes > kSpreadSmem ? kBytes : kSpreadSmem));
-    if (cfg_err == cudaSuccess) dist = resident_ctas(col_pass_kernel<L, MODE, EV, PREC>, Cfg::THREADS, kBytes);
-  });
+  static DeviceOnce once;
+  int dist = 0;  // CTAs one wave ahead
+  const cudaError_t cfg_err = once.run(
+      [](int* ahead) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(col_pass_kernel<L, MODE, EV, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kBytes > kSpreadSmem ? kBytes : kSpreadSmem));
+        if (e == cudaSuccess) *ahead = resident_ctas(col_pass_kernel<L, MODE, EV, PREC>, Cfg::THREADS, kBytes);
+        return e;
+      },
+      &dist);
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid(ncols / Cfg::W), block(Cfg::THREADS);
   ColArgs b = a;

@@ -11,8 +11,6 @@
 // Column 0 packs the two real-signal columns kx = 0 and kx = nx/2 as
 // Z = A + i B (see wf_cols_common.cuh), treated as separate modes with their
 // own eigenvalues.
-#include <mutex>
-
 #include "wf_cols_common.cuh"
 
 namespace wf {
@@ -296,11 +294,9 @@ col_kernel(ColArgs a) {
 template <int L, int MODE>
 static int launch_col_kernel(const ColArgs& a, cudaStream_t s) {
   using Cfg = ColCfg<L>;
-  // once per instantiation and process (plans may run on several host threads)
-  static std::once_flag once;
-  static cudaError_t cfg_err = cudaSuccess;
-  std::call_once(once, [] {
-    cfg_err = cudaFuncSetAttribute(col_kernel<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes);
+  static DeviceOnce once;
+  const cudaError_t cfg_err = once.run([](int*) {
+    return cudaFuncSetAttribute(col_kernel<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes);
   });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid((a.nx / 2 + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);

@@ -28,8 +28,6 @@
 // resident at once (it fails instead of starting otherwise).
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "wf_cols_common.cuh"
 #include "wf_device.cuh"
 #include "wf_internal.h"
@@ -232,11 +230,10 @@ fused_sweep_kernel(FusedArgs a) {
 template <int N, bool SRC>
 static int launch_fused_n(const FusedArgs& a, cudaStream_t s) {
   using F = FusedCfg<N>;
-  static std::once_flag once;
-  static cudaError_t cfg_err = cudaSuccess;
-  std::call_once(once, [] {
-    cfg_err = cudaFuncSetAttribute(fused_sweep_kernel<N, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)F::bytes);
+  static DeviceOnce once;
+  const cudaError_t cfg_err = once.run([](int*) {
+    return cudaFuncSetAttribute(fused_sweep_kernel<N, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)F::bytes);
   });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   cudaLaunchConfig_t cfg = {};

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "../../include/wf.h"
@@ -163,6 +164,35 @@ inline size_t spread_smem(int grid, size_t bytes, int sms) {
   return bytes > want ? bytes : want;
 }
 constexpr size_t kSpreadSmem = kSmSmem / 2 - kCtaSmem + 128;  // the most it asks for
+
+// What the runtime keeps for a kernel (its limit on dynamic shared memory)
+// belongs to the device that was current when it was set: a launcher sets it
+// once on every device it launches on.  setup(value) returns a cudaError_t and
+// may leave a number for the launches of that device.  Plans may run on
+// several host threads.
+class DeviceOnce {
+  static constexpr int kDevices = 64;
+  std::once_flag once_[kDevices];
+  cudaError_t err_[kDevices] = {};
+  int value_[kDevices] = {};
+
+ public:
+  template <typename F>
+  cudaError_t run(F&& setup, int* value = nullptr) {
+    int dev = 0, v = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kDevices) {
+      e = setup(&v);
+    } else {
+      std::call_once(once_[dev], [&] { err_[dev] = setup(&value_[dev]); });
+      e = err_[dev];
+      v = value_[dev];
+    }
+    if (value != nullptr) *value = v;
+    return e;
+  }
+};
 
 // CTAs of a kernel resident at once on the current device (SMs x CTAs per
 // SM for the block and dynamic shared memory), or 0 if the query fails: the

@@ -8,8 +8,6 @@
 // forward row transform, and the stripe-basis updates (eqs. 2mess_d0 and
 // 2mess_t0 analogues: stripe noise, diagonal in the row-wise DFT) follow the
 // forward transform, so a row is read and written once per iteration.
-#include <mutex>
-
 #include "wf_device.cuh"
 #include "wf_internal.h"
 #include "wf_rows_common.cuh"
@@ -426,12 +424,10 @@ template <int M, int MODE, int EV>
 static int launch_row_pass_e(const RowArgs& a, cudaStream_t s) {
   using Cfg = RowPassCfg<M, EV>;
   constexpr size_t bytes = RowPassSmem<M, MODE, EV>::bytes;
-  // once per instantiation and process (plans may run on several host threads)
-  static std::once_flag once;
-  static cudaError_t cfg_err = cudaSuccess;
-  std::call_once(once, [] {
-    cfg_err = cudaFuncSetAttribute(row_pass_kernel<M, MODE, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(bytes > kSpreadSmem ? bytes : kSpreadSmem));
+  static DeviceOnce once;
+  const cudaError_t cfg_err = once.run([](int*) {
+    return cudaFuncSetAttribute(row_pass_kernel<M, MODE, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(bytes > kSpreadSmem ? bytes : kSpreadSmem));
   });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid(a.ny / Cfg::ROWS), block(Cfg::THREADS);
