@@ -16,6 +16,8 @@
 // cudaGetSymbolAddress, with that device current, and handed to the kernels.
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/wf.h"
@@ -62,13 +64,26 @@ __device__ void stage_entry(float2* tab, int i, int L, int E) {
   }
 }
 
-__global__ void static_twiddles(float2* tw, int nx, int ny, int row_e, int col_e) {
+// values in the stage table of a length-L transform with E values per thread
+int stage_size(int L, int E) {
+  const int p2 = E & -E;
+  int n = 0;
+  for (int ns = 1, r = 0; ns < L; ns *= r) {
+    r = (ns == 1 && L % 3 == 0) ? E : std::min(p2, L / ns);
+    if (ns > 1) n += ns * std::max(1, r / 4);
+  }
+  return n;
+}
+
+// A thread makes one entry of the three tables: a sine and cosine in double is
+// a chain of a few microseconds, and the transforms wait for it (with the
+// three entries of a number in one thread a forward and an inverse 1024^2
+// transform took 65 us instead of 53).
+__global__ void static_twiddles(float2* tw, int nx, int ny, int row_e, int col_e, int ncol, int nrow) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nx) tw[i] = twiddle(i, nx);
-  if (i < kMaxSide / 2) {
-    stage_entry(tw + kColTable, i, ny, col_e);
-    stage_entry(tw + kRowTable, i, nx / 2, row_e);
-  }
+  else if (i < nx + ncol) stage_entry(tw + kColTable, i - nx, ny, col_e);
+  else if (i < nx + ncol + nrow) stage_entry(tw + kRowTable, i - nx - ncol, nx / 2, row_e);
 }
 
 // Device address of the array on the current device (set up on first use).
@@ -115,15 +130,15 @@ extern "C" int wf_fft2_noalloc(int ny, int nx, const float* in, float* out, int 
   cudaStream_t s = (cudaStream_t)stream;
   float2* twx = base;
   float2* spec = base + 2 * kMaxSide;
-  const int nmax = nx > kMaxSide / 2 ? nx : kMaxSide / 2;
+  const int row_e = wf::row_kernel_e(nx / 2), col_e = wf::col_kernel_e(ny);
+  const int ncol = stage_size(ny, col_e), nrow = stage_size(nx / 2, row_e);
   // launched with cudaLaunchKernelEx, whose return value is this launch's
   // own status (an error some earlier call left pending is not collected)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((nmax + 255) / 256);
-  cfg.blockDim = dim3(256);
+  cfg.gridDim = dim3((nx + ncol + nrow + 63) / 64);
+  cfg.blockDim = dim3(64);
   cfg.stream = s;
-  if (cudaLaunchKernelEx(&cfg, static_twiddles, base, nx, ny, wf::row_kernel_e(nx / 2), wf::col_kernel_e(ny)) !=
-      cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, static_twiddles, base, nx, ny, row_e, col_e, ncol, nrow) != cudaSuccess)
     return WF_ECUDA;
 
   wf::RowArgs ra{};
