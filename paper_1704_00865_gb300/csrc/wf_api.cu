@@ -1340,12 +1340,10 @@ int wf_get_field(wf_plan_t P, int field, float* out) {
     case WF_FIELD_T_2DF: {
       if (!P->has_f || P->merge) return WF_EINVAL;
       ColArgs ca = col_args(P, 0);
-      ca.in = P->f_t0;  // column-tiled: to row-major first, then in place
+      ca.in = P->f_t0;
       ca.out = P->r_g;
-      CKI(launch_col(COL_UNTILE, ca, P->stream));
-      ca.in = P->r_g;
-      CKI(launch_col(COL_INV, ca, P->stream));
-      P->launches += 2;
+      CKI(launch_col(COL_INV_TILED, ca, P->stream));
+      P->launches += 1;
       ra.in_rf = P->r_g;
       break;
     }

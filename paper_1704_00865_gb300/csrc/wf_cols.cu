@@ -36,7 +36,9 @@ struct ColCfg {
 // long columns share an SM
 template <int L, int MODE>
 constexpr int col_min_ctas() {
-  return (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED) && L >= 1024 ? 1024 / ColCfg<L>::THREADS : 1;
+  return (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED || MODE == COL_INV_TILED) && L >= 1024
+             ? 1024 / ColCfg<L>::THREADS
+             : 1;
 }
 
 template <int L, int MODE>
@@ -276,11 +278,13 @@ col_kernel(ColArgs a) {
 #pragma unroll
       for (int m = 0; m < E; ++m) a.out[at(t + m * TPC)] = a.in[att(t + m * TPC)];
     }
-  } else if constexpr (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED) {
+  } else if constexpr (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED || MODE == COL_INV_TILED) {
+    constexpr bool INV = (MODE == COL_INV || MODE == COL_INV_TILED), TILED_IN = (MODE == COL_INV_TILED);
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = valid ? a.in[at(t + m * TPC)] : make_float2(0.f, 0.f);
-    fft_staged<L, E, MODE == COL_INV>(v, sb, t, a.twk);
-    const float sc = (MODE == COL_INV) ? 1.0f / (float)L : 1.0f;
+    for (int m = 0; m < E; ++m)
+      v[m] = valid ? a.in[TILED_IN ? att(t + m * TPC) : at(t + m * TPC)] : make_float2(0.f, 0.f);
+    fft_staged<L, E, INV>(v, sb, t, a.twk);
+    const float sc = INV ? 1.0f / (float)L : 1.0f;
     if (valid) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
@@ -318,6 +322,7 @@ static int launch_col_L(int mode, const ColArgs& a, cudaStream_t s) {
     case COL_UNTILE: return launch_col_kernel<L, COL_UNTILE>(a, s);
     case COL_FWD_TILED: return launch_col_kernel<L, COL_FWD_TILED>(a, s);
     case COL_WARM: return launch_col_kernel<L, COL_WARM>(a, s);
+    case COL_INV_TILED: return launch_col_kernel<L, COL_INV_TILED>(a, s);
     default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();

@@ -79,7 +79,7 @@ enum ColMode : int {
   COL_FWD_TILED = 9,  // RF -> 2D Fourier, column-tiled output
   COL_PASS_MERGE_SRC = 10,  // COL_PASS_MERGE with a source term (defect correction)
   COL_WARM = 11,      // warm start: s in RF -> the signal-side field (tiled) and a tiled copy
-  COL_NMODES = 11
+  COL_INV_TILED = 12, // COL_INV of a column-tiled field (row-major output)
 };
 
 struct RowArgs {
