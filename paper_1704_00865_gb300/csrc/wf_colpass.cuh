@@ -96,8 +96,11 @@ __device__ __forceinline__ uint64_t* tc5_mbar(unsigned char* smem) {
 // forward and inverse column DFTs).  d_2DF goes straight from the registers of
 // the last stage to global memory (a warp covers 8 rows of a tile, 256
 // contiguous bytes), at 4096 the messenger and the tables come the same way.
-template <int L, int MODE, int EV, int PREC = 0>
-__global__ void __launch_bounds__(ColPassCfg<L, MODE, EV, PREC>::THREADS, PREC ? 1 : ColPassCfg<L, MODE, EV, PREC>::min_ctas)
+// ONE: compiled for one CTA per SM (the plain sweep's unstaged columns on a grid
+// that gives an SM no second one).
+template <int L, int MODE, int EV, int PREC = 0, bool ONE = false>
+__global__ void __launch_bounds__(ColPassCfg<L, MODE, EV, PREC>::THREADS,
+                                  PREC || ONE ? 1 : ColPassCfg<L, MODE, EV, PREC>::min_ctas)
 col_pass_kernel(ColArgs a) {
   using Cfg = ColPassCfg<L, MODE, EV, PREC>;
   constexpr int E = Cfg::E, TPC = Cfg::TPC, W = Cfg::W;
@@ -206,11 +209,19 @@ col_pass_kernel(ColArgs a) {
   else fft_staged<L, E, false, false, Cfg::TWS>(v, sb, t, Cfg::TWS ? s_tw : a.tws);
 
   // partner values Z[-k] for the packed column 0, read below from shared
-  // memory (CTA 0 only; uniform)
+  // memory (CTA 0 only; uniform).  Unstaged, t_2DF's partners too, since the
+  // update overwrites the field: column 1's buffer is free for them (held in
+  // registers they spilled 344 bytes a thread: 22.3 us a sweep at 4096 x 32)
+  constexpr bool T0_DIRECT = Cfg::T0 && !STAGED;
+  static_assert(!T0_DIRECT || W > 1, "a second buffer for the partners of t_2DF");
   if (blockIdx.x == 0) {
     if constexpr (!Cfg::PP) __syncthreads();
 #pragma unroll
-    for (int m = 0; m < E; ++m) sb[spad(t + m * TPC)] = v[m];
+    for (int m = 0; m < E; ++m) {
+      const int k = t + m * TPC;
+      if constexpr (T0_DIRECT) sb[spad(k)] = c == 0 ? v[m] : a.f_t0[tile0 + (size_t)k * WF_TW];
+      else sb[spad(k)] = v[m];
+    }
     __syncthreads();
   }
 
@@ -238,14 +249,7 @@ col_pass_kernel(ColArgs a) {
       }
     }
   } else {
-    // the CTA of the packed column.  Partners of t_2DF are overwritten below:
-    // read them first
-    float2 tp[Cfg::T0 ? E : 1];
-    if constexpr (Cfg::T0 && !STAGED) {
-#pragma unroll
-      for (int m = 0; m < E; ++m) tp[m] = third(neg_mod<L>(t + m * TPC));
-      __syncthreads();
-    }
+    // the CTA of the packed column
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const int k = t + m * TPC;
@@ -262,7 +266,7 @@ col_pass_kernel(ColArgs a) {
         v[m] = merged_pair<SRC>(v[m], vp, e, egn, off0, Tl, jv, jp);
       } else {
         const float2 t0o = third(k);
-        const float2 t0p = STAGED ? third(neg_mod<L>(k)) : tp[Cfg::T0 ? m : 0];
+        const float2 t0p = STAGED ? third(neg_mod<L>(k)) : s_fft[Cfg::STRIDE + spad(neg_mod<L>(k))];
         // (the pair is formed by every lane and kept by the packed column's)
         float2 yA, yB, tA, tB, tnA, tnB;
         unpack_pair(v[m], vp, yA, yB);
@@ -304,30 +308,41 @@ col_pass_kernel(ColArgs a) {
   for (int m = 0; m < E; ++m) a.f_x[at0 + (size_t)(t + m * TPC) * WF_TW] = cscale(v[m], sc);
 }
 
+template <int L, int MODE, int EV, int PREC, bool ONE>
+static int launch_col_pass_one(const ColArgs& a, cudaStream_t s) {
+  using Cfg = ColPassCfg<L, MODE, EV, PREC>;
+  constexpr size_t kBytes = Cfg::bytes + Tc5Smem<L, MODE, EV, PREC>::bytes;
+  static_assert(kBytes <= kMaxDynSmem, "column pass staging exceeds shared memory");
+  static_assert(PREC < 3 || Cfg::THREADS % 128 == 0, "tcgen05 tiles are 128 threads");
+  constexpr auto kernel = col_pass_kernel<L, MODE, EV, PREC, ONE>;
+  static DeviceOnce once;
+  int dist = 0;  // CTAs one wave ahead
+  const cudaError_t cfg_err = once.run(
+      [](int* ahead) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(kBytes > kSpreadSmem ? kBytes : kSpreadSmem));
+        if (e == cudaSuccess) *ahead = resident_ctas(kernel, Cfg::THREADS, kBytes);
+        return e;
+      },
+      &dist);
+  if (cfg_err != cudaSuccess) return (int)cfg_err;
+  const dim3 grid(a.nx / 2 / Cfg::W), block(Cfg::THREADS);
+  ColArgs b = a;
+  b.pf = a.prefetch ? dist : 0;
+  return launch_pdl(kernel, grid, block, spread_smem(grid.x, kBytes, a.sms), s, b);
+}
+
 template <int L, int MODE, int EV, int PREC = 0>
 static int launch_col_pass_e(const ColArgs& a, cudaStream_t s) {
   using Cfg = ColPassCfg<L, MODE, EV, PREC>;
   const int ncols = a.nx / 2;
   if (ncols % Cfg::W != 0) return (int)cudaErrorInvalidValue;
-  constexpr size_t kBytes = Cfg::bytes + Tc5Smem<L, MODE, EV, PREC>::bytes;
-  static_assert(kBytes <= kMaxDynSmem, "column pass staging exceeds shared memory");
-  static_assert(PREC < 3 || Cfg::THREADS % 128 == 0, "tcgen05 tiles are 128 threads");
-  static DeviceOnce once;
-  int dist = 0;  // CTAs one wave ahead
-  const cudaError_t cfg_err = once.run(
-      [](int* ahead) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(col_pass_kernel<L, MODE, EV, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kBytes > kSpreadSmem ? kBytes : kSpreadSmem));
-        if (e == cudaSuccess) *ahead = resident_ctas(col_pass_kernel<L, MODE, EV, PREC>, Cfg::THREADS, kBytes);
-        return e;
-      },
-      &dist);
-  if (cfg_err != cudaSuccess) return (int)cfg_err;
-  const dim3 grid(ncols / Cfg::W), block(Cfg::THREADS);
-  ColArgs b = a;
-  b.pf = a.prefetch ? dist : 0;
-  return launch_pdl(col_pass_kernel<L, MODE, EV, PREC>, grid, block, spread_smem(grid.x, kBytes, a.sms), s, b);
+  // t_2DF, (C, P1f) and the values of an unstaged column do not fit in the 64
+  // registers that two CTAs per SM leave (56 bytes spilled, the loads in
+  // several batches): with no more CTAs than SMs there is nothing to trade
+  if constexpr (Cfg::T0 && !Cfg::STAGED)
+    if (ncols / Cfg::W <= kSms) return launch_col_pass_one<L, MODE, EV, PREC, true>(a, s);
+  return launch_col_pass_one<L, MODE, EV, PREC, false>(a, s);
 }
 
 }  // namespace wf

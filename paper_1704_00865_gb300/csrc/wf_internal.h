@@ -144,6 +144,8 @@ struct ColArgs {
   int sms;                    // as in RowArgs
 };
 
+constexpr int kSms = 152;  // SMs of a GB300
+
 // Dynamic shared memory per CTA and per SM (1 KB of it reserved per CTA).
 constexpr size_t kMaxDynSmem = 227 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024;
 
