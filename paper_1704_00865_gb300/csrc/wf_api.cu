@@ -514,6 +514,7 @@ static ColArgs col_args(wf_plan_s* P, int parity) {
   a.variant = a.prec ? 0 : P->col_variant;  // the tensor-core stages use the 16-value shape
   a.prefetch = P->l2_prefetch;
   a.sms = P->sms;
+  a.row_ctas = P->ny / row_pass_rows(P->M, P->row_variant);
   a.ny = P->ny;
   a.nx = P->nx;
   a.has_rf = P->has_rf;

@@ -329,7 +329,7 @@ static int launch_col_pass_one(const ColArgs& a, cudaStream_t s) {
   const dim3 grid(a.nx / 2 / Cfg::W), block(Cfg::THREADS);
   ColArgs b = a;
   b.pf = a.prefetch ? dist : 0;
-  return launch_pdl(kernel, grid, block, spread_smem(grid.x, kBytes, a.sms), s, b);
+  return launch_pdl(kernel, grid, block, spread_cols_smem(grid.x, kBytes, a.sms, a.row_ctas), s, b);
 }
 
 template <int L, int MODE, int EV, int PREC = 0>
