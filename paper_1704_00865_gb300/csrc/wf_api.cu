@@ -87,7 +87,8 @@ struct wf_plan_s {
   bool tuned = false;
   // the row pass's tensor maps of the column-tiled fields, per shape
   CUtensorMap tm_t[2], tm_x[2];
-  int sms = 0;              // SMs the passes' CTAs are spread over (0: other plans run beside this one)
+  int sms = 0;              // SMs of the device, over which the passes' CTAs are spread
+  bool shares_gpu = false;  // unless other plans run beside this one
   // the column pass hints the next wave's tiles into L2 (maps whose sweep
   // moves more bytes than L2 holds)
   bool l2_prefetch = false;
@@ -484,7 +485,7 @@ int wf_plan_create(wf_plan_t* out, int ny, int nx, unsigned parts, const wf_para
 static RowArgs row_args(wf_plan_s* P) {
   RowArgs a{};
   a.variant = P->row_variant;
-  a.sms = P->sms;
+  a.sms = P->shares_gpu ? 0 : P->sms;
   a.tm_t = P->tm_t[P->row_variant];
   a.tm_x = P->tm_x[P->row_variant];
   a.ny = P->ny;
@@ -513,7 +514,7 @@ static ColArgs col_args(wf_plan_s* P, int parity) {
   a.prec = P->p.dft_precision;
   a.variant = a.prec ? 0 : P->col_variant;  // the tensor-core stages use the 16-value shape
   a.prefetch = P->l2_prefetch;
-  a.sms = P->sms;
+  a.sms = P->shares_gpu ? 0 : P->sms;
   a.row_ctas = P->ny / row_pass_rows(P->M, P->row_variant);
   a.ny = P->ny;
   a.nx = P->nx;
@@ -743,6 +744,10 @@ static int autotune(wf_plan_s* P) {
     if (!rc && cudaMemcpyAsync(P->st_save, P->st, sizeof(WfState), cudaMemcpyDeviceToDevice, P->stream) != cudaSuccess)
       rc = WF_ECUDA;
     if (!rc && launch_set_lambda(P->st, 1.0, 1, P->stream)) rc = WF_ECUDA;
+    // as a plan of its own runs them, also for a batch's plan: the answer is
+    // kept for both, and a batch gives what its maps give alone, bit for bit
+    const bool shares = P->shares_gpu;
+    P->shares_gpu = false;
     double least = 0.0;
     for (int r = 0; r < (two_rows ? 2 : 1) && !rc; ++r)
       for (int c = 0; c < (two_cols ? 2 : 1) && !rc; ++c) {
@@ -757,6 +762,7 @@ static int autotune(wf_plan_s* P) {
         }
       }
     P->row_variant = P->col_variant = 0;
+    P->shares_gpu = shares;
     if (!rc && cudaMemcpyAsync(P->st, P->st_save, sizeof(WfState), cudaMemcpyDeviceToDevice, P->stream) != cudaSuccess)
       rc = WF_ECUDA;
     const size_t nhb = (size_t)P->ny * P->M * sizeof(float2);
@@ -914,7 +920,7 @@ bool wf::plan_batch_ok(const wf_plan_t P) {
 }
 
 int wf::plan_size(const wf_plan_t P) { return P->ny; }
-void wf::plan_shares_gpu(wf_plan_t P) { P->sms = 0; }
+void wf::plan_shares_gpu(wf_plan_t P) { P->shares_gpu = true; }
 int wf::plan_autotune(const wf_plan_t P) { return P->p.autotune; }
 
 // Runs the iteration of several loaded plans together (wf_run for each, with
