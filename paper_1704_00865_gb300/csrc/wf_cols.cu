@@ -15,13 +15,15 @@
 
 namespace wf {
 
-template <int L>
+// NARROW (long columns): at most 256 threads, one or two columns per CTA.
+template <int L, bool NARROW = false>
 struct ColCfg {
   static constexpr int E = col_kernel_e(L);
   static constexpr int TPC = L / E;
   // whole tiles, 32-byte pieces of the row-major fields (half of that at 4096,
   // where four columns would not fit)
-  static constexpr int W = TPC < 16 ? 64 / TPC : (L >= 4096 ? 2 : WF_TW);
+  static constexpr int W = NARROW ? 256 / TPC : TPC < 16 ? 64 / TPC : (L >= 4096 ? 2 : WF_TW);
+  static_assert(!NARROW || (TPC >= 128 && TPC <= 256), "one or two long columns");
   static constexpr int THREADS = W * TPC;
   // Stride between the per-column FFT buffers (complex values): a half-warp
   // covers W columns x 16/W consecutive indices, which are bank-conflict free
@@ -34,17 +36,17 @@ struct ColCfg {
 
 // the plain transforms are held to 64 registers a thread, so that two CTAs of
 // long columns share an SM
-template <int L, int MODE>
+template <int L, int MODE, bool NARROW>
 constexpr int col_min_ctas() {
-  return (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED || MODE == COL_INV_TILED) && L >= 1024
+  return (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED || MODE == COL_INV_TILED) && L >= 1024 && !NARROW
              ? 1024 / ColCfg<L>::THREADS
              : 1;
 }
 
-template <int L, int MODE>
-__global__ void __launch_bounds__(ColCfg<L>::THREADS, col_min_ctas<L, MODE>())
+template <int L, int MODE, bool NARROW = false>
+__global__ void __launch_bounds__(ColCfg<L, NARROW>::THREADS, col_min_ctas<L, MODE, NARROW>())
 col_kernel(ColArgs a) {
-  using Cfg = ColCfg<L>;
+  using Cfg = ColCfg<L, NARROW>;
   constexpr int E = Cfg::E, TPC = Cfg::TPC, W = Cfg::W;
   extern __shared__ __align__(16) float2 sbuf[];  // [W][STRIDE]
 
@@ -295,16 +297,27 @@ col_kernel(ColArgs a) {
   }
 }
 
-template <int L, int MODE>
-static int launch_col_kernel(const ColArgs& a, cudaStream_t s) {
-  using Cfg = ColCfg<L>;
+template <int L, int MODE, bool NARROW>
+static int launch_col_kernel_w(const ColArgs& a, cudaStream_t s) {
+  using Cfg = ColCfg<L, NARROW>;
+  constexpr auto kernel = col_kernel<L, MODE, NARROW>;
   static DeviceOnce once;
-  const cudaError_t cfg_err = once.run([](int*) {
-    return cudaFuncSetAttribute(col_kernel<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes);
-  });
+  const cudaError_t cfg_err = once.run(
+      [](int*) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes); });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid((a.nx / 2 + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);
-  return launch_pdl(col_kernel<L, MODE>, grid, block, Cfg::bytes, s, a);
+  return launch_pdl(kernel, grid, block, Cfg::bytes, s, a);
+}
+
+template <int L, int MODE>
+static int launch_col_kernel(const ColArgs& a, cudaStream_t s) {
+  // Narrow CTAs while there are no more of them than SMs: with wider ones half
+  // the SMs stay idle (a forward and an inverse transform of 2048 x 512 59.6 us,
+  // 51.7 narrow; of 4096 x 256 69.3 and 58.2).  Beyond, whole 32-byte pieces count
+  // (4096 x 1024: 87.8 us, 107 narrow).  1024-long columns take 10 us either way.
+  if constexpr (L >= 1536)
+    if (a.nx / 2 / ColCfg<L, true>::W <= kSms) return launch_col_kernel_w<L, MODE, true>(a, s);
+  return launch_col_kernel_w<L, MODE, false>(a, s);
 }
 
 template <int L>
