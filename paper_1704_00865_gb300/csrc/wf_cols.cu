@@ -306,7 +306,8 @@ static int launch_col_kernel_w(const ColArgs& a, cudaStream_t s) {
       [](int*) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes); });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
   const dim3 grid((a.nx / 2 + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);
-  return launch_pdl(kernel, grid, block, Cfg::bytes, s, a);
+  const bool whole = (MODE == COL_RESID_A || MODE == COL_RESID_C) && whole_split(a.ny, a.nx, a.sms);
+  return launch_pdl_split(whole, kernel, grid, block, Cfg::bytes, s, a);
 }
 
 template <int L, int MODE>

@@ -34,21 +34,27 @@ constexpr int WF_TW = 4;
 #define WF_PDL 1
 #endif
 template <typename... KArgs, typename... Args>
-inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                      Args... args) {
+inline int launch_pdl_split(bool whole, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                            Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = WF_PDL;
+  at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;  // with `whole`: all of it shared memory
+  at[1].val.sharedMemCarveout = 100;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = whole ? 2 : 1;
   // the return value is this launch's own status (an error left pending by
   // an earlier, unrelated call is not collected here)
   return (int)cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+  return launch_pdl_split(false, kernel, grid, block, smem, s, args...);
 }
 __host__ __device__ __forceinline__ size_t tidx(int y, int kx, int ny) {
   return (size_t)(kx / WF_TW) * ny * WF_TW + (size_t)y * WF_TW + (kx % WF_TW);
@@ -147,6 +153,8 @@ struct ColArgs {
 
 constexpr int kSms = 152;  // SMs of a GB300
 
+int row_grid(int nx, int ny);  // CTAs of a residual row kernel (size of partial-sum arrays)
+
 // Dynamic shared memory per CTA and per SM (1 KB of it reserved per CTA).
 constexpr size_t kMaxDynSmem = 227 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024;
 
@@ -171,6 +179,18 @@ inline size_t spread_smem(int grid, size_t bytes, int sms) {
 // white 5.7 us a sweep instead of 7.7, three parts 7.0 instead of 7.9).
 inline size_t spread_cols_smem(int grid, size_t bytes, int sms, int row_ctas) {
   return spread_smem(grid, bytes, grid <= sms && row_ctas > sms && row_ctas <= 2 * sms ? 0 : sms);
+}
+// An SM divides its 256 KB between L1 and shared memory and changes that only
+// when it is empty, so a kernel does not start beside one of another split.
+// Left to the driver, the residual's kernels (a few KB a CTA) get another one
+// than the passes that ask for tens of KB to spread, and a checkpoint waits for
+// the changes.  With a hundred row CTAs and more, on maps small enough that
+// this counts, they ask for all of it as shared memory: a checkpoint of 512 x
+// 1024 white noise 41.3 us instead of 45.6 (39.5 beside unspread passes), of
+// 1024 x 128 29.1 instead of 38.4.  Larger maps miss the L1 (2048^2: a residual 199
+// us instead of 187), smaller ones gain nothing.
+inline bool whole_split(int ny, int nx, int sms) {
+  return sms > 0 && row_grid(nx, ny) >= 128 && (size_t)ny * nx <= (size_t)1 << 19;
 }
 constexpr size_t kSpreadSmem = kSmSmem / 2 - kCtaSmem + 128;  // the most it asks for
 
@@ -220,7 +240,6 @@ int resident_ctas(K kernel, int threads, size_t smem) {
 // launchers (return a cudaError_t as int)
 int launch_row(int mode, const RowArgs& a, cudaStream_t s);
 int launch_col(int mode, const ColArgs& a, cudaStream_t s);
-int row_grid(int nx, int ny);  // CTAs of a row pass (size of partial-sum arrays)
 bool size_supported(int n);
 // argument checks of wf_plan_create (host only; WF_OK or a WF_E* code)
 int check_plan_args(int ny, int nx, unsigned parts, const wf_params* p);

@@ -447,11 +447,12 @@ template <int M>
 static int launch_row_M(int mode, const RowArgs& a, cudaStream_t s) {
   using Cfg = RowCfg<M>;
   const dim3 grid((a.ny + Cfg::ROWS - 1) / Cfg::ROWS), block(Cfg::THREADS);
+  const bool whole = whole_split(a.ny, a.nx, a.sms);
   switch (mode) {
     case ROW_PASS_RF: return launch_row_pass<M, ROW_PASS_RF>(a, s);
     case ROW_PASS_NORF: return launch_row_pass<M, ROW_PASS_NORF>(a, s);
-    case ROW_RESID_B: return launch_pdl(row_kernel<M, ROW_RESID_B>, grid, block, 0, s, a);
-    case ROW_RESID_D: return launch_pdl(row_kernel<M, ROW_RESID_D>, grid, block, 0, s, a);
+    case ROW_RESID_B: return launch_pdl_split(whole, row_kernel<M, ROW_RESID_B>, grid, block, 0, s, a);
+    case ROW_RESID_D: return launch_pdl_split(whole, row_kernel<M, ROW_RESID_D>, grid, block, 0, s, a);
     case ROW_C2R: return launch_pdl(row_kernel<M, ROW_C2R>, grid, block, 0, s, a);
     case ROW_R2C: return launch_pdl(row_kernel<M, ROW_R2C>, grid, block, 0, s, a);
     default: return (int)cudaErrorInvalidValue;

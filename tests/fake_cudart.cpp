@@ -20,6 +20,7 @@ struct Launch {
   std::string name;
   size_t smem;
   bool refused;
+  int carveout;  // preferred share of shared memory in percent, -1 without one
 };
 std::mutex mu;
 std::map<const void*, std::string>& names() {  // built before any static constructor registers a kernel
@@ -34,12 +35,12 @@ int device = 0;
 const size_t kDefault = 48 * 1024, kOptin = 227 * 1024, kSm = 228 * 1024;
 thread_local struct { dim3 grid, block; size_t smem; cudaStream_t s; } call;
 
-cudaError_t launch(const void* f, size_t smem) {
+cudaError_t launch(const void* f, size_t smem, int carveout = -1) {
   std::lock_guard<std::mutex> lk(mu);
   auto it = limit.find({f, device});
   const bool refused = smem > (it == limit.end() ? kDefault : it->second);
   auto n = names().find(f);
-  launches.push_back({device, n == names().end() ? "?" : n->second, smem, refused});
+  launches.push_back({device, n == names().end() ? "?" : n->second, smem, refused, carveout});
   return refused ? cudaErrorInvalidValue : cudaSuccess;
 }
 cudaError_t allocate(void** p, size_t n) {
@@ -63,6 +64,7 @@ void* fake_alloc(size_t n) {
   return p;
 }
 int fake_launches(void) { return (int)launches.size(); }
+int fake_carveout(int i) { return launches[i].carveout; }
 const char* fake_launch(int i, int* dev, size_t* smem, int* refused) {
   *dev = launches[i].dev;
   *smem = launches[i].smem;
@@ -100,7 +102,10 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, 
   return e;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
-  const cudaError_t e = launch(f, c->dynamicSmemBytes);
+  int carveout = -1;
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    if (c->attrs[i].id == cudaLaunchAttributePreferredSharedMemoryCarveout) carveout = (int)c->attrs[i].val.sharedMemCarveout;
+  const cudaError_t e = launch(f, c->dynamicSmemBytes, carveout);
   if (e != cudaSuccess) last = e;
   return e;
 }
