@@ -493,13 +493,9 @@ static RowArgs row_args(wf_plan_s* P) {
   a.has_rf = P->has_rf;
   a.dn = P->dn;
   a.f_d1 = P->f_d1;
-  a.f_t1 = P->f_t1;
-  a.f_x = P->f_x;
-  a.f_y = P->f_y;
   a.pst = P->pst;
   a.a2 = P->a2;
   a.twx = P->twx;
-  a.twh = P->twh;
   a.tws = P->tws_row[P->row_variant];
   a.twk = P->twk_row;
   a.st = P->st;

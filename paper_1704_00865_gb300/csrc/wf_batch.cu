@@ -32,7 +32,6 @@
 #include <mutex>
 #include <numeric>
 #include <thread>
-
 #include <vector>
 
 #include "../../include/wf.h"

@@ -53,9 +53,7 @@ col_kernel(ColArgs a) {
   const int c = threadIdx.x % W;
   const int t = threadIdx.x / W;
   const int ncols = a.nx / 2;
-  const int col = blockIdx.x * W + c;
-  constexpr bool valid = true;  // ncols is a multiple of W
-  const int colv = col;
+  const int col = blockIdx.x * W + c;  // ncols is a multiple of W
   float2* sb = sbuf + c * Cfg::STRIDE;
 
   pdl_trigger();
@@ -64,17 +62,17 @@ col_kernel(ColArgs a) {
   float2 eg0[PRE ? E : 1];
   if constexpr (PRE) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) eg0[m] = valid ? __ldg(&a.eig[tidx(t + m * TPC, colv, a.ny)]) : make_float2(1.f, 0.f);
+    for (int m = 0; m < E; ++m) eg0[m] = __ldg(&a.eig[tidx(t + m * TPC, col, a.ny)]);
   }
   pdl_wait();
   // uniform: both flags are set only between launches
   if ((a.check_done && a.st->done) || (a.skip_ok && a.st->skip_resid)) return;
 
   auto eig_at = [&](int m) -> float2 {
-    return PRE ? eg0[PRE ? m : 0] : (valid ? a.eig[tidx(t + m * TPC, colv, a.ny)] : make_float2(1.f, 0.f));
+    return PRE ? eg0[PRE ? m : 0] : a.eig[tidx(t + m * TPC, col, a.ny)];
   };
-  auto at = [&](int k) -> size_t { return (size_t)k * ncols + colv; };       // row-major
-  auto att = [&](int k) -> size_t { return tidx(k, colv, a.ny); };           // column-tiled
+  auto at = [&](int k) -> size_t { return (size_t)k * ncols + col; };       // row-major
+  auto att = [&](int k) -> size_t { return tidx(k, col, a.ny); };           // column-tiled
   float2 v[E];
 
   // Partner value Z[-k] of column 0 (only meaningful where col == 0).  Every
@@ -118,14 +116,14 @@ col_kernel(ColArgs a) {
       const float off0 = (float)a.st->off[0];
       float2 w[E];
 #pragma unroll
-      for (int m = 0; m < E; ++m) v[m] = valid ? a.f_y[att(t + m * TPC)] : make_float2(0.f, 0.f);
+      for (int m = 0; m < E; ++m) v[m] = a.f_y[att(t + m * TPC)];
       fft_staged<L, E, false>(v, sb, t, a.twk);
       if (blockIdx.x == 0) exchange0(v, vp);
       each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
         const float2 eg = eig_at(m);
         // with a source j: g = (y + (N0 + T) j^) / (C + N0 + T)
-        const float2 jv = (a.src != nullptr && valid) ? a.src[att(k)] : make_float2(0.f, 0.f);
+        const float2 jv = (a.src != nullptr) ? a.src[att(k)] : make_float2(0.f, 0.f);
         if (pk) {
           const float2 egb = a.eig_nyq[k];
           const float2 jp = (a.src != nullptr) ? a.src[att(neg_mod<L>(k))] : make_float2(0.f, 0.f);
@@ -147,16 +145,14 @@ col_kernel(ColArgs a) {
       });
       fft_staged<L, E, true>(v, sb, t, a.twk);
       fft_staged<L, E, true>(w, sb, t, a.twk);
-      if (valid) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-          a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
-          a.r_q[at(t + m * TPC)] = cscale(w[m], sc);
-        }
+      for (int m = 0; m < E; ++m) {
+        a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
+        a.r_q[at(t + m * TPC)] = cscale(w[m], sc);
       }
     } else if (a.has_f) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) v[m] = valid ? a.f_t0[att(t + m * TPC)] : make_float2(0.f, 0.f);
+      for (int m = 0; m < E; ++m) v[m] = a.f_t0[att(t + m * TPC)];
       const float T0s = a.st->T0s[a.parity];
       float2 w[E];
       each_mode([&](int m, bool pk) {
@@ -179,19 +175,17 @@ col_kernel(ColArgs a) {
       });
       fft_staged<L, E, true>(v, sb, t, a.twk);
       fft_staged<L, E, true>(w, sb, t, a.twk);
-      if (valid) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-          a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
-          a.r_q[at(t + m * TPC)] = cscale(w[m], sc);
-        }
+      for (int m = 0; m < E; ++m) {
+        a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
+        a.r_q[at(t + m * TPC)] = cscale(w[m], sc);
       }
     }
   } else if constexpr (MODE == COL_RESID_C) {
     // q += N_2DF g'  (the given 1/f eigenvalues)
     float2 vp[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = valid ? a.r_g[at(t + m * TPC)] : make_float2(0.f, 0.f);
+    for (int m = 0; m < E; ++m) v[m] = a.r_g[at(t + m * TPC)];
     fft_staged<L, E, false>(v, sb, t, a.twk);
     if (blockIdx.x == 0) exchange0(v, vp);
     each_mode([&](int m, bool pk) {
@@ -207,19 +201,17 @@ col_kernel(ColArgs a) {
     });
     fft_staged<L, E, true>(v, sb, t, a.twk);
     const float sc = 1.0f / (float)L;
-    if (valid) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) {
-        const size_t i = at(t + m * TPC);
-        const float2 q = a.r_q[i];
-        a.r_q[i] = make_float2(fmaf(v[m].x, sc, q.x), fmaf(v[m].y, sc, q.y));
-      }
+    for (int m = 0; m < E; ++m) {
+      const size_t i = at(t + m * TPC);
+      const float2 q = a.r_q[i];
+      a.r_q[i] = make_float2(fmaf(v[m].x, sc, q.x), fmaf(v[m].y, sc, q.y));
     }
   } else if constexpr (MODE == COL_G_FROM_S) {
     // residual of a given s: r_q holds s in RF (kept); r_g <- S^-1 s in RF
     float2 vp[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = valid ? a.r_q[at(t + m * TPC)] : make_float2(0.f, 0.f);
+    for (int m = 0; m < E; ++m) v[m] = a.r_q[at(t + m * TPC)];
     fft_staged<L, E, false>(v, sb, t, a.twk);
     if (blockIdx.x == 0) exchange0(v, vp);
     each_mode([&](int m, bool pk) {
@@ -235,10 +227,8 @@ col_kernel(ColArgs a) {
     });
     fft_staged<L, E, true>(v, sb, t, a.twk);
     const float sc = 1.0f / (float)L;
-    if (valid) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
-    }
+    for (int m = 0; m < E; ++m) a.r_g[at(t + m * TPC)] = cscale(v[m], sc);
   } else if constexpr (MODE == COL_WARM) {
     // warm start from s (in RF, row-major in a.in): the data-side messenger
     // gets s itself (tiled copy), the signal-side field d_2DF = (C + N_0)/C s
@@ -246,8 +236,8 @@ col_kernel(ColArgs a) {
     float2 vp[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      v[m] = valid ? a.in[at(t + m * TPC)] : make_float2(0.f, 0.f);
-      if (valid) a.warm_copy[att(t + m * TPC)] = v[m];
+      v[m] = a.in[at(t + m * TPC)];
+      a.warm_copy[att(t + m * TPC)] = v[m];
     }
     if (a.has_f) {
       const float off0 = (float)a.st->off[0];
@@ -255,7 +245,7 @@ col_kernel(ColArgs a) {
       if (blockIdx.x == 0) exchange0(v, vp);
       each_mode([&](int m, bool pk) {
         const int k = t + m * TPC;
-        const float2 eg = valid ? a.eig[att(k)] : make_float2(1.f, 0.f);
+        const float2 eg = a.eig[att(k)];
         const float fa = __fdividef(eg.x + eg.y + off0, eg.x);
         if (pk) {
           const float2 egb = a.eig_nyq[k];
@@ -271,28 +261,22 @@ col_kernel(ColArgs a) {
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = cscale(v[m], sc);
     }
-    if (valid) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) a.out[att(t + m * TPC)] = v[m];
-    }
+    for (int m = 0; m < E; ++m) a.out[att(t + m * TPC)] = v[m];
   } else if constexpr (MODE == COL_UNTILE) {
-    if (valid) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) a.out[at(t + m * TPC)] = a.in[att(t + m * TPC)];
-    }
+    for (int m = 0; m < E; ++m) a.out[at(t + m * TPC)] = a.in[att(t + m * TPC)];
   } else if constexpr (MODE == COL_FWD || MODE == COL_INV || MODE == COL_FWD_TILED || MODE == COL_INV_TILED) {
     constexpr bool INV = (MODE == COL_INV || MODE == COL_INV_TILED), TILED_IN = (MODE == COL_INV_TILED);
 #pragma unroll
     for (int m = 0; m < E; ++m)
-      v[m] = valid ? a.in[TILED_IN ? att(t + m * TPC) : at(t + m * TPC)] : make_float2(0.f, 0.f);
+      v[m] = a.in[TILED_IN ? att(t + m * TPC) : at(t + m * TPC)];
     fft_staged<L, E, INV>(v, sb, t, a.twk);
     const float sc = INV ? 1.0f / (float)L : 1.0f;
-    if (valid) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) {
-        if constexpr (MODE == COL_FWD_TILED) a.out[att(t + m * TPC)] = cscale(v[m], sc);
-        else a.out[at(t + m * TPC)] = cscale(v[m], sc);
-      }
+    for (int m = 0; m < E; ++m) {
+      if constexpr (MODE == COL_FWD_TILED) a.out[att(t + m * TPC)] = cscale(v[m], sc);
+      else a.out[at(t + m * TPC)] = cscale(v[m], sc);
     }
   }
 }
@@ -305,7 +289,8 @@ static int launch_col_kernel_w(const ColArgs& a, cudaStream_t s) {
   const cudaError_t cfg_err = once.run(
       [](int*) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::bytes); });
   if (cfg_err != cudaSuccess) return (int)cfg_err;
-  const dim3 grid((a.nx / 2 + Cfg::W - 1) / Cfg::W), block(Cfg::THREADS);
+  if (a.nx / 2 % Cfg::W != 0) return (int)cudaErrorInvalidValue;
+  const dim3 grid(a.nx / 2 / Cfg::W), block(Cfg::THREADS);
   const bool whole = (MODE == COL_RESID_A || MODE == COL_RESID_C) && whole_split(a.ny, a.nx, a.sms);
   return launch_pdl_split(whole, kernel, grid, block, Cfg::bytes, s, a);
 }

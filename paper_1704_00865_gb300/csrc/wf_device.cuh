@@ -436,12 +436,9 @@ __device__ __forceinline__ void bulk_store_wait() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// Ampere-style asynchronous copies (16 or 8 bytes per thread) for strided tiles.
+// Ampere-style asynchronous copies (16 bytes per thread) for strided tiles.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 // L2 prefetch hint for a contiguous range of bytes (16-byte aligned, a
 // multiple of 16, issued in pieces of at most 64 KB).  It changes no data and

@@ -94,14 +94,10 @@ struct RowArgs {
   int check_done;             // return at once when the solver is done
   int skip_ok;                // residual kernels: return at once when st->skip_resid
   const float4* dn;           // [ny][nx/2] pixel pairs (d0, nb0, d1, nb1); nb < 0 = masked
-  float2* f_d1;               // RF fields [ny][nx/2]
-  float2* f_t1;
-  const float2* f_x;          // signal-side neighbour in RF (d_2DF or s)
-  float2* f_y;                // t_PX in RF (no stripe part)
+  float2* f_d1;               // d_RF [ny][nx/2]
   const float* pst;           // [nx/2+1] stripe eigenvalues
   const float* a2;            // [ny] a(y)^2 or nullptr
   const float2* twx;          // exp(-2 pi i k/nx), k < nx
-  const float2* twh;          // exp(-2 pi i k/(nx/2)), k < nx/2
   const float2* tws;          // row pass: stage table of its shape (StageTable)
   const float2* twk;          // the other row kernels' stage table
   WfState* st;
@@ -117,8 +113,8 @@ struct RowArgs {
   float2* gm_out;             // S^-1 s on masked pixels (pairs), 0 elsewhere, or nullptr
   int variant;                // row pass shape (0 or 1), chosen by the autotuner
   int sms;                    // SMs of the device the pass's CTAs are spread over, or 0
-  CUtensorMap tm_t;           // row pass: t_RF (or t_PX) and the signal-side field as tiles
-  CUtensorMap tm_x;           // (tile_map, rows of the pass's shape)
+  CUtensorMap tm_t;           // row pass: t_RF (t_PX without stripes) as tiles (tile_map, rows of
+  CUtensorMap tm_x;           // the pass's shape), and the signal-side field (d_2DF or s)
 };
 
 struct ColArgs {

@@ -58,9 +58,9 @@ row_kernel(RowArgs a) {
   float2* sb = sbuf[g];
   pdl_trigger();
   // the pixel table, fixed during a solve, while the previous kernel drains
-  constexpr bool PX = (MODE == ROW_RESID_B || MODE == ROW_RESID_D), PRE = PX && E <= 12;
-  float4 px[PRE ? E : 1];
-  if constexpr (PRE) {
+  constexpr bool PX = (MODE == ROW_RESID_B || MODE == ROW_RESID_D);
+  float4 px[PX ? E : 1];
+  if constexpr (PX) {
 #pragma unroll
     for (int m = 0; m < E; ++m) px[m] = valid ? __ldg(&a.dn[row0 + t + m * TPF]) : make_float4(0.f, -1.f, 0.f, -1.f);
   }
@@ -87,7 +87,7 @@ row_kernel(RowArgs a) {
     double gm2 = 0.0, g2 = 0.0;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const float4 q = PRE ? px[PRE ? m : 0] : (valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f));
+      const float4 q = px[m];
       const float2 jm = (valid && a.src_px != nullptr) ? a.src_px[row0 + t + m * TPF] : make_float2(0.f, 0.f);
       float gp[2], qp[2], go[2];
       const float gv[2] = {v[m].x, v[m].y}, sv[2] = {w[m].x, w[m].y};
@@ -148,7 +148,7 @@ row_kernel(RowArgs a) {
     double r2 = 0.0;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const float4 q = PRE ? px[PRE ? m : 0] : (valid ? a.dn[row0 + t + m * TPF] : make_float4(0.f, -1.f, 0.f, -1.f));
+      const float4 q = px[m];
       if (valid) {
         const double r0 = q.y >= 0.f ? (double)v[m].x : 0.0, r1 = q.w >= 0.f ? (double)v[m].y : 0.0;
         r2 += r0 * r0;
