@@ -152,7 +152,8 @@ col_pass_kernel(ColArgs a) {
     for (int m = 0; m < E; ++m) eq[STAGED ? m : 0] = __ldg(&a.eig_nyq[t + m * TPC]);
   }
   // the row pass's CTAs may start beside this one: their prologue (the pixel
-  // table) then costs nothing (256^2 sweep 6.5 -> 5.5 us, 2048^2 40.8 -> 39.7)
+  // table) then costs nothing (when this came in: 256^2 sweep 6.5 -> 5.5 us,
+  // 2048^2 40.8 -> 39.7)
   pdl_trigger();
   // Maps above L2: the CTA that will run on this SM one wave later (pf CTAs
   // on) finds its tiles in L2 -- (C, P1f) now, the messenger once the

@@ -75,7 +75,7 @@ __global__ void to_half_kernel(const float* __restrict__ src, __half* __restrict
 //   synth        S -> pixels along rows, + W h + bias, GELU (or the adjoint,
 //                times GELU')
 //
-// A layer is four launches forward and six backward; each activation map is
+// A layer is four launches forward and seven backward; each activation map is
 // read twice and written once.  Before, the transforms were one output per
 // thread with both operands from L2, and the channel products kept their
 // operands in local memory: inference of one 512^2 map (32 channels, 16 x 32
@@ -121,8 +121,9 @@ __global__ void lift_fwd(const float* __restrict__ x, const __half* __restrict__
 // The folded rows are staged transposed, row groups XOR-swizzled by x so that
 // the stores are conflict-free.  KS groups of warps share the pixels of a row
 // (each with its own stage and its own barrier) so that few rows still fill
-// the SMs; their sums (of at most 128 terms) are added in a fixed order.  FP32
-// bound: N/2 * 32 FMA per row for 16 modes.
+// the SMs; their sums (of N / (2 KS) terms: 128 at 1024^2 with four groups, up
+// to 512 with one) are added in a fixed order.  FP32 bound: N/2 * 32 FMA per row
+// for 16 modes.
 template <int KS, int KW>
 __global__ void __launch_bounds__(KS * KW * 64, KW == 1 ? (KS == 4 ? 3 : 10) : 1)
 analysis(const float* __restrict__ in, float2* __restrict__ part, const float2* __restrict__ tw_k,

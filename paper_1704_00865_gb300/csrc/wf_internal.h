@@ -158,10 +158,11 @@ constexpr size_t kMaxDynSmem = 227 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024
 // spreads evenly over its SMs: with programmatic launch the CTAs go to the SMs
 // that drain first, several to some and none to others, so no more than
 // ceil(grid / sms) of them should fit on one.  At 1024^2 (128 column CTAs, 1024
-// row CTAs) a sweep takes 11.5 us instead of 13.2, at 512^2 6.6 instead of 7.1.
-// Not where that number is 2, or 1 with most SMs free: small grids leave room
-// anyway, and the larger footprint would keep the next kernel's CTAs from
-// starting beside them (256^2: 6.3 us instead of 5.4).
+// row CTAs) a sweep takes 10.0 us instead of 10.5, at 512 x 1536 11.9 instead of
+// 15.7.  Not where that number is 2, or 1 with most SMs free: small grids leave
+// room anyway, and the larger footprint would keep the next kernel's CTAs from
+// starting beside them (256^2, with the passes that the rule came in with: 6.3
+// us instead of 5.4).
 inline size_t spread_smem(int grid, size_t bytes, int sms) {
   if (sms <= 0) return bytes;
   const size_t k = ((size_t)grid + sms - 1) / sms;
