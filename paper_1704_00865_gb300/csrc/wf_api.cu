@@ -241,8 +241,9 @@ static std::vector<float2> stage_table(const std::vector<float2>& tab, int E) {
   for (int ns = 1, r = 0; ns < L; ns *= r) {
     r = (ns == 1 && L % 3 == 0) ? E : std::min(p2, L / ns);
     if (ns == 1) continue;
-    for (int q = 0; q == 0 || 4 * q < r; ++q)
-      for (int jm = 0; jm < ns; ++jm) out.push_back(tab[(size_t)jm * (L / (ns * r)) * (q ? 4 * q : 1)]);
+    auto power = [&](int q) { return E == 4 ? q + 1 : std::max(1, 4 * q); };
+    for (int q = 0; power(q) < r; ++q)
+      for (int jm = 0; jm < ns; ++jm) out.push_back(tab[(size_t)jm * (L / (ns * r)) * power(q)]);
   }
   return out;
 }

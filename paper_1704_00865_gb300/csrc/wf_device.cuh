@@ -193,16 +193,16 @@ struct StageRadix {
 };
 
 // Twiddles of one transform in the order its stages read them: for every stage
-// after the first (sub-transform length NS, radix R) and q = 0, 1, ...
-// (the powers 1, 4, 8, 12 below R), NS values W_{NS R}^{jm q'} over jm.  The lanes
+// after the first (sub-transform length NS, radix R) and every power q below R of
+// 1, 4, 8, 12 (of 1, 2, 3 for 4 values per thread), NS values W_{NS R}^{jm q} over jm.  The lanes
 // of a warp read consecutive ones, where the table exp(-2 pi i k / L) has them
 // 8 lines apart.  Built by stage_table (wf_api.cu).
-template <int R>
-struct StageQ { static constexpr int n = R <= 4 ? 1 : (R == 8 ? 2 : (R == 12 ? 3 : 4)); };
+template <int R, int E>
+struct StageQ { static constexpr int n = E == 4 ? R - 1 : (R + 3) / 4; };
 template <int L, int E, int NS = 1>
 struct StageTable {
   static constexpr int R = StageRadix<L, E, NS>::value;
-  static constexpr int here = NS == 1 ? 0 : NS * StageQ<R>::n;
+  static constexpr int here = NS == 1 ? 0 : NS * StageQ<R, E>::n;
   static constexpr int size = here + StageTable<L, E, NS * R>::size;
 };
 template <int L, int E>
@@ -700,7 +700,7 @@ __device__ __forceinline__ void tc5_teardown() {
 template <int L, int E, int NS, bool INV, bool WARP, bool TWS = false, int PREC = 0, int OFF = -1>
 struct FFTStages {
   static constexpr int R = StageRadix<L, E, NS>::value;
-  static constexpr int NEXT = OFF < 0 ? -1 : OFF + (NS == 1 ? 0 : NS * StageQ<R>::n);
+  static constexpr int NEXT = OFF < 0 ? -1 : OFF + (NS == 1 ? 0 : NS * StageQ<R, E>::n);
   static __device__ __forceinline__ void run(float2 (&v)[E], float2* sb, int t,
                                              const float2* __restrict__ twtab, int twstride) {
     constexpr int TPF = L / E;
@@ -735,18 +735,23 @@ struct FFTStages {
       for (int r = 0; r < R; ++r) u[r] = v[b + r * B];
       if constexpr (NS > 1) {
         // twiddles W_{NS R}^{jm r}: exact table values every 4th power,
-        // products in between (at most 3 multiplications deep)
+        // products in between (at most 3 multiplications deep); with 4 values
+        // per thread, which take more stages, exact values throughout (with
+        // products that shape was 25 to 33 % further from 64 bits than 8 values
+        // per thread after 200 plain or white sweeps, now 4 to 30 % nearer; the
+        // sweep's time is the same within 2 %)
+        constexpr bool EXACT = OFF >= 0 && E == 4;
         const int step = OFF < 0 ? jm * (L / (NS * R)) * twstride : 0;
         auto tw = [&](int r) {
-          return tw_dir<INV>(tw_load<TWS>(twtab, OFF < 0 ? step * r : OFF + (r / 4) * NS + jm));
+          return tw_dir<INV>(tw_load<TWS>(twtab, OFF < 0 ? step * r : OFF + (EXACT ? r - 1 : r / 4) * NS + jm));
         };
         float2 w1 = tw(1);
         float2 wr = w1;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          if ((r & 3) == 0) wr = tw(r);
+          if ((r & 3) == 0 || (EXACT && r > 1)) wr = tw(r);
           u[r] = cmul(u[r], wr);
-          wr = cmul(wr, w1);
+          if constexpr (!EXACT) wr = cmul(wr, w1);
         }
       }
       dftR<R, INV>(u);
