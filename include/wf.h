@@ -503,7 +503,9 @@ typedef struct {
  *           items, a grid barrier between the row and column phases and
  *           per-map done flags (each map keeps its own lambda, residual and
  *           stop test); every polling chunk of checkpoints, with each map's
- *           residual and controller kernels, is one CUDA graph.  Maps must
+ *           residual and controller kernels, is one CUDA graph.  For callers
+ *           that can spare one host thread only: at every size slower than
+ *           lanes, and than lanes = 1 (0.6 to 0.8 of its rate).  Maps must
  *           be square with sides 256, 384, 512, 768, 1024, 1536 or 2048,
  *           with a stripe part and the merged 2DF block (or no 1/f part),
  *           dft_precision 0 (WF_EUNSUPPORTED otherwise).  Each size has one

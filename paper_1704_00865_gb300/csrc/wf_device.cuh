@@ -738,7 +738,7 @@ struct FFTStages {
         // products in between (at most 3 multiplications deep); with 4 values
         // per thread, which take more stages, exact values throughout (with
         // products that shape was 25 to 33 % further from 64 bits than 8 values
-        // per thread after 200 plain or white sweeps, now 4 to 30 % nearer; the
+        // per thread after 200 plain or white sweeps, now 7 to 34 % nearer; the
         // sweep's time is the same within 2 %)
         constexpr bool EXACT = OFF >= 0 && E == 4;
         const int step = OFF < 0 ? jm * (L / (NS * R)) * twstride : 0;
