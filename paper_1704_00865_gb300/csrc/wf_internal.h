@@ -179,7 +179,7 @@ inline size_t spread_cols_smem(int grid, size_t bytes, int sms, int row_ctas) {
 }
 // An SM divides its 256 KB between L1 and shared memory and changes that only
 // when it is empty, so a kernel does not start beside one of another split.
-// Left to the driver, the residual's kernels (a few KB a CTA) get another one
+// Left to CUDA, the residual's kernels (a few KB a CTA) get another one
 // than the passes that ask for tens of KB to spread, and a checkpoint waits for
 // the changes.  With a hundred row CTAs and more, on maps small enough that
 // this counts, they ask for all of it as shared memory: a checkpoint of 512 x
